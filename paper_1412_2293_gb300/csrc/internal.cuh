@@ -206,6 +206,10 @@ cudaError_t launch_basis_prob(qs_ctx* h, const void* psi, int n, int members, ui
 cudaError_t launch_dm_trace(qs_ctx* h, const void* rho, int n, double* out_dev);
 cudaError_t launch_dm_expect(qs_ctx* h, const void* rho, const void* ref, int n, double* out_dev);
 cudaError_t launch_convert_ref(qs_ctx* h, const double* src_dev, void* dst, size_t count);
+// out[g] from `members` rows of `chunks` complex partials: |sum|^2 (mode 0) or
+// the real sum (mode 1) of each member, added over runs of `group` members
+cudaError_t launch_finalize(const double* partials, int members, int chunks, int mode, int group, double* out,
+                            cudaStream_t s);
 
 // fixed rank, every member of the handle (counts in h->rc): expansion of the
 // factors into L' with K Kraus operators (member b's at E + b e_stride,

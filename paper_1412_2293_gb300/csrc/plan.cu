@@ -1317,29 +1317,6 @@ cudaError_t launch_pass_kernel(qs_plan p, const PassPlan& P, cudaStream_t s, int
   return cudaGetLastError();
 }
 
-// fused fidelity: out[b] = |sum over the last pass's tiles of member b|^2.
-// One warp per member: lane l adds slots l, l + 32, ... in order, then the
-// lanes' sums meet in a fixed shuffle tree (FP64 throughout, the same order
-// on every run).
-__global__ void __launch_bounds__(256) k_fid_finalize(const double* __restrict__ partials, int members, int tiles,
-                                                      double* __restrict__ out) {
-  const int b = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (b >= members) return;                            // uniform per warp
-  const double* pm = partials + 2 * (uint64_t)b * tiles;
-  double re = 0.0, im = 0.0;
-  for (int t = lane; t < tiles; t += 32) {
-    re += pm[2 * t];
-    im += pm[2 * t + 1];
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    re += __shfl_xor_sync(0xffffffffu, re, o);
-    im += __shfl_xor_sync(0xffffffffu, im, o);
-  }
-  if (lane == 0) out[b] = re * re + im * im;
-}
-
 cudaError_t set_smem_attrs(size_t esize) {
   static std::atomic<bool> done[2] = {false, false};
   const int which = esize == 8 ? 0 : 1;
@@ -1588,8 +1565,7 @@ qs_status enqueue_run(qs_plan p, cudaStream_t s, int synth, int fid) {
       if (e == cudaSuccess) e = f32 ? launch_pass_kernel<float>(p, P, s, sy, fd) : launch_pass_kernel<double>(p, P, s, sy, fd);
       mark(P.high ? 2 : 1);
       if (e == cudaSuccess && fd) {
-        k_fid_finalize<<<(h->batch + 7) / 8, 256, 0, s>>>(p->d_fid, h->batch, fid_slots(p, P), h->small + kSmallOutIndex);
-        e = cudaGetLastError();
+        e = launch_finalize(p->d_fid, h->batch, fid_slots(p, P), 0, 1, h->small + kSmallOutIndex, s);
       }
       if (e != cudaSuccess) { h->stream = saved; return pfail(p, QS_ERR_CUDA, std::string("fused pass: ") + cudaGetErrorString(e)); }
     } else {

@@ -45,24 +45,56 @@ __device__ __forceinline__ double2 block_sum2(double a, double b) {
   return r;
 }
 
-// partial[member][chunk] = sum over the chunk of conj(ref_i) psi_i
+// A thread's kPer amplitudes of a full chunk are read as 16-byte vectors
+// (two complex64 amplitudes or one complex128) before any of them is used:
+// the sweep is bound by HBM latency otherwise (one 8-byte load in flight per
+// thread and iteration read 1 GiB of members at 3.3 TB/s; see k_dot_partials).
+constexpr int kPer = kChunk / kRBlock;   // 16 amplitudes per thread
+template <typename R> struct Vec;
+template <> struct Vec<float> { using T = float4; static constexpr int N = 2; };
+template <> struct Vec<double> { using T = double2; static constexpr int N = 1; };
+__device__ __forceinline__ float2 vget(const float4& v, int k) { return k ? make_float2(v.z, v.w) : make_float2(v.x, v.y); }
+__device__ __forceinline__ double2 vget(const double2& v, int) { return v; }
+
+// f(amplitude, reference) over the chunk starting at beg (p, r: the member's
+// and the reference's first amplitude; r may be null for REF = false)
+template <typename R, bool REF, typename F>
+__device__ __forceinline__ void chunk_each(const cplx<R>* __restrict__ p, const cplx<R>* __restrict__ r, uint64_t beg,
+                                           uint64_t N, F&& f) {
+  using V = typename Vec<R>::T;
+  constexpr int W = Vec<R>::N, L = kPer / W;
+  if (beg + kChunk <= N) {
+    const V* pv = reinterpret_cast<const V*>(p + beg) + threadIdx.x;
+    const V* rv = reinterpret_cast<const V*>(r + beg) + threadIdx.x;
+    V a[L];
+#pragma unroll
+    for (int i = 0; i < L; ++i) a[i] = __ldcs(pv + i * kRBlock);
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      V q = a[i];
+      if constexpr (REF) q = __ldg(rv + i * kRBlock);
+#pragma unroll
+      for (int k = 0; k < W; ++k) f(vget(a[i], k), vget(q, k));
+    }
+  } else {                                             // a member smaller than a chunk
+    for (uint64_t x = beg + threadIdx.x; x < N; x += blockDim.x) f(p[x], REF ? r[x] : p[x]);
+  }
+}
+
+// partial[member][chunk] = sum over the chunk of conj(ref_i) psi_i.  Bound by
+// HBM (the members; the reference stays in L2): 64 members of 2^21 complex64
+// amplitudes 328 -> 175 us (6.1 TB/s) with the loads above.
 template <typename R>
 __global__ void __launch_bounds__(kRBlock) k_dot_partials(const cplx<R>* __restrict__ psi,
                                                           const cplx<R>* __restrict__ ref, int n,
-                                                          int chunks, int chunk, double* partials) {
+                                                          int chunks, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  const uint64_t beg = (uint64_t)c * chunk;
-  const cplx<R>* p = psi + (uint64_t)b * N;
   R re = 0, im = 0;
-  for (int i = threadIdx.x; i < chunk; i += blockDim.x) {
-    const uint64_t x = beg + i;
-    if (x < N) {
-      const cplx<R> a = p[x], r = ref[x];
-      re += r.x * a.x + r.y * a.y;
-      im += r.x * a.y - r.y * a.x;
-    }
-  }
+  chunk_each<R, true>(psi + (uint64_t)b * N, ref, (uint64_t)c * kChunk, N, [&](cplx<R> a, cplx<R> r) {
+    re += r.x * a.x + r.y * a.y;
+    im += r.x * a.y - r.y * a.x;
+  });
   const double2 s = block_sum2((double)re, (double)im);
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = s.x;
@@ -73,16 +105,12 @@ __global__ void __launch_bounds__(kRBlock) k_dot_partials(const cplx<R>* __restr
 // partial[member][chunk] = sum |psi_i|^2 (stored in the .x slot)
 template <typename R>
 __global__ void __launch_bounds__(kRBlock) k_norm_partials(const cplx<R>* __restrict__ psi, int n,
-                                                           int chunks, int chunk, double* partials) {
+                                                           int chunks, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  const uint64_t beg = (uint64_t)c * chunk;
-  const cplx<R>* p = psi + (uint64_t)b * N;
   R s = 0;
-  for (int i = threadIdx.x; i < chunk; i += blockDim.x) {
-    const uint64_t x = beg + i;
-    if (x < N) { const cplx<R> a = p[x]; s += a.x * a.x + a.y * a.y; }
-  }
+  chunk_each<R, false>(psi + (uint64_t)b * N, psi, (uint64_t)c * kChunk, N,
+                       [&](cplx<R> a, cplx<R>) { s += a.x * a.x + a.y * a.y; });
   const double2 t = block_sum2((double)s, 0.0);
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = t.x;
@@ -92,32 +120,69 @@ __global__ void __launch_bounds__(kRBlock) k_norm_partials(const cplx<R>* __rest
 
 // v_b = |sum_c partial|^2 (mode 0) or sum_c partial.x (mode 1); out[g] =
 // v_{g group} + ... + v_{g group + group - 1} in order (group = 1: out[b] =
-// v_b).  One warp per output: lane l adds chunks l, l + 32, ... in order, the
-// lanes meet in a fixed shuffle tree (the same order on every call).
-__global__ void __launch_bounds__(256) k_finalize(const double* partials, int members, int chunks, int mode, int group,
-                                                  double* out) {
+// v_b).  WIDE = 0: one warp per output, lane l adds chunks l, l + 32, ... in
+// order and the lanes meet in a fixed shuffle tree.  WIDE = 1: one block per
+// output, its 8 warps shared out over the members of the group (8 / group
+// warps each, at least one) and a member's warps taking its chunks in turn;
+// their sums are added in warp order.  Either order is fixed by the shape.
+// The kernel is a chain of dependent loads, so the wide form is taken when an
+// output has more than 64 partials: one output of 16384 (a 14-qubit density
+// matrix) 247 -> 9 us, 27 of 8192 (fused passes at 23 qubits) 55 -> 6 us; with
+// fewer the narrow form starts fewer blocks and is as fast.
+template <int WIDE>
+__global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ partials, int members, int chunks, int mode,
+                                                  int group, double* __restrict__ out) {
+  const double2* part = reinterpret_cast<const double2*>(partials);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int outs = members / group;
-  const int lane = threadIdx.x & 31;
-  const int warps = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); g < outs; g += warps) {
-    double s = 0.0;
-    for (int b = g * group; b < (g + 1) * group; ++b) {
-      const double* pb = partials + 2 * (uint64_t)b * chunks;
-      double re = 0.0, im = 0.0;
-      for (int c = lane; c < chunks; c += 32) {
-        re += pb[2 * c];
-        im += pb[2 * c + 1];
+  auto strided = [&](const double2* pb, int first, int step) {
+    double2 a[4] = {};
+    int c = first;
+    for (; c + 3 * step < chunks; c += 4 * step) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const double2 v = pb[c + k * step];
+        a[k].x += v.x;
+        a[k].y += v.y;
       }
-      re = warp_sum(re);
-      im = warp_sum(im);
-      s += mode == 0 ? re * re + im * im : re;
     }
-    if (lane == 0) out[g] = s;
+    for (; c < chunks; c += step) { const double2 v = pb[c]; a[0].x += v.x; a[0].y += v.y; }
+    return make_double2(warp_sum((a[0].x + a[1].x) + (a[2].x + a[3].x)), warp_sum((a[0].y + a[1].y) + (a[2].y + a[3].y)));
+  };
+  if constexpr (WIDE == 0) {
+    const int warps = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); g < outs; g += warps) {
+      double s = 0.0;
+      for (int b = g * group; b < (g + 1) * group; ++b) {
+        const double2 v = strided(part + (uint64_t)b * chunks, lane, 32);
+        s += mode == 0 ? v.x * v.x + v.y * v.y : v.x;
+      }
+      if (lane == 0) out[g] = s;
+    }
+  } else {
+    __shared__ double2 ws[8];
+    const int per = group >= 8 ? 1 : 8 / group;          // warps per member
+    const int at_once = 8 / per;                         // members summed side by side
+    for (int g = blockIdx.x; g < outs; g += gridDim.x) {
+      double s = 0.0;
+      for (int b0 = 0; b0 < group; b0 += at_once) {
+        const int b = b0 + warp / per;
+        double2 v = make_double2(0.0, 0.0);
+        if (b < group && warp < per * at_once)
+          v = strided(part + ((uint64_t)g * group + b) * chunks, (warp % per) * 32 + lane, 32 * per);
+        if (lane == 0) ws[warp] = v;
+        __syncthreads();
+        for (int k = 0; k < at_once && b0 + k < group; ++k) {
+          double re = 0.0, im = 0.0;
+          for (int q = 0; q < per; ++q) { re += ws[k * per + q].x; im += ws[k * per + q].y; }
+          s += mode == 0 ? re * re + im * im : re;
+        }
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) out[g] = s;
+    }
   }
 }
-
-// warps of the finalize launch for `outs` outputs (eight per block)
-inline unsigned finalize_blocks(int outs) { return (unsigned)std::max(1, std::min((outs + 7) / 8, 4096)); }
 
 template <typename R>
 __global__ void k_basis_prob(const cplx<R>* psi, int n, int members, uint64_t x, int group, double* out) {
@@ -147,25 +212,69 @@ __global__ void __launch_bounds__(kRBlock) k_dm_trace_partials(const cplx<R>* rh
   if (threadIdx.x == 0) { partials[2 * blockIdx.x] = t.x; partials[2 * blockIdx.x + 1] = 0.0; }
 }
 
-// <phi|rho|phi> = sum_i conj(phi_i) sum_j rho[i][j] phi_j, one block per row
-template <typename R>
+// Sums of products to more than FP64's input precision on the FP32 pipe: a
+// product of two floats as (rounded, exact remainder), the running sum as
+// (sum, what its roundings lost) -- the compensated dot product of Ogita, Rump
+// and Oishi (SIAM J. Sci. Comput. 26, 2005), as accurate as a 48-bit sum.  A
+// multiply-add takes 10 FP32 instructions; the FP64 one and its two
+// conversions hold a scheduler's FP64 unit for about 64 cycles each on GB300.
+struct Sum2 {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
+    s = t;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+struct Sum1 {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <typename R> struct SumOf;
+template <> struct SumOf<float> { using T = Sum2; };
+template <> struct SumOf<double> { using T = Sum1; };
+
+// <phi|rho|phi> = sum_i conj(phi_i) sum_j rho[i][j] phi_j, one block per row.
+// HERM (an exactly Hermitian rho): the entries right of the diagonal only,
+// their real part counted twice, 2 Re sum_{i<j}, plus the real diagonal; the
+// part of a row that is summed starts at i, so blocks take rows from both
+// ends in turn.  Bound by the FP64 pipe in complex128, four multiply-adds an
+// entry (14 qubits 2.99 -> 0.95 ms for half the entries), and by HBM in
+// complex64 with Sum2 (13 qubits 1.28 -> 0.06 ms).
+template <typename R, bool HERM>
 __global__ void __launch_bounds__(kRBlock) k_dm_expect_rows(const cplx<R>* __restrict__ rho,
                                                             const cplx<R>* __restrict__ phi, int n,
                                                             double* partials) {
   const uint64_t N = 1ull << n;
-  const uint64_t i = blockIdx.x;
+  const uint64_t bi = blockIdx.x;
+  const uint64_t i = HERM ? ((bi & 1) ? N - 1 - (bi >> 1) : bi >> 1) : bi;
   const cplx<R>* row = rho + i * N;
-  double re = 0.0, im = 0.0;
-  for (uint64_t j = threadIdx.x; j < N; j += blockDim.x) {
+  typename SumOf<R>::T re, im;
+  // whole aligned steps of the block from the one that holds column i + 1
+  const uint64_t j0 = HERM ? ((i + 1) & ~(uint64_t)(kRBlock - 1)) : 0;
+#pragma unroll 4
+  for (uint64_t j = j0 + threadIdx.x; j < N; j += kRBlock) {
+    if (HERM && j <= i) continue;
     const cplx<R> a = row[j], f = phi[j];
-    re += (double)a.x * f.x - (double)a.y * f.y;
-    im += (double)a.x * f.y + (double)a.y * f.x;
+    re.add(a.x, f.x);
+    re.add(-a.y, f.y);
+    im.add(a.x, f.y);
+    im.add(a.y, f.x);
   }
-  const double2 v = block_sum2(re, im);
+  const double2 v = block_sum2(re.value(), im.value());
   if (threadIdx.x == 0) {
     const cplx<R> f = phi[i];
-    partials[2 * i] = (double)f.x * v.x + (double)f.y * v.y;         // Re(conj(f) v)
-    partials[2 * i + 1] = (double)f.x * v.y - (double)f.y * v.x;
+    double r = (double)f.x * v.x + (double)f.y * v.y;                  // Re(conj(f) v)
+    double m = (double)f.x * v.y - (double)f.y * v.x;
+    if (HERM) {
+      r = 2.0 * r + (double)row[i].x * ((double)f.x * f.x + (double)f.y * f.y);
+      m = 0.0;
+    }
+    partials[2 * i] = r;
+    partials[2 * i + 1] = m;
   }
 }
 
@@ -192,17 +301,27 @@ int chunk_count(int n) {
 
 }  // namespace
 
+cudaError_t launch_finalize(const double* partials, int members, int chunks, int mode, int group, double* out,
+                            cudaStream_t s) {
+  const int outs = members / group;
+  if ((uint64_t)chunks * group > 64)                    // see k_finalize
+    k_finalize<1><<<(unsigned)std::min(outs, 65535), 256, 0, s>>>(partials, members, chunks, mode, group, out);
+  else
+    k_finalize<0><<<(unsigned)std::max(1, std::min((outs + 7) / 8, 4096)), 256, 0, s>>>(partials, members, chunks, mode,
+                                                                                      group, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_dot(qs_ctx* h, const void* psi, const void* ref, int n, int members,
                        int group, double* out) {
   const int chunks = chunk_count(n);
   if (!ensure_partials(h, (size_t)2 * chunks * members)) return cudaErrorMemoryAllocation;
   dim3 grid(chunks, members);
   if (h->dtype == QS_C64)
-    k_dot_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, (const float2*)ref, n, chunks, kChunk, h->partials);
+    k_dot_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, (const float2*)ref, n, chunks, h->partials);
   else
-    k_dot_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, (const double2*)ref, n, chunks, kChunk, h->partials);
-  k_finalize<<<finalize_blocks(members / group), 256, 0, h->stream>>>(h->partials, members, chunks, 0, group, out);
-  return cudaGetLastError();
+    k_dot_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, (const double2*)ref, n, chunks, h->partials);
+  return launch_finalize(h->partials, members, chunks, 0, group, out, h->stream);
 }
 
 cudaError_t launch_norm(qs_ctx* h, const void* psi, int n, int members, int group, double* out) {
@@ -210,11 +329,10 @@ cudaError_t launch_norm(qs_ctx* h, const void* psi, int n, int members, int grou
   if (!ensure_partials(h, (size_t)2 * chunks * members)) return cudaErrorMemoryAllocation;
   dim3 grid(chunks, members);
   if (h->dtype == QS_C64)
-    k_norm_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, n, chunks, kChunk, h->partials);
+    k_norm_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, n, chunks, h->partials);
   else
-    k_norm_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, n, chunks, kChunk, h->partials);
-  k_finalize<<<finalize_blocks(members / group), 256, 0, h->stream>>>(h->partials, members, chunks, 1, group, out);
-  return cudaGetLastError();
+    k_norm_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, n, chunks, h->partials);
+  return launch_finalize(h->partials, members, chunks, 1, group, out, h->stream);
 }
 
 cudaError_t launch_basis_prob(qs_ctx* h, const void* psi, int n, int members, uint64_t x,
@@ -234,20 +352,24 @@ cudaError_t launch_dm_trace(qs_ctx* h, const void* rho, int n, double* out) {
     k_dm_trace_partials<float><<<chunks, kRBlock, 0, h->stream>>>((const float2*)rho, n, chunks, kChunk, h->partials);
   else
     k_dm_trace_partials<double><<<chunks, kRBlock, 0, h->stream>>>((const double2*)rho, n, chunks, kChunk, h->partials);
-  k_finalize<<<1, 32, 0, h->stream>>>(h->partials, 1, chunks, 1, 1, out);
-  return cudaGetLastError();
+  return launch_finalize(h->partials, 1, chunks, 1, 1, out, h->stream);
 }
 
 cudaError_t launch_dm_expect(qs_ctx* h, const void* rho, const void* phi, int n, double* out) {
   const uint64_t N = 1ull << n;
   if (!ensure_partials(h, (size_t)2 * N)) return cudaErrorMemoryAllocation;
-  if (h->dtype == QS_C64)
-    k_dm_expect_rows<float><<<(unsigned)N, kRBlock, 0, h->stream>>>((const float2*)rho, (const float2*)phi, n, h->partials);
-  else
-    k_dm_expect_rows<double><<<(unsigned)N, kRBlock, 0, h->stream>>>((const double2*)rho, (const double2*)phi, n, h->partials);
+  const unsigned g = (unsigned)N;
+  if (h->dtype == QS_C64) {
+    auto *r = (const float2*)rho, *f = (const float2*)phi;
+    if (h->hermitian) k_dm_expect_rows<float, true><<<g, kRBlock, 0, h->stream>>>(r, f, n, h->partials);
+    else k_dm_expect_rows<float, false><<<g, kRBlock, 0, h->stream>>>(r, f, n, h->partials);
+  } else {
+    auto *r = (const double2*)rho, *f = (const double2*)phi;
+    if (h->hermitian) k_dm_expect_rows<double, true><<<g, kRBlock, 0, h->stream>>>(r, f, n, h->partials);
+    else k_dm_expect_rows<double, false><<<g, kRBlock, 0, h->stream>>>(r, f, n, h->partials);
+  }
   // sum of N row partials: treat them as one member with N chunks, real part
-  k_finalize<<<1, 32, 0, h->stream>>>(h->partials, 1, (int)N, 1, 1, out);
-  return cudaGetLastError();
+  return launch_finalize(h->partials, 1, (int)N, 1, 1, out, h->stream);
 }
 
 cudaError_t launch_convert_ref(qs_ctx* h, const double* src, void* dst, size_t count) {
