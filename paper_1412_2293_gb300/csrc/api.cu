@@ -232,23 +232,18 @@ qs_status rank_upload_counts(qs_handle h) {
   return QS_OK;
 }
 
-// Gram matrices, eigensolver, truncation and projection of every member's L'
-// (M_b columns on the device); keep_b = min(r_b, M_b) (r_b = trunc_r when > 0)
-// mirrored on the host.  K: Kraus operators of the channel (L' = K m_b columns).
-qs_status rank_truncate_work(qs_handle h, int K, int trunc_r, int normalize) {
-  int max_M = 0, max_keep = 0;
+// Host mirror of a truncation after a channel of K operators: keep_b = min(r_b,
+// K m_b) (r_b = trunc_r when > 0); the largest M and keep over the members.
+void advance_counts(qs_handle h, int K, int trunc_r, int* max_M, int* max_keep) {
+  *max_M = *max_keep = 0;
   for (int b = 0; b < h->batch; ++b) {
     const int M = K * h->m_cols[b];
     const int keep = std::min(trunc_r > 0 ? trunc_r : h->m_rank[b], M);
-    max_M = std::max(max_M, M);
-    max_keep = std::max(max_keep, keep);
+    *max_M = std::max(*max_M, M);
+    *max_keep = std::max(*max_keep, keep);
     h->m_cols[b] = keep;
   }
-  QS_CUDA(h, qs::launch_gram(h, h->real_factor, max_M));
-  QS_CUDA(h, qs::launch_eig_truncate(h, trunc_r, normalize));
-  QS_CUDA(h, qs::launch_project(h, h->real_factor, K, max_keep));
   h->cols = *std::max_element(h->m_cols.begin(), h->m_cols.end());
-  return QS_OK;
 }
 
 // FIXED_RANK: L'_b = [E_1 L_b | ..], then truncation when K > 1.  ks: one
@@ -276,8 +271,13 @@ qs_status rank_apply_kraus(qs_handle h, const int* targets, int k, const std::ve
     QS_CUDA(h, cudaMemcpyAsync(Edev, e.data(), set_bytes, cudaMemcpyHostToDevice, h->stream));
   }
   const Targets tg = qs::make_targets(h->n, targets, k);
-  QS_CUDA(h, qs::launch_kraus_expand(h, tg, h->real_factor, Edev, K, per_member ? qs::kRankStride : 0, max_cols));
-  return rank_truncate_work(h, K, 0, h->normalize);
+  bool diag = true;
+  for (const auto& E : ks) diag &= is_diagonal(E, d);
+  int max_M, max_keep;
+  advance_counts(h, K, 0, &max_M, &max_keep);
+  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, Edev, K, per_member ? qs::kRankStride : 0,
+                                     qs::KrausGate{}, max_cols, max_keep, h->normalize));
+  return QS_OK;
 }
 
 // FIXED_RANK: the averaged channel of a noisy gate on every member, then
@@ -294,8 +294,11 @@ qs_status rank_channel_gate(qs_handle h, const int* targets, const qs::KrausGate
     max_cols = std::max(max_cols, h->m_cols[b]);
   }
   const Targets tg = qs::make_targets(h->n, targets, g.k);
-  QS_CUDA(h, qs::launch_kraus_expand_gate(h, tg, h->real_factor, g, max_cols));
-  return rank_truncate_work(h, K, 0, h->normalize);
+  const bool diag = g.noise == QS_NOISE_PHASE && qs::gate_diagonal(g.U, g.k);
+  int max_M, max_keep;
+  advance_counts(h, K, 0, &max_M, &max_keep);
+  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, nullptr, K, 0, g, max_cols, max_keep, h->normalize));
+  return QS_OK;
 }
 
 // FIXED_RANK: column c = 0 of every member <- |x> (or Eq. 16's state), the rest 0
@@ -403,6 +406,9 @@ qs_status qs_create(int n, int batch, int rank, qs_mode mode, qs_dtype dtype, vo
     int* counts = nullptr;
     if (cudaMalloc((void**)&counts, 4 * (size_t)batch * sizeof(int)) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
     h->rc = qs::RankCounts{counts, counts + batch, counts + 2 * batch, counts + 3 * batch};
+    const size_t counter_bytes = (size_t)batch * qs::rank_counters() * sizeof(uint32_t);
+    if (cudaMalloc((void**)&h->rcounters, counter_bytes) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
+    if (cudaMemsetAsync(h->rcounters, 0, counter_bytes, h->stream) != cudaSuccess) return bail(QS_ERR_CUDA);
     h->m_cols.assign(batch, 1);
     h->m_rank.assign(batch, rank);
     if (qs::rank_kernel_attributes() != cudaSuccess) return bail(QS_ERR_CUDA);
@@ -411,7 +417,7 @@ qs_status qs_create(int n, int batch, int rank, qs_mode mode, qs_dtype dtype, vo
   const uint64_t chunks = (N + 4095) / 4096;
   size_t partials = 2 * chunks * members;
   if (mode == QS_DENSITY) partials = std::max<size_t>(partials, 2 * N);
-  if (mode == QS_FIXED_RANK) partials = std::max<size_t>(partials, qs::gram_partials_doubles(n, batch));
+  if (mode == QS_FIXED_RANK) partials = std::max<size_t>(partials, qs::gram_partials_doubles(n, batch, rank));
   h->partials_cap = partials;
   if (cudaMalloc((void**)&h->partials, partials * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
   h->mats_cap = std::max<size_t>((size_t)batch * 2 * 16, 2 * 1024) * (h->esize / 2);
@@ -435,7 +441,7 @@ qs_status qs_destroy(qs_handle h) {
   if (!h) return QS_ERR_INVALID_ARG;
   cudaStreamSynchronize(h->stream);
   void* ptrs[] = {h->state, h->work, h->partials, h->mats, h->small, h->dstatus, h->m_e,
-                  h->m_seed, h->m_traj, h->m_marked, h->ref, h->m_basis, h->rsmall, h->rc.cols};
+                  h->m_seed, h->m_traj, h->m_marked, h->ref, h->m_basis, h->rsmall, h->rc.cols, h->rcounters};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (h->hpinned) cudaFreeHost(h->hpinned);
   delete h;
@@ -672,7 +678,12 @@ qs_status qs_truncate_rank(qs_handle h, int r, int normalize) {
   QS_CUDA(h, cudaMemcpy2DAsync(h->work, (size_t)h->mcap * col_bytes, h->state, (size_t)h->rank * col_bytes,
                                (size_t)h->rank * col_bytes, h->batch, cudaMemcpyDeviceToDevice, h->stream));
   QS_CUDA(h, cudaMemcpyAsync(h->rc.M, h->m_cols.data(), h->batch * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-  return rank_truncate_work(h, 1, r, normalize);
+  int max_M, max_keep;
+  advance_counts(h, 1, r, &max_M, &max_keep);
+  QS_CUDA(h, qs::launch_gram(h, h->real_factor, max_M));
+  QS_CUDA(h, qs::launch_eig_truncate(h, r, normalize));
+  QS_CUDA(h, qs::launch_project(h, h->real_factor, 1, max_keep));
+  return QS_OK;
 }
 
 qs_status qs_set_tensor_cores(qs_handle h, int on) {

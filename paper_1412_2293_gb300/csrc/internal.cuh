@@ -110,7 +110,8 @@ struct qs_ctx {
   int cols = 1;
   int normalize = 0;
   qs::RankCounts rc{};
-  double* rsmall = nullptr;              // per member: Gram, eigenvectors, eigenvalues, scale, Kraus sets
+  double* rsmall = nullptr;              // per member: Gram, eigenvectors, eigenvalues, scale, Kraus sets, V
+  uint32_t* rcounters = nullptr;         // arrivals of the moments' row blocks (zero between launches)
   std::vector<int> m_cols, m_rank;
   // FIXED_RANK: every entry of L has a zero imaginary part (real start, real
   // gates and Kraus operators so far); the channel kernels then use real
@@ -205,11 +206,11 @@ cudaError_t launch_basis_prob(qs_ctx* h, const void* psi, int n, int members, ui
                               int group, double* out_dev);
 cudaError_t launch_dm_trace(qs_ctx* h, const void* rho, int n, double* out_dev);
 cudaError_t launch_dm_expect(qs_ctx* h, const void* rho, const void* ref, int n, double* out_dev);
-cudaError_t launch_convert_ref(qs_ctx* h, const double* src_dev, void* dst, size_t count);
 // out[g] from `members` rows of `chunks` complex partials: |sum|^2 (mode 0) or
 // the real sum (mode 1) of each member, added over runs of `group` members
 cudaError_t launch_finalize(const double* partials, int members, int chunks, int mode, int group, double* out,
                             cudaStream_t s);
+cudaError_t launch_convert_ref(qs_ctx* h, const double* src_dev, void* dst, size_t count);
 
 // fixed rank, every member of the handle (counts in h->rc): expansion of the
 // factors into L' with K Kraus operators (member b's at E + b e_stride,
@@ -226,10 +227,17 @@ inline int kraus_count(int k, int noise) { return noise == QS_NOISE_ROTATION && 
 cudaError_t launch_gram(qs_ctx* h, bool real, int max_M);
 cudaError_t launch_eig_truncate(qs_ctx* h, int trunc_r, int normalize);
 cudaError_t launch_project(qs_ctx* h, bool real, int K, int max_keep);
+// A whole channel (Kraus operators E as above, or g's averaged set when g.k >
+// 0) with truncation to the members' ranks.  diag: every operator is diagonal.
+// One-qubit and diagonal channels never form L' (k_moments, k_project_fused).
+cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool diag, const double* E_dev, int K,
+                                int e_stride, const KrausGate& g, int max_cols, int max_keep, int normalize);
+bool gate_diagonal(const double* U, int k);   // U (2^k x 2^k interleaved) has no off-diagonal entry
+int rank_counters();                          // words of h->rcounters per member
 int gram_rows_per_block(int n);
 // one-time kernel attributes of the fixed-rank kernels (outside any capture)
 cudaError_t rank_kernel_attributes();
-size_t gram_partials_doubles(int n, int members);
+size_t gram_partials_doubles(int n, int members, int rank);
 
 // debug noise
 cudaError_t launch_debug_noise(uint64_t seed, uint64_t traj, uint64_t gate_id, int count,
@@ -242,7 +250,8 @@ constexpr size_t kSmallW = 2048;       // eigenvectors, 2 * 32 * 16
 constexpr size_t kSmallLam = 3072;     // eigenvalues, 32
 constexpr size_t kSmallScale = 3104;   // 1
 constexpr size_t kSmallE = 3200;       // Kraus operators, <= 2 * 8 * 16
-constexpr int kRankStride = 3456;
+constexpr size_t kSmallV = 3456;       // the projection's matrices V_ij, <= 2 * 4 * 16 * 16
+constexpr int kRankStride = 3456 + 2048;
 constexpr size_t kSmallOutIndex = 4096;  // results, batch doubles
 
 // Write a pending basis start state into memory (no-op when none is pending).

@@ -1493,10 +1493,8 @@ qs_status run_rank_ops(qs_plan p) {
         kg.e_member = member_e ? h->m_e : nullptr;
         kg.e_run = &p->d_run->e;
         const int K = kraus_count(g.k, g.noise);
-        e = launch_kraus_expand_gate(h, tg, real, kg, h->rank);
-        if (e == cudaSuccess) e = launch_gram(h, real, std::min(kMaxGramDim, K * h->rank));
-        if (e == cudaSuccess) e = launch_eig_truncate(h, 0, normalize);
-        if (e == cudaSuccess) e = launch_project(h, real, K, p->rank_kmax);
+        const bool diag = g.noise == QS_NOISE_PHASE && gate_diagonal(g.U, g.k);
+        e = launch_rank_channel(h, tg, real, diag, nullptr, K, 0, kg, h->rank, p->rank_kmax, normalize);
       }
     }
     if (e != cudaSuccess) return pfail(p, QS_ERR_CUDA, std::string("fixed-rank plan: ") + cudaGetErrorString(e));
@@ -1934,7 +1932,13 @@ qs_status qs_plan_create(qs_handle h, const qs_gate* gates, int num_gates, qs_pl
   count_launches(p);
   if (!p->rank_ops.empty()) {
     p->kernels -= 1;
-    for (const RankOp& op : p->rank_ops) p->kernels += op.kind == 4 ? 5 : 1;   // channel: expand, Gram x 2, eig, project
+    for (const RankOp& op : p->rank_ops) {
+      // a channel: moments, eigensolver, projection; a dense two-qubit one:
+      // expansion, Gram matrix (two), eigensolver, projection
+      const qs_gate& g = p->gates[op.gate].g;
+      const bool through_work = g.k == 2 && !(g.noise == QS_NOISE_PHASE && gate_diagonal(g.U, g.k));
+      p->kernels += op.kind == 4 ? (through_work ? 5 : 3) : 1;
+    }
     if (rank_kernel_attributes() != cudaSuccess) { qs_plan_destroy(p); return QS_ERR_CUDA; }
   }
   *out = p;
