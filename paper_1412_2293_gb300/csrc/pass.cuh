@@ -103,10 +103,20 @@ struct PassArgs {
   uint64_t tiles;
   int tile_shift;             // log2(tiles per member)
   int* status;                // device status word
-  // first pass of a run started from basis states: synthesise, do not load
+  // A run started from basis states: the amplitudes that can differ from zero
+  // are those whose inactive qubits (no dense gate so far) still have the start's
+  // values.  synth = kUnit: the start itself, synthesised; kMasked: only the
+  // amplitudes whose qubits in `inact` have the start's values are read, straight
+  // into registers, the others are taken as zero (whatever memory holds there).
+  // rshift >= 0: only the tiles whose inactive outside bits match the start are
+  // run, 2^rshift per member, tile_active = their free bits among the tile index.
   int synth;
+  int rshift;
+  uint64_t tile_active;
+  uint64_t inact;
   const uint64_t* basis;      // per-member basis index, or null: basis0
   const uint64_t* basis0;     // device word
+  uint64_t basis_mask;        // qubits of it the pass sees (a pass over one window alone)
   // last pass of a run with a fused fidelity: partials of <ref|psi>
   int fid;
   const void* ref;            // 2^n reference amplitudes
@@ -124,6 +134,19 @@ struct PassArgs {
   // take kSpinLimit
   uint32_t spin_limit;
 };
+
+enum : int { kLoad = 0, kUnit = 1, kMasked = 3 };   // PassArgs::synth
+
+// the low bits of v spread over the set bits of mask
+__device__ __forceinline__ uint64_t deposit(uint64_t v, uint64_t mask) {
+  uint64_t r = 0;
+  for (; mask; mask &= mask - 1, v >>= 1)
+    if (v & 1) r |= mask & (~mask + 1);
+  return r;
+}
+__device__ __forceinline__ uint64_t start_index(const PassArgs& A, uint64_t member) {
+  return (A.basis ? A.basis[member] : A.basis0[0]) & A.basis_mask;
+}
 
 // First window bit held in registers in stage S of a window of M bits.
 __host__ __device__ constexpr int stage_base(int m, int s) { return s == 0 ? m - kRegBits : (s == 1 ? 0 : 5); }
@@ -653,7 +676,12 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
         }
       }
     };
-    const uint64_t base = ti << M;
+    uint64_t base = ti << M;
+    if (A.rshift >= 0) {
+      const uint64_t b = ti >> A.rshift, x = start_index(A, b);
+      const uint64_t tl = deposit(ti & ((1ull << A.rshift) - 1), A.tile_active) | ((x >> M) & ~A.tile_active);
+      base = (b << A.n) | (tl << M);
+    }
     const uint64_t member = base >> A.n;
     const uint64_t mloc = base & nmask;
     const R* P = params + member * (uint64_t)A.param_stride;
@@ -661,9 +689,18 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
     // read at the end of the tile: into L1 now
     if (A.alpha_tab && wig == 0 && lane < 2) prefetch_l1(static_cast<const C*>(A.alpha_tab) + aidx + lane * 8);
     C a[kAmps];
-    if (A.synth) {
+    if (A.synth == kMasked) {
+      const uint64_t x = start_index(A, member), i0 = mloc | (uint64_t)t;
+      constexpr int sh = M - kRegBits;
+      const bool own = ((i0 ^ x) & A.inact & ~(31ull << sh)) == 0;
+      const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
+      const C* src = psi + base + t;
+#pragma unroll
+      for (int r = 0; r < kAmps; ++r)
+        a[r] = own && ((r ^ xr) & rmask) == 0 ? src[r << sh] : mk<R>(R(0), R(0));
+    } else if (A.synth) {
       // the one amplitude equal to 1: register x >> (M-5) & 31 of thread x & (2^(M-5) - 1)
-      const uint64_t x = A.basis ? A.basis[member] : A.basis0[0];
+      const uint64_t x = start_index(A, member);
 #pragma unroll
       for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
       if ((x & ~(uint64_t)(S::TILE - 1)) == mloc && (int)(x & ((1u << (M - 5)) - 1)) == t) {
@@ -902,8 +939,14 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
         }
       }
     };
-    const uint64_t member = t >> A.tile_shift;
-    const uint64_t tl = t & ((1ull << A.tile_shift) - 1);
+    uint64_t member = t >> A.tile_shift;
+    uint64_t tl = t & ((1ull << A.tile_shift) - 1);
+    if (A.rshift >= 0) {
+      member = t >> A.rshift;
+      const uint64_t x = start_index(A, member);
+      const uint64_t xt = ((x >> (c0 + M)) << cshift) | ((x >> COLB) & cmask);
+      tl = deposit(t & ((1ull << A.rshift) - 1), A.tile_active) | (xt & ~A.tile_active);
+    }
     // member-local offset of the tile (bits outside the window and the
     // columns), and the same bits packed below each other (the out-factor
     // table's index: bits below the window, then the bits above it)
@@ -920,10 +963,23 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
     }
     C a[kAmps];
     int stage = A.start_stage;
-    if (A.synth) {
+    if (A.synth == kMasked) {
+      const uint64_t x = start_index(A, member);
+      with_stage<M>(stage, [&](auto SC) {
+        constexpr int SS = decltype(SC)::value;
+        const int sh = c0 + stage_base(M, SS);
+        const Off fixed = tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0);
+        const bool own = (((uint64_t)fixed ^ x) & A.inact & ~(31ull << sh)) == 0;
+        const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
+        const C* src = psi + (member << A.n) + fixed;
+#pragma unroll
+        for (int r = 0; r < kAmps; ++r)
+          a[r] = own && ((r ^ xr) & rmask) == 0 ? src[(Off)r << sh] : mk<R>(R(0), R(0));
+      });
+    } else if (A.synth) {
       // the one amplitude equal to 1: register (x >> sh) & 31 of the thread
       // whose other bits match (one thread of the member's whole state)
-      const uint64_t x = A.basis ? A.basis[member] : A.basis0[0];
+      const uint64_t x = start_index(A, member);
 #pragma unroll
       for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
       with_stage<M>(stage, [&](auto SC) {

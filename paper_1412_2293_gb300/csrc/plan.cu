@@ -522,6 +522,152 @@ __global__ void __launch_bounds__(256) k_out_table(cplx<R>* __restrict__ tab, co
   }
 }
 
+// The out factors of the tiles that a pass from a basis start runs (see
+// PassArgs::rshift): entries o whose inactive bits have the start's values,
+// active = the free bits, one thread per entry and attach.
+template <typename R>
+__global__ void __launch_bounds__(256) k_out_entries(cplx<R>* __restrict__ tab, const R* __restrict__ params, int stride,
+                                                     const OutTerm* __restrict__ outs, OutStarts starts, int diag_off,
+                                                     int obits, int wstart, int m, uint64_t active, int shift,
+                                                     uint64_t members, const uint64_t* basis, const uint64_t* basis0) {
+  const int A = m + 1;
+  const uint64_t total = (members << shift) * A;
+  for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += (uint64_t)gridDim.x * blockDim.x) {
+    const int a = (int)(k % A);
+    const uint64_t e = k / A, b = e >> shift;
+    const uint64_t x = basis ? basis[b] : basis0[0];
+    const uint64_t low = (1ull << wstart) - 1;
+    const uint64_t xo = ((x >> (wstart + m)) << wstart) | (x & low);
+    const uint64_t o = deposit(e & ((1ull << shift) - 1), active) | (xo & ~active);
+    const uint64_t full = ((o >> wstart) << (wstart + m)) | (o & low);
+    const R* P = params + b * (uint64_t)stride;
+    cplx<R> v = mk<R>(diag_off >= 0 ? P[diag_off + a] : R(1), R(0));
+    for (int q = starts.v[a]; q < starts.v[a + 1]; ++q) {
+      const OutTerm t = outs[q];
+      if ((full & t.cmask) == t.cmask) v = cmul(v, mk<R>(P[t.off], P[t.off + 1]));
+    }
+    tab[((b << obits) | o) * A + a] = v;
+  }
+}
+
+// The pass that completes the support of a run from basis states, when none of
+// its window's qubits is active before it (low window, no out terms, no flips):
+// every tile then holds one amplitude c at the start's window value, and the pass
+// is linear, so tile y becomes c_y V with V the pass applied to the start's
+// window state alone.  V is computed by the pass kernel itself (one tile per
+// member), the c_y are gathered, and this kernel writes the product (and reduces
+// <ref|psi>): bound by the HBM write of the state.  A block keeps 1024 entries
+// of V of MB members in registers and takes a run of tiles y, so the reference's
+// entries are read once for MB members.  Each member's overlap is summed over a
+// tile's 4 entries per thread in R and over the tiles by compensated sums in R
+// (two floats; FP64 for complex128), then in FP64 across the block.
+constexpr int kOuterThreads = 256;
+constexpr int kOuterTiles = 32;          // tiles of a block
+template <typename R> struct Acc2 {      // running sum with its rounding errors
+  R s = R(0), c = R(0);
+  __device__ __forceinline__ void add(R v) {
+    if constexpr (sizeof(R) == 4) {
+      const float t = __fadd_rn(s, v), z = __fadd_rn(t, -s);
+      c = __fadd_rn(c, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(v, -z)));
+      s = t;
+    } else {
+      s += v;
+    }
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
+template <typename R, int MB, bool FID>
+__global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ psi, const cplx<R>* __restrict__ V,
+                                                         const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ ref,
+                                                         double* __restrict__ fid, int n, int m, int members) {
+  using C = cplx<R>;
+  constexpr int W = sizeof(R) == 4 ? 2 : 1;              // amplitudes of a 16-byte vector
+  constexpr int L = 4 / W;                               // vectors per thread
+  struct alignas(16) Vec { C v[W]; };
+  const uint64_t tiles = 1ull << (n - m);
+  const int slices = 1 << (m - 10);                      // 1024-amplitude slices of a tile
+  const unsigned runs = (unsigned)((tiles + kOuterTiles - 1) / kOuterTiles);
+  const unsigned run = blockIdx.x % runs;                // grid: runs of tiles, groups of members
+  const uint64_t y0 = (uint64_t)run * kOuterTiles;
+  const uint64_t y1 = y0 + kOuterTiles < tiles ? y0 + kOuterTiles : tiles;
+  const int slice = blockIdx.y;
+  const int b0 = (int)(blockIdx.x / runs) * MB;
+  const uint64_t off = (uint64_t)slice * 1024;
+  Vec v[MB][L];
+  Acc2<R> ar[MB], ai[MB];
+#pragma unroll
+  for (int b = 0; b < MB; ++b)
+#pragma unroll
+    for (int l = 0; l < L; ++l)
+      if (b0 + b < members)
+        v[b][l] = *reinterpret_cast<const Vec*>(V + (((uint64_t)(b0 + b)) << m) + off + (l * kOuterThreads + threadIdx.x) * W);
+  for (uint64_t y = y0; y < y1; ++y) {
+    Vec r[L];
+    if constexpr (FID) {
+#pragma unroll
+      for (int l = 0; l < L; ++l)
+        r[l] = *reinterpret_cast<const Vec*>(ref + (y << m) + off + (l * kOuterThreads + threadIdx.x) * W);
+    }
+#pragma unroll
+    for (int b = 0; b < MB; ++b) {
+      if (b0 + b >= members) break;
+      const C c = cs[((uint64_t)(b0 + b) << (n - m)) + y];
+      C* out = psi + ((uint64_t)(b0 + b) << n) + (y << m) + off;
+      C d = mk<R>(R(0), R(0));
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        Vec o;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          o.v[w] = pmul<R>(c, v[b][l].v[w]);
+          if constexpr (FID) d = pdot<R>(d, r[l].v[w], o.v[w]);
+        }
+        __stcs(reinterpret_cast<typename std::conditional<sizeof(R) == 4, float4, double2>::type*>(out + (l * kOuterThreads + threadIdx.x) * W),
+               *reinterpret_cast<typename std::conditional<sizeof(R) == 4, float4, double2>::type*>(&o));
+      }
+      if constexpr (FID) {
+        ar[b].add(d.x);
+        ai[b].add(d.y);
+      }
+    }
+  }
+  if constexpr (FID) {
+    __shared__ double red[2][kOuterThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = 0; b < MB && b0 + b < members; ++b) {
+      double re = 0.0, im = 0.0;
+#pragma unroll
+      for (int k = 0; k < MB; ++k)
+        if (k == b) { re = ar[k].value(); im = ai[k].value(); }
+      re = warp_sum_d(re);
+      im = warp_sum_d(im);
+      __syncthreads();
+      if (lane == 0) { red[0][warp] = re; red[1][warp] = im; }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double sr = 0.0, si = 0.0;
+        for (int w = 0; w < kOuterThreads / 32; ++w) { sr += red[0][w]; si += red[1][w]; }
+        const uint64_t slot = ((uint64_t)(b0 + b) * runs + run) * slices + slice;
+        fid[2 * slot] = sr;
+        fid[2 * slot + 1] = si;
+      }
+    }
+  }
+}
+
+// c_y of every tile y of every member (see k_outer)
+template <typename R>
+__global__ void __launch_bounds__(256) k_gather_start(const cplx<R>* __restrict__ psi, cplx<R>* __restrict__ cs, int n,
+                                                      int m, uint64_t total, const uint64_t* basis,
+                                                      const uint64_t* basis0) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t b = i >> (n - m);
+    const uint64_t x = (basis ? basis[b] : basis0[0]) & ((1ull << m) - 1);
+    cs[i] = psi[(i << m) | x];
+  }
+}
+
 // A run of diagonal channels on the exact density matrix (Sec. 3): noiseless
 // diagonal gates and phase flips (rho -> D rho D^dagger) and noisy diagonal
 // gates with the phase-noise Kraus pair of Eq. 9.  Each multiplies rho[x][y]
@@ -592,6 +738,7 @@ struct PassPlan {
   int tile_shift = 0;             // log2(tiles per member)
   std::vector<Seg> segs;          // the ops in canonical segments (what the kernels run)
   int prog = 0;                   // compile-time program of the pass kernel (0: interpreted)
+  uint64_t dense = 0;             // qubits its dense gates act on
   std::vector<Flip> flips;
   CUtensorMap tmap;               // HIGH: [members * 2^(n-c) rows][2^c columns] (c = win[0]), boxes of 2^colb columns
   CUtensorMap tmap4;              // HIGH complex64, m = 10: the same with boxes of 4 columns (configuration 2)
@@ -664,6 +811,15 @@ struct qs_plan_s {
   int launches = 0;               // timing slots of a run (precompute, pass, single step)
   int kernels = 0;                // kernels one run launches
   bool timing = false;
+  // Runs from basis states: the support grows by the qubits each pass's dense
+  // gates act on.  start_full = the first step that completes it (all steps up to it
+  // fused passes; -1: none, the first pass then writes the whole state);
+  // start_outer: that pass runs as one window and an outer product (k_outer), with
+  // these buffers.
+  int start_full = -1;
+  bool start_outer = false;
+  void* d_start_c = nullptr;
+  void* d_start_v = nullptr;
   std::vector<cudaEvent_t> events;     // launches + 1 when timing
   std::vector<int> event_kinds;
   std::string err;
@@ -752,11 +908,11 @@ bool two_shear_safe(const std::vector<PGate>& gates, double e_max) {
 // gates; -1 when none is allowed (c >= colb, and the tensor map's row
 // coordinate, members x 2^(n-c), within 31 bits).
 int choose_window(const std::vector<PGate>& G, const std::vector<int>& rem, int n, int colb, uint64_t batch, int q,
-                  int m) {
+                  int m, bool split) {
   int best = -1, best_count = -1;
   const int cand[3] = {n - m, q - (m - 1), q};
   for (int c : cand) {
-    c = std::min(std::max(c, colb), n - m);
+    c = std::min(std::max(c, split ? std::max(m, colb) : colb), n - m);
     if (c < colb || q < c || q >= c + m) continue;
     if (n - c >= 31 || (batch << (n - c)) >= (1ull << 31)) continue;
     int count = 0;
@@ -771,7 +927,7 @@ int choose_window(const std::vector<PGate>& G, const std::vector<int>& rem, int 
 }
 
 bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n, int colb, uint64_t batch,
-                size_t op_budget, int m, PassPlan* P, std::vector<char>* absorbed) {
+                size_t op_budget, int m, bool split, PassPlan* P, std::vector<char>* absorbed) {
   P->colb = colb;
   P->m = m;
   // window from the first fusable dense gate (lookahead)
@@ -785,7 +941,7 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
   int c0 = 0;
   if (q >= m) {
     if (n < m + colb) return false;                  // a high tile needs 2^colb columns
-    c0 = choose_window(G, rem, n, colb, batch, q, m);
+    c0 = choose_window(G, rem, n, colb, batch, q, m, split);
     if (c0 < 0) return false;
     P->high = true;
   }
@@ -830,7 +986,7 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
     if (ok) {
       if (g.dense1) {
         const int l = loc[g.g.targets[0]];
-        can = l >= 0 && !((locked >> l) & 1);
+        can = l >= 0 && !((locked >> l) & 1) && !(split && P->high && g.g.targets[0] < m);
       } else {
         can = true;                                     // diagonal gates always fit
       }
@@ -843,6 +999,7 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
     (*absorbed)[i] = 1;
     if (g.dense1) {
       const int l = loc[g.g.targets[0]];
+      P->dense |= 1ull << g.g.targets[0];
       need_stage(l);
       FOp x{};
       x.type = OP_DENSE;
@@ -1192,7 +1349,37 @@ int fid_slots(qs_plan p, const PassPlan& P) {
   return (1 << launch_tile_shift(p, P)) * (P.high ? 1 : 1 << (P.m - kWin));
 }
 
-PassArgs pass_args(qs_plan p, const PassPlan& P, int synth, int fid) {
+// How step i of a run executes: from memory, or as part of a run from basis
+// states (synth = 1: one start, 2: per member).
+struct PassMode {
+  int synth = 0;                 // the run's start (0: from memory)
+  int load = kLoad;              // PassArgs::synth
+  bool restricted = false;       // only the tiles of the support
+  bool outer = false;            // window state and outer product
+  uint64_t act = 0;              // active qubits before the pass
+};
+PassMode pass_mode(qs_plan p, size_t i, int synth) {
+  PassMode M;
+  if (!synth) return M;
+  if (p->start_full < 1) {       // the first pass writes the whole state
+    if (i == 0) { M.synth = synth; M.load = kUnit; M.act = 0; }
+    return M;
+  }
+  if ((int)i > p->start_full) return M;
+  M.synth = synth;
+  for (size_t j = 0; j < i; ++j) M.act |= p->passes[p->steps[j].pass].dense;
+  M.load = i == 0 ? kUnit : kMasked;
+  M.restricted = (int)i < p->start_full;
+  // the outer product adds two launches (about 9 us) and saves the pass's
+  // arithmetic, 3 ps an amplitude in complex64 and 80 in complex128: 2^22 (2^18)
+  // amplitudes is where that is 12 us (21 us); 64 members of 13 qubits, 2^19, took
+  // 182 us a launch with it and 172 without
+  const uint64_t amps = (uint64_t)p->h->batch << p->h->n;
+  M.outer = (int)i == p->start_full && p->start_outer && p->d_start_v && amps >= (p->h->esize == 8 ? 1ull << 22 : 1ull << 18);
+  return M;
+}
+
+PassArgs pass_args(qs_plan p, const PassPlan& P, const PassMode& mode, int fid) {
   qs_ctx* h = p->h;
   PassArgs A{};
   A.n = h->n;
@@ -1210,8 +1397,19 @@ PassArgs pass_args(qs_plan p, const PassPlan& P, int synth, int fid) {
   A.tile_shift = launch_tile_shift(p, P);
   A.tiles = total >> (P.m + launch_colb(p, P));
   A.status = h->dstatus + 2;
-  A.synth = synth ? 1 : 0;
-  A.basis = synth == 2 ? h->m_basis : nullptr;
+  A.synth = mode.load;
+  A.rshift = -1;
+  A.basis_mask = ~0ull;
+  A.inact = ((1ull << h->n) - 1) & ~mode.act;
+  if (mode.restricted) {
+    // the tile index: the bits between the columns and the window, then those above it
+    const int cb = launch_colb(p, P), c0 = P.win[0];
+    A.tile_active = P.high ? ((mode.act >> cb) & ((1ull << (c0 - cb)) - 1)) | ((mode.act >> (c0 + P.m)) << (c0 - cb))
+                           : mode.act >> P.m;
+    A.rshift = __builtin_popcountll(A.tile_active);
+    A.tiles = (uint64_t)h->batch << A.rshift;
+  }
+  A.basis = mode.synth == 2 ? h->m_basis : nullptr;
   A.basis0 = &p->d_run->basis;
   A.fid = fid;
   A.ref = h->ref;
@@ -1232,7 +1430,7 @@ size_t precompute_smem(size_t contribs, size_t dwin, size_t tab_entries, size_t 
 
 // Members' noise draws, matrices, phase tables and out factors of one pass.
 template <typename R>
-cudaError_t launch_precompute(qs_plan p, const PassPlan& P, cudaStream_t s) {
+cudaError_t launch_precompute(qs_plan p, const PassPlan& P, const PassMode& mode, cudaStream_t s) {
   qs_ctx* h = p->h;
   NoiseSrc src{};
   if (h->member_noise) { src.e = h->m_e; src.seed = h->m_seed; src.traj = h->m_traj; }
@@ -1246,6 +1444,17 @@ cudaError_t launch_precompute(qs_plan p, const PassPlan& P, cudaStream_t s) {
     for (int i = 0; i < kMaxWin + 2; ++i) st.v[i] = P.out_start[i];
     const int obits = h->n - P.m;
     const int nterms = P.out_start[P.m + 1];
+    if (mode.restricted) {
+      const int c0 = P.win[0];
+      const uint64_t active = (mode.act & ((1ull << c0) - 1)) | ((mode.act >> (c0 + P.m)) << c0);
+      const int shift = __builtin_popcountll(active);
+      const uint64_t total = ((uint64_t)h->batch << shift) * (P.m + 1);
+      const unsigned g = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16);
+      k_out_entries<R><<<g, 256, 0, s>>>((cplx<R>*)P.d_alpha, (const R*)P.d_params, P.stride, P.d_outs, st, P.diag_off, obits,
+                                         c0, P.m, active, shift, (uint64_t)h->batch,
+                                         mode.synth == 2 ? h->m_basis : nullptr, &p->d_run->basis);
+      return cudaGetLastError();
+    }
     const int L = obits < kOutLoBits ? obits : kOutLoBits;
     const int rows = out_table_rows(obits, P.m);
     const uint32_t chunks = (uint32_t)(((1ull << (obits - L)) + rows - 1) / rows);
@@ -1259,17 +1468,14 @@ cudaError_t launch_precompute(qs_plan p, const PassPlan& P, cudaStream_t s) {
 }
 
 template <typename R>
-cudaError_t launch_pass_kernel(qs_plan p, const PassPlan& P, cudaStream_t s, int synth, int fid) {
+cudaError_t launch_pass_args(qs_plan p, const PassPlan& P, const PassArgs& A, cplx<R>* psi, cudaStream_t s) {
   using C = cplx<R>;
-  qs_ctx* h = p->h;
-  const PassArgs A = pass_args(p, P, synth, fid);
   const int prog = p->stable ? 0 : P.prog;               // the compiled programs take two shears
   const int sms = num_sms();
   auto grid = [&](uint64_t units, int per_sm) {
     const uint64_t cap = (uint64_t)sms * per_sm;
     return (int)(units < cap ? units : cap);
   };
-  C* psi = (C*)h->state;
   constexpr int kQft = prog_layers(0x1f, 0x1e);
   if constexpr (sizeof(R) == 4) {
     // wider windows (n <= 32, checked when the width is set)
@@ -1315,6 +1521,45 @@ cudaError_t launch_pass_kernel(qs_plan p, const PassPlan& P, cudaStream_t s, int
     k_pass_high<R, CB, 2><<<grid(A.tiles, 1), HighShape<CB>::THREADS, high_smem<R, CB, 2>(), s>>>(psi, P.tmap, A);
   }
   return cudaGetLastError();
+}
+
+// fidelity slots per member of the outer product
+int outer_slots(qs_plan p, const PassPlan& P) {
+  const uint64_t tiles = 1ull << (p->h->n - P.m);
+  return (int)((tiles + kOuterTiles - 1) / kOuterTiles) << (P.m - kWin);
+}
+
+// The pass on the start's window state alone, one tile per member, then the
+// outer product with the amplitudes it starts from (see k_outer).
+template <typename R>
+cudaError_t launch_outer(qs_plan p, const PassPlan& P, const PassMode& mode, int fid, cudaStream_t s) {
+  using C = cplx<R>;
+  qs_ctx* h = p->h;
+  PassArgs A = pass_args(p, P, mode, 0);
+  const uint64_t total = (uint64_t)h->batch << (h->n - P.m);
+  const unsigned g = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16);
+  k_gather_start<R><<<g, 256, 0, s>>>((const C*)h->state, (C*)p->d_start_c, h->n, P.m, total, A.basis, A.basis0);
+  A.synth = kUnit;
+  A.n = P.m;
+  A.tile_shift = 0;
+  A.tiles = (uint64_t)h->batch;
+  A.basis_mask = (1ull << P.m) - 1;
+  cudaError_t e = launch_pass_args<R>(p, P, A, (C*)p->d_start_v, s);
+  if (e != cudaSuccess) return e;
+  constexpr int MB = sizeof(R) == 4 ? 4 : 2;
+  const unsigned runs = (unsigned)(((1ull << (h->n - P.m)) + kOuterTiles - 1) / kOuterTiles);
+  const dim3 grid(runs * (unsigned)((h->batch + MB - 1) / MB), 1u << (P.m - kWin));
+  auto* psi = (C*)h->state;
+  auto *v = (const C*)p->d_start_v, *c = (const C*)p->d_start_c, *ref = (const C*)h->ref;
+  if (fid) k_outer<R, MB, true><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, p->d_fid, h->n, P.m, h->batch);
+  else k_outer<R, MB, false><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, p->d_fid, h->n, P.m, h->batch);
+  return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_pass_kernel(qs_plan p, const PassPlan& P, cudaStream_t s, const PassMode& mode, int fid) {
+  if (mode.outer) return launch_outer<R>(p, P, mode, fid, s);
+  return launch_pass_args<R>(p, P, pass_args(p, P, mode, fid), (cplx<R>*)p->h->state, s);
 }
 
 cudaError_t set_smem_attrs(size_t esize) {
@@ -1556,14 +1801,14 @@ qs_status enqueue_run(qs_plan p, cudaStream_t s, int synth, int fid) {
     const Step& st = p->steps[i];
     if (st.kind == 0) {
       const PassPlan& P = p->passes[st.pass];
-      const int sy = i == 0 ? synth : 0;
+      const PassMode mode = pass_mode(p, i, synth);
       const int fd = (i + 1 == p->steps.size()) ? fid : 0;
-      cudaError_t e = f32 ? launch_precompute<float>(p, P, s) : launch_precompute<double>(p, P, s);
+      cudaError_t e = f32 ? launch_precompute<float>(p, P, mode, s) : launch_precompute<double>(p, P, mode, s);
       mark(0);
-      if (e == cudaSuccess) e = f32 ? launch_pass_kernel<float>(p, P, s, sy, fd) : launch_pass_kernel<double>(p, P, s, sy, fd);
+      if (e == cudaSuccess) e = f32 ? launch_pass_kernel<float>(p, P, s, mode, fd) : launch_pass_kernel<double>(p, P, s, mode, fd);
       mark(P.high ? 2 : 1);
       if (e == cudaSuccess && fd) {
-        e = launch_finalize(p->d_fid, h->batch, fid_slots(p, P), 0, 1, h->small + kSmallOutIndex, s);
+        e = launch_finalize(p->d_fid, h->batch, mode.outer ? outer_slots(p, P) : fid_slots(p, P), 0, 1, h->small + kSmallOutIndex, s);
       }
       if (e != cudaSuccess) { h->stream = saved; return pfail(p, QS_ERR_CUDA, std::string("fused pass: ") + cudaGetErrorString(e)); }
     } else {
@@ -1654,9 +1899,29 @@ qs_status run_plan(qs_plan p, double e, uint64_t seed, uint64_t gate_id0, int wa
   return st;
 }
 
+// Where the support of a run from basis states becomes the whole state, and
+// whether that pass can run as an outer product (see k_outer).
+void find_start(qs_plan p) {
+  p->start_full = -1;
+  p->start_outer = false;
+  const uint64_t all = (1ull << p->h->n) - 1;
+  uint64_t act = 0;
+  for (size_t i = 0; i < p->steps.size() && p->steps[i].kind == 0; ++i) {
+    const PassPlan& P = p->passes[p->steps[i].pass];
+    if ((act | P.dense) == all) {
+      p->start_full = (int)i;
+      const uint64_t win = (1ull << P.m) - 1;
+      p->start_outer = i > 0 && !P.high && (act & win) == 0 && P.out_start[P.m + 1] == 0 && P.flips.empty();
+      return;
+    }
+    act |= P.dense;
+  }
+}
+
 // Fused passes of a state-vector plan (window width p->m) for the gates in
-// rem, in order; a gate no pass can hold becomes a single step.
-void plan_passes(qs_plan p, std::vector<int> rem) {
+// rem, in order; a gate no pass can hold becomes a single step.  split: high
+// passes leave the qubits below m to the low window.
+void plan_passes_as(qs_plan p, std::vector<int> rem, bool split) {
   qs_ctx* h = p->h;
   const bool fuse = h->mode == QS_STATEVEC && h->n >= p->m;
   while (!rem.empty()) {
@@ -1669,7 +1934,7 @@ void plan_passes(qs_plan p, std::vector<int> rem) {
         std::fill(absorbed.begin(), absorbed.end(), 0);
         // a high window starts at or above the columns of a tile
         const int colb = p->m == kWin ? p->colb : wide_colb(p->m);
-        if (!build_pass(p->gates, rem, h->n, colb, (uint64_t)h->batch, budget, p->m, &P, &absorbed)) break;
+        if (!build_pass(p->gates, rem, h->n, colb, (uint64_t)h->batch, budget, p->m, split, &P, &absorbed)) break;
         built = segment_pass(&P);
         if (built) P.prog = choose_prog(P);
       }
@@ -1689,6 +1954,27 @@ void plan_passes(qs_plan p, std::vector<int> rem) {
     p->steps.push_back(Step{1, -1, rem[0]});
     rem.erase(rem.begin());
   }
+}
+
+// The same gates grouped so that a run from basis states ends in the outer
+// product, when that takes no more passes: the high passes then leave the qubits
+// below m, which the low window has to take anyway, to the low pass.  A run from
+// any other state does the same work in as many passes.
+void plan_passes(qs_plan p, const std::vector<int>& rem) {
+  const std::vector<Step> before = p->steps;
+  plan_passes_as(p, rem, false);
+  find_start(p);
+  if (p->start_outer || p->start_full < 1) return;
+  std::vector<PassPlan> passes;
+  std::vector<Step> steps = before;
+  passes.swap(p->passes);
+  steps.swap(p->steps);
+  plan_passes_as(p, rem, true);
+  find_start(p);
+  if (p->start_outer && p->steps.size() <= steps.size()) return;
+  p->passes.swap(passes);
+  p->steps.swap(steps);
+  find_start(p);
 }
 
 // Device copies of the passes' op lists, their tensor maps, and the buffers
@@ -1728,6 +2014,16 @@ qs_status alloc_passes(qs_plan p) {
   if (st == QS_OK && !p->passes.empty() &&
       cudaMalloc((void**)&p->d_fid, 2 * fid_slots_max * h->batch * sizeof(double)) != cudaSuccess)
     st = pfail(p, QS_ERR_OUT_OF_MEMORY, "fidelity partials");
+  if (st == QS_OK && p->start_outer) {
+    // without room for these the pass runs on every tile instead
+    const PassPlan& P = p->passes[p->steps[p->start_full].pass];
+    if (cudaMalloc(&p->d_start_c, ((size_t)h->batch << (h->n - P.m)) * h->esize) != cudaSuccess ||
+        cudaMalloc(&p->d_start_v, ((size_t)h->batch << P.m) * h->esize) != cudaSuccess) {
+      cudaGetLastError();
+      if (p->d_start_c) cudaFree(p->d_start_c);
+      p->d_start_c = p->d_start_v = nullptr;
+    }
+  }
   return st;
 }
 
@@ -1740,6 +2036,9 @@ void free_passes(qs_plan p) {
   if (p->d_params) cudaFree(p->d_params);
   if (p->d_alpha) cudaFree(p->d_alpha);
   if (p->d_fid) cudaFree(p->d_fid);
+  if (p->d_start_c) cudaFree(p->d_start_c);
+  if (p->d_start_v) cudaFree(p->d_start_v);
+  p->d_start_c = p->d_start_v = nullptr;
   p->d_params = p->d_alpha = nullptr;
   p->d_fid = nullptr;
 }
@@ -1999,15 +2298,16 @@ qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t
   cudaEventRecord(ev[k++], h->stream);
   for (int r = 0; r < reps && result == QS_OK; ++r) {
     int li = 0;
-    for (const Step& st : p->steps) {
+    for (size_t si = 0; si < p->steps.size(); ++si) {
+      const Step& st = p->steps[si];
       if (st.kind == 0) {
         const PassPlan& P = p->passes[st.pass];
         const bool f32 = h->dtype == QS_C64;
-        const int sy = li == 0 ? synth : 0;
-        cudaError_t x = f32 ? launch_precompute<float>(p, P, h->stream) : launch_precompute<double>(p, P, h->stream);
+        const PassMode mode = pass_mode(p, si, synth);
+        cudaError_t x = f32 ? launch_precompute<float>(p, P, mode, h->stream) : launch_precompute<double>(p, P, mode, h->stream);
         cudaEventRecord(ev[k++], h->stream);
         kind[li++] = 0;
-        if (x == cudaSuccess) x = f32 ? launch_pass_kernel<float>(p, P, h->stream, sy, 0) : launch_pass_kernel<double>(p, P, h->stream, sy, 0);
+        if (x == cudaSuccess) x = f32 ? launch_pass_kernel<float>(p, P, h->stream, mode, 0) : launch_pass_kernel<double>(p, P, h->stream, mode, 0);
         cudaEventRecord(ev[k++], h->stream);
         kind[li++] = P.high ? 2 : 1;
         if (x != cudaSuccess) { result = pfail(p, QS_ERR_CUDA, cudaGetErrorString(x)); break; }
@@ -2248,7 +2548,11 @@ qs_status qs_plan_last_times(qs_plan p, double* ms, int* kinds, int cap, int* co
 qs_status qs_plan_info(qs_plan p, int* passes, int* launches) {
   if (!p) return QS_ERR_INVALID_ARG;
   if (passes) *passes = (int)p->steps.size();
-  if (launches) *launches = p->kernels;
+  if (launches) {
+    *launches = p->kernels;
+    // the gather and the outer product beside the pass they run
+    if (p->h->pending && p->start_full > 0 && pass_mode(p, (size_t)p->start_full, p->h->pending).outer) *launches += 2;
+  }
   return QS_OK;
 }
 
