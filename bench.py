@@ -207,11 +207,9 @@ def run_ours(args, rank, world, local_rank):
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
-    order_kinds = []
     for _ in range(args.steps):
         fid = step()
         ms, kinds = qs.qs_plan_last_times(p, h=h)
-        order_kinds = [k for k in kinds if k.startswith("pass")]
         for m, k in zip(ms, kinds):
             kern.setdefault(k, []).append(m)
     ev1.record(stream)
@@ -961,7 +959,13 @@ def run_channels(args, rank, world, local_rank):
         # diagonal: half of it (the sweeps on qubits below 5 still do all of it)
         totals = {k: len(per_kind[k]) * kinds[k] for k in kinds}
         dom = max(totals, key=totals.get)
-        flop = (1 << (2 * n)) * (14 if dom == "dm_diag_block" else 16) // 2
+        if dom == "dm_window":
+            # a window sweep: the circuit's Hadamards and the runs of controlled phases
+            # between them, shared out over its sweeps
+            nh = sum(1 for o in ops if o.kind == "H")
+            flop = (1 << (2 * n)) * (16 * nh + 14 * (nh - 1)) // 2 * args.steps // len(per_kind[dom])
+        else:
+            flop = (1 << (2 * n)) * (14 if dom == "dm_diag_block" else 16) // 2
         bytes_ = 3 * (1 << (2 * n)) * 16 // 2
     else:
         # the whole step: every channel's Gram matrix (M(M+1)/2 pairs of columns) and
@@ -996,6 +1000,7 @@ def run_channels(args, rank, world, local_rank):
                         "frac": round(achieved / fp64_peak, 4), "traffic": None,
                         "kernel": {"H_channel": "noisy-H channel (all its launches)",
                                    "dm_diag_block": "k_dm_diag_block (runs of diagonal channels)",
+                                   "dm_window": "k_dm_window (channels of five qubits and the diagonal runs between)",
                                    "fixed_rank_step": "the whole circuit (expansion, Gram, eigensolver, "
                                                       "projection per channel)"}.get(dom, dom),
                         "avg_launch_ms": round(avg, 4),

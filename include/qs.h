@@ -357,7 +357,9 @@ qs_status qs_plan_destroy(qs_plan p);
  * used up afterwards).  ms[i] = mean duration of launch i of a run, kinds[i] =
  * 0 noise/parameter precompute, 1 low-window pass, 2 high-window pass,
  * 3 single-gate step (all kernels of the step together), 4 density-matrix
- * run of diagonal channels (one sweep); at most `cap`
+ * run of diagonal channels (one sweep), 5 density-matrix window sweep (one-qubit
+ * channels on a few qubits and the diagonal channels between them, one sweep; from
+ * 8 qubits in complex64, 11 in complex128); at most `cap`
  * entries, *count = launches per run.  Synchronises. */
 qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t gate_id0,
                           double* ms, int* kinds, int cap, int* count);

@@ -344,6 +344,14 @@ qs_status materialize_basis(qs_ctx* h) {
   return QS_OK;
 }
 
+void dm_real_superop1(const double* U, int noisy, int noise, double e, double* S) {
+  const auto M = to_cplx(U, 2);
+  std::vector<std::vector<cd>> ks = {M};
+  if (noisy) ks = averaged_kraus(M, 1, noise, e);
+  const auto sup = superop(ks, 2);
+  for (int i = 0; i < 16; ++i) S[i] = sup[i].real();
+}
+
 NoiseSrc noise_src(qs_ctx* h, double e, uint64_t seed) {
   NoiseSrc s{};
   s.e0 = e;
@@ -650,6 +658,19 @@ qs_status qs_apply_relaxation(qs_handle h, const int* qubits, int count, double 
   { const qs_status st = qs::materialize_basis(h); if (st != QS_OK) return st; }
   const double keep = std::exp(-t / T1), c = std::exp(-t / T2), gamma = 1.0 - keep;
   if (count == 0 || (gamma == 0.0 && c == 1.0)) return QS_OK;
+  if (h->mode == QS_DENSITY && h->hermitian && qs::dm_window_applicable(h)) {
+    // several qubits per sweep of the upper triangle
+    QS_CUDA(h, qs::dm_window_attributes(h));
+    const int w = qs::dm_window_qubits(h);
+    for (int i = 0; i < count; i += w) {
+      qs::DmWindowOp ops[qs::kDmWindowOps];
+      const int m = std::min(w, count - i);
+      for (int k = 0; k < m; ++k)
+        ops[k] = qs::DmWindowOp{qubits[i + k], {1, 0, 0, gamma, 0, c, 0, 0, 0, 0, c, 0, 0, 0, 0, keep}, nullptr, nullptr, 1.0, 1};
+      QS_CUDA(h, qs::launch_dm_window(h, ops, m));
+    }
+    return QS_OK;
+  }
   if (h->mode == QS_DENSITY) {
     QS_CUDA(h, qs::launch_dm_relax(h, h->state, h->n, qubits, count, gamma, keep, c));
     return QS_OK;

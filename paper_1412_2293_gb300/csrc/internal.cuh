@@ -194,6 +194,27 @@ cudaError_t launch_dm_relax(qs_ctx* h, void* rho, int n, const int* qubits, int 
 // memory.  S_dev: 16 values of the handle's precision with stride 2.
 cudaError_t launch_dm_superop1_herm(qs_ctx* h, void* rho, int n, int t, const void* S_dev);
 
+// One item of a window sweep of a Hermitian density matrix (dm.cu): a one-qubit
+// channel with a real superoperator S (row-major, local index bit 0 = column bit,
+// bit 1 = row bit) on `qubit` (-1: none), then a run of diagonal channels given by
+// its tables (u in the handle's precision, mask; null: none) and sqrt(P).
+struct DmWindowOp {
+  int qubit;
+  double S[16];
+  const void* u;
+  const uint32_t* mask;
+  double q;
+  int relax = 0;                       // 1: S is a T1/T2 relaxation (S[3] = gamma, S[15] = keep, S[5] = c)
+};
+constexpr int kDmWindowOps = 10;       // items of a sweep at most
+bool dm_window_applicable(const qs_ctx* h);
+int dm_window_qubits(const qs_ctx* h); // distinct qubits of a sweep's channels
+cudaError_t dm_window_attributes(const qs_ctx* h);
+cudaError_t launch_dm_window(qs_ctx* h, const DmWindowOp* ops, int nops);
+// Real superoperator of a one-qubit gate's channel (noisy: the averaged set at e;
+// U real), S[16] as above.
+void dm_real_superop1(const double* U, int noisy, int noise, double e, double* S);
+
 // reductions (results land in h->small, as doubles)
 // reductions over `members` state vectors of 2^n; with group > 1 the values
 // of each run of `group` consecutive members are added (a fixed-rank

@@ -753,9 +753,9 @@ struct PassPlan {
 
 struct Step {
   int kind;               // 0 = fused pass, 1 = single gate, 2 = density-matrix diagonal block,
-                          // 5 = the gates of a fixed-rank plan (RankOp list)
+                          // 5 = the gates of a fixed-rank plan (RankOp list), 6 = density-matrix window sweep
   int pass = -1;
-  int gate = -1;          // single gate, or the diagonal block's index
+  int gate = -1;          // single gate, the diagonal block's index, or the sweep's (dm_sweeps)
 };
 
 // One gate of a fixed-rank plan, applied to every member with launch shapes
@@ -773,6 +773,12 @@ struct DmBlock {          // density matrix: a run of diagonal channels (k_dm_di
   float2* d_uf = nullptr;         // complex64 handles
   uint32_t* d_mask = nullptr;
   int noisy = 0;
+};
+
+// One window sweep: channels (a gate's index) and diagonal blocks, in order.
+struct DmSweep {
+  struct Item { int gate; int block; };  // one of them -1
+  std::vector<Item> items;
 };
 
 }  // namespace
@@ -799,6 +805,7 @@ struct qs_plan_s {
   void* d_params = nullptr;       // per-member gate parameters of the running pass (shared by the passes)
   void* d_alpha = nullptr;        // out factors of the running pass (shared by the passes)
   std::vector<DmBlock> dm_blocks;
+  std::vector<DmSweep> dm_sweeps;
   std::vector<RankOp> rank_ops;   // FIXED_RANK plans
   void* d_rank_mats = nullptr;
   int rank_variant = 0;           // the running variant: real start, per-member noise, normalisation
@@ -1695,11 +1702,80 @@ qs_status run_dm_block(qs_plan p, const DmBlock& b, const RunParams& rp) {
   return e == cudaSuccess ? QS_OK : pfail(p, QS_ERR_CUDA, cudaGetErrorString(e));
 }
 
+// A window sweep; its items one by one while rho is not exactly Hermitian.
+qs_status run_dm_sweep(qs_plan p, const DmSweep& sw, const RunParams& rp) {
+  qs_ctx* h = p->h;
+  if (!h->hermitian) {
+    for (const auto& it : sw.items) {
+      const qs_status st = it.block >= 0 ? run_dm_block(p, p->dm_blocks[it.block], rp)
+                                         : run_single(p, p->gates[it.gate], rp, it.gate);
+      if (st != QS_OK) return st;
+    }
+    return QS_OK;
+  }
+  DmWindowOp ops[kDmWindowOps];
+  int nops = 0;
+  const double q = std::sqrt(std::exp(-rp.e * rp.e));
+  for (const auto& it : sw.items) {
+    if (it.block >= 0) {
+      // a diagonal run joins the channel before it
+      if (nops == 0 || ops[nops - 1].mask) ops[nops++] = DmWindowOp{-1, {}, nullptr, nullptr, 1.0};
+      const DmBlock& b = p->dm_blocks[it.block];
+      DmWindowOp& o = ops[nops - 1];
+      o.u = h->dtype == QS_C64 ? static_cast<const void*>(b.d_uf) : static_cast<const void*>(b.d_u);
+      o.mask = b.d_mask;
+      o.q = q;
+    } else {
+      const qs_gate& g = p->gates[it.gate].g;
+      DmWindowOp o{g.targets[0], {}, nullptr, nullptr, 1.0};
+      dm_real_superop1(g.U, g.noisy, g.noise, rp.e, o.S);
+      ops[nops++] = o;
+    }
+  }
+  const cudaError_t e = launch_dm_window(h, ops, nops);
+  return e == cudaSuccess ? QS_OK : pfail(p, QS_ERR_CUDA, cudaGetErrorString(e));
+}
+
+// Groups consecutive single one-qubit channels with real superoperators and
+// diagonal blocks into window sweeps (up to dm_window_qubits distinct qubits, and
+// the items a sweep holds).
+void group_dm_sweeps(qs_plan p) {
+  if (!dm_window_applicable(p->h)) return;
+  const int most = dm_window_qubits(p->h);
+  std::vector<Step> out;
+  DmSweep cur;
+  uint64_t qubits = 0;
+  auto close = [&]() {
+    if (cur.items.empty()) return;
+    out.push_back(Step{6, -1, (int)p->dm_sweeps.size()});
+    p->dm_sweeps.push_back(cur);
+    cur.items.clear();
+    qubits = 0;
+  };
+  for (const Step& st : p->steps) {
+    const PGate* g = st.kind == 1 ? &p->gates[st.gate] : nullptr;
+    bool real = g && g->g.kind == QS_GATE_DENSE && g->g.k == 1;
+    if (real) for (const auto& v : g->U) real &= v.imag() == 0.0;
+    if (st.kind != 2 && !real) {
+      close();
+      out.push_back(st);
+      continue;
+    }
+    const uint64_t bit = real ? 1ull << g->g.targets[0] : 0;
+    if ((int)cur.items.size() == kDmWindowOps || __builtin_popcountll(qubits | bit) > most) close();
+    cur.items.push_back(st.kind == 2 ? DmSweep::Item{-1, st.gate} : DmSweep::Item{st.gate, -1});
+    qubits |= bit;
+  }
+  close();
+  p->steps.swap(out);
+}
+
 qs_status run_rank_ops(qs_plan p);
 
 qs_status run_step(qs_plan p, const Step& st, const RunParams& rp) {
   if (st.kind == 2) return run_dm_block(p, p->dm_blocks[st.gate], rp);
   if (st.kind == 5) return run_rank_ops(p);
+  if (st.kind == 6) return run_dm_sweep(p, p->dm_sweeps[st.gate], rp);
   return run_single(p, p->gates[st.gate], rp, st.gate);
 }
 
@@ -1813,7 +1889,7 @@ qs_status enqueue_run(qs_plan p, cudaStream_t s, int synth, int fid) {
       if (e != cudaSuccess) { h->stream = saved; return pfail(p, QS_ERR_CUDA, std::string("fused pass: ") + cudaGetErrorString(e)); }
     } else {
       qs_status r = run_step(p, st, *p->h_run);
-      mark(st.kind == 2 ? 4 : 3);
+      mark(st.kind == 6 ? 5 : (st.kind == 2 ? 4 : 3));
       if (r != QS_OK) { h->stream = saved; return r; }
     }
   }
@@ -2164,6 +2240,7 @@ qs_status qs_plan_create(qs_handle h, const qs_gate* gates, int num_gates, qs_pl
     }
     close();
     rem.clear();
+    group_dm_sweeps(p);
   }
   plan_passes(p, rem);
   std::vector<DGate> dg(p->gates.size());
@@ -2226,6 +2303,8 @@ qs_status qs_plan_create(qs_handle h, const qs_gate* gates, int num_gates, qs_pl
   if (st == QS_OK) st = alloc_passes(p);
   if (st == QS_OK && cudaMalloc((void**)&p->d_run, sizeof(RunParams)) != cudaSuccess) st = pfail(p, QS_ERR_OUT_OF_MEMORY, "run params");
   if (st == QS_OK && cudaMallocHost((void**)&p->h_run, sizeof(RunParams)) != cudaSuccess) st = pfail(p, QS_ERR_OUT_OF_MEMORY, "run params");
+  if (st == QS_OK && !p->dm_sweeps.empty() && dm_window_attributes(h) != cudaSuccess)
+    st = pfail(p, QS_ERR_CUDA, "shared memory attribute");
   if (st == QS_OK && set_smem_attrs(h->esize) != cudaSuccess) st = pfail(p, QS_ERR_CUDA, "shared memory attribute");
   if (st != QS_OK) { qs_plan_destroy(p); return st; }
   count_launches(p);
@@ -2314,7 +2393,7 @@ qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t
       } else {
         result = run_step(p, st, *p->h_run);
         cudaEventRecord(ev[k++], h->stream);
-        kind[li++] = st.kind == 2 ? 4 : 3;
+        kind[li++] = st.kind == 6 ? 5 : (st.kind == 2 ? 4 : 3);
         if (result != QS_OK) break;
       }
     }
