@@ -50,7 +50,7 @@ struct FOp {
   uint8_t type;
   uint8_t j;          // local window bit (DENSE, DWIN)
   uint8_t real;       // DENSE: matrix is real
-  uint8_t pad;
+  uint8_t stage;      // register stage it runs in (flips: any)
   uint32_t off;       // parameter offset (R units) in the member block
   uint64_t index;     // FLIP: member-local amplitude index
 };

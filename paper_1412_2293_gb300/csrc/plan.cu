@@ -176,7 +176,18 @@ template <typename R> __device__ __forceinline__ double min_pivot() { return siz
 
 constexpr int kSmallBits = 5;        // table levels the precompute runs for all parts together
 
-// Members' parameters of one pass, one block of 128 threads per member: the
+// What k_precompute builds for one pass.
+struct PreDesc {
+  void* params;                          // R: the members' parameter blocks
+  const Producer* prods;
+  const Contrib* contribs;
+  int stride, num_prods, num_contribs, num_dwin, num_dense, tab_entries, diag_off;
+};
+
+// Members' parameters of the passes of a run, one block of 128 threads per pass
+// and member (pass-major): the blocks of a pass alone are a chain of FP64 and
+// barrier latencies (31 us for 500 members of a Grover pass, 18 times a run), so
+// all passes' are launched together: the
 // noisy matrices of the dense gates in their factored forms, the phase
 // tables, the out factors.  The producer list holds the dense gates, then the
 // tables, then the out terms (the order build_pass writes).  Every draw and
@@ -185,11 +196,15 @@ constexpr int kSmallBits = 5;        // table levels the precompute runs for all
 // one table; warp 0 runs the first (one lane per window bit), warps 1-3 the
 // second (whole tables per warp), with no block barrier between them.
 template <typename R>
-__global__ void __launch_bounds__(128) k_precompute(R* __restrict__ params, int stride, const DGate* __restrict__ gates,
-                                                    const Producer* __restrict__ prods, int num_prods,
-                                                    const Contrib* __restrict__ contribs, int num_contribs,
-                                                    int num_dwin, int num_dense, int tab_entries, int diag_off,
-                                                    NoiseSrc src, const RunParams* rp, int stable, int m) {
+__global__ void __launch_bounds__(128) k_precompute(const PreDesc* __restrict__ descs, int members,
+                                                    const DGate* __restrict__ gates, NoiseSrc src, const RunParams* rp,
+                                                    int stable, int m) {
+  const PreDesc D = descs[blockIdx.x / members];
+  R* __restrict__ params = static_cast<R*>(D.params);
+  const Producer* __restrict__ prods = D.prods;
+  const Contrib* __restrict__ contribs = D.contribs;
+  const int stride = D.stride, num_prods = D.num_prods, num_contribs = D.num_contribs, num_dwin = D.num_dwin,
+            num_dense = D.num_dense, tab_entries = D.tab_entries, diag_off = D.diag_off;
   // shared: [num_contribs] factors, [num_dwin][kMaxWin] partner factors,
   // [tab_entries] FP64 table scratch (a table's parts from its toff), the
   // dense matrices ([num_dense][4] complex), then a copy of the dense and
@@ -202,7 +217,7 @@ __global__ void __launch_bounds__(128) k_precompute(R* __restrict__ params, int 
   Producer* sp = reinterpret_cast<Producer*>(dmat + 4 * (size_t)num_dense);
   const int nsp = num_dense + num_dwin;
   unsigned char* cbit = reinterpret_cast<unsigned char*>(sp + nsp);
-  const int b = blockIdx.x, tid = threadIdx.x;
+  const int b = blockIdx.x % members, tid = threadIdx.x;
   double e;
   uint64_t seed, traj;
   member_noise(src, rp, b, &e, &seed, &traj);
@@ -802,7 +817,9 @@ struct qs_plan_s {
   int64_t graph_wait_polls[kVariants] = {};
   int stable = 0;                 // the running variant: 1 = pivoted real gates
   double* d_fid = nullptr;        // fused-fidelity partials [member][tile] complex
-  void* d_params = nullptr;       // per-member gate parameters of the running pass (shared by the passes)
+  void* d_params = nullptr;       // per-member gate parameters: a block per pass (params_apart), or one they share
+  bool params_apart = false;
+  PreDesc* d_pre = nullptr;       // one per pass
   void* d_alpha = nullptr;        // out factors of the running pass (shared by the passes)
   std::vector<DmBlock> dm_blocks;
   std::vector<DmSweep> dm_sweeps;
@@ -933,6 +950,76 @@ int choose_window(const std::vector<PGate>& G, const std::vector<int>& rem, int 
   return best;
 }
 
+// Reorder a pass's ops so that the register stage changes as rarely as their
+// order allows (an exchange is a write and a read of the whole tile in shared
+// memory): commuting ops of the current stage run first.  A layer of Hadamards, a
+// flip and another layer (two windows' worth of Grover's search) take two
+// exchanges instead of four.  partners: the lower window bits of each phase table;
+// end_stage: the stage the given order ends in.
+void order_stages(PassPlan* P, const std::vector<uint32_t>& partners, int end_stage) {
+  std::vector<FOp> ops;
+  int given = !P->high && end_stage == 1 ? 1 : 0;        // a low pass stores from stage A or C
+  for (const FOp& x : P->ops) {
+    if (x.type == OP_EXCH) ++given;
+    else ops.push_back(x);
+  }
+  const size_t n = ops.size();
+  auto is_flip = [](const FOp& x) { return x.type == OP_FLIP || x.type == OP_FLIPM; };
+  auto commutes = [&](const FOp& a, const FOp& b) {
+    if (a.type != OP_DENSE && b.type != OP_DENSE) return true;
+    if (is_flip(a) || is_flip(b)) return false;
+    if (a.type == OP_DENSE && b.type == OP_DENSE) return a.j != b.j;
+    const FOp &d = a.type == OP_DENSE ? a : b, &w = a.type == OP_DENSE ? b : a;
+    return d.j != w.j && !((partners[w.off] >> d.j) & 1);
+  };
+  std::vector<std::vector<int>> after(n);
+  std::vector<int> before(n, 0);
+  for (size_t i = 0; i < n; ++i)
+    for (size_t k = i + 1; k < n; ++k)
+      if (!commutes(ops[i], ops[k])) { after[i].push_back((int)k); ++before[k]; }
+  const int stages = P->m > kWin ? 3 : 2;
+  std::vector<FOp> best;
+  int best_count = given, best_start = P->start_stage;
+  for (int start = 0; start < (P->high ? stages : 1); ++start) {
+    std::vector<int> left = before;
+    std::vector<char> done(n, 0);
+    std::vector<FOp> out;
+    int stage = start, count = 0;
+    size_t emitted = 0;
+    while (emitted < n) {
+      bool any = true;
+      while (any) {
+        any = false;
+        for (size_t i = 0; i < n; ++i) {
+          if (done[i] || left[i] || (!is_flip(ops[i]) && ops[i].stage != stage)) continue;
+          done[i] = 1;
+          ++emitted;
+          any = true;
+          out.push_back(ops[i]);
+          for (int k : after[i]) --left[k];
+        }
+      }
+      if (emitted == n) break;
+      int ready[3] = {0, 0, 0};
+      for (size_t i = 0; i < n; ++i)
+        if (!done[i] && !left[i]) ++ready[ops[i].stage];
+      int to = 0;
+      for (int s = 1; s < 3; ++s) if (ready[s] > ready[to]) to = s;
+      stage = to;
+      ++count;
+      FOp x{};
+      x.type = OP_EXCH;
+      x.j = (uint8_t)to;
+      out.push_back(x);
+    }
+    if (!P->high && stage == 1) ++count;
+    if (count < best_count) { best_count = count; best = out; best_start = start; }
+  }
+  if (best.empty()) return;
+  P->ops = best;
+  P->start_stage = best_start;
+}
+
 bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n, int colb, uint64_t batch,
                 size_t op_budget, int m, bool split, PassPlan* P, std::vector<char>* absorbed) {
   P->colb = colb;
@@ -1015,6 +1102,7 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
       for (const auto& v : g.U) if (v.imag() != 0.0) real = false;
       if (g.g.noisy && g.g.noise == QS_NOISE_PHASE) real = false;
       x.real = real ? 1 : 0;
+      x.stage = (uint8_t)stage;
       Producer pr{};
       pr.kind = PD_DENSE;
       pr.gate = rem[i];
@@ -1042,6 +1130,7 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
           FOp x{};
           x.type = OP_DWIN;
           x.j = (uint8_t)a;
+          x.stage = (uint8_t)stage;
           x.off = (uint32_t)dwins.size();
           // windows above 10 qubits keep the table as its factors over the
           // thread's bits and the register bits of the stage
@@ -1073,6 +1162,12 @@ bool build_pass(const std::vector<PGate>& G, const std::vector<int>& rem, int n,
     if (!any) return false;
   }
   if (stage == -1) { stage = 0; P->start_stage = 0; }
+  {
+    std::vector<uint32_t> partners(dwins.size(), 0u);
+    for (size_t i = 0; i < dwins.size(); ++i)
+      for (const Contrib& c : dwins[i].cs) partners[i] |= 1u << c.m;
+    order_stages(P, partners, stage);
+  }
 
   // parameter layout: dense matrices, tables, out factors
   std::vector<Producer> prods;
@@ -1435,17 +1530,25 @@ size_t precompute_smem(size_t contribs, size_t dwin, size_t tab_entries, size_t 
          contribs;
 }
 
-// Members' noise draws, matrices, phase tables and out factors of one pass.
+// Members' noise draws, matrices and phase tables -- of every pass with the first
+// one when each has its own parameter block, else of the pass about to run -- and
+// the pass's out factors.
 template <typename R>
 cudaError_t launch_precompute(qs_plan p, const PassPlan& P, const PassMode& mode, cudaStream_t s) {
   qs_ctx* h = p->h;
   NoiseSrc src{};
   if (h->member_noise) { src.e = h->m_e; src.seed = h->m_seed; src.traj = h->m_traj; }
-  const size_t pre_smem = precompute_smem(P.contribs.size(), P.num_dwin, P.tab_entries, P.num_dense);
-  k_precompute<R><<<h->batch, 128, pre_smem, s>>>((R*)P.d_params, P.stride, p->d_gates, P.d_prods,
-                                                   (int)P.prods.size(), P.d_contribs, (int)P.contribs.size(),
-                                                   P.num_dwin, P.num_dense, P.tab_entries, P.diag_off, src,
-                                                   p->d_run, p->stable, P.m);
+  const size_t index = (size_t)(&P - p->passes.data());
+  if (!p->params_apart || index == 0) {
+    const size_t first = p->params_apart ? 0 : index, count = p->params_apart ? p->passes.size() : 1;
+    size_t pre_smem = 0;
+    for (size_t i = first; i < first + count; ++i) {
+      const PassPlan& Q = p->passes[i];
+      pre_smem = std::max(pre_smem, precompute_smem(Q.contribs.size(), Q.num_dwin, Q.tab_entries, Q.num_dense));
+    }
+    k_precompute<R><<<(unsigned)(h->batch * count), 128, pre_smem, s>>>(p->d_pre + first, h->batch, p->d_gates, src,
+                                                                      p->d_run, p->stable, P.m);
+  }
   if (P.d_alpha) {
     OutStarts st{};
     for (int i = 0; i < kMaxWin + 2; ++i) st.v[i] = P.out_start[i];
@@ -2060,7 +2163,7 @@ void plan_passes(qs_plan p, const std::vector<int>& rem) {
 qs_status alloc_passes(qs_plan p) {
   qs_ctx* h = p->h;
   qs_status st = QS_OK;
-  size_t params_bytes = 16, alpha_bytes = 0;
+  size_t params_bytes = 16, params_sum = 0, alpha_bytes = 0;
   for (auto& P : p->passes) {
     if (st != QS_OK) break;
     st = upload(p, &P.d_ops, P.ops);
@@ -2068,7 +2171,9 @@ qs_status alloc_passes(qs_plan p) {
     if (st == QS_OK) st = upload(p, &P.d_prods, P.prods);
     if (st == QS_OK) st = upload(p, &P.d_contribs, P.contribs);
     if (st == QS_OK) {
-      params_bytes = std::max(params_bytes, (size_t)P.stride * h->batch * (h->esize / 2));
+      const size_t bytes = (((size_t)P.stride * h->batch * (h->esize / 2)) + 255) & ~(size_t)255;
+      params_bytes = std::max(params_bytes, bytes);
+      params_sum += bytes;
       // out factors of every tile: members x 2^(n-m) tile values x (m + 1) complex
       if (P.out_start[P.m + 1] > 0)
         alpha_bytes = std::max(alpha_bytes, (((size_t)h->batch * (P.m + 1)) << (h->n - P.m)) * h->esize);
@@ -2079,13 +2184,28 @@ qs_status alloc_passes(qs_plan p) {
   // the most fidelity partials any configuration writes: 2^(n-10) per member
   const size_t fid_slots_max = (size_t)1 << (h->n - kWin);
   if (st == QS_OK && !p->passes.empty()) {
-    if (cudaMalloc(&p->d_params, params_bytes) != cudaSuccess) st = pfail(p, QS_ERR_OUT_OF_MEMORY, "plan params");
+    // a parameter block per pass, computed in one launch, while all of them take
+    // less than 1/64 of the state (or 64 MB)
+    p->params_apart = params_sum <= std::max<size_t>(h->state_elems * h->esize / 64, 64u << 20) &&
+                      (uint64_t)h->batch * p->passes.size() < (1ull << 31);
+    if (p->params_apart && cudaMalloc(&p->d_params, std::max<size_t>(params_sum, 16)) != cudaSuccess) {
+      cudaGetLastError();
+      p->d_params = nullptr;
+      p->params_apart = false;
+    }
+    if (!p->d_params && cudaMalloc(&p->d_params, params_bytes) != cudaSuccess) st = pfail(p, QS_ERR_OUT_OF_MEMORY, "plan params");
     if (st == QS_OK && alpha_bytes && cudaMalloc(&p->d_alpha, alpha_bytes) != cudaSuccess)
       st = pfail(p, QS_ERR_OUT_OF_MEMORY, "plan out factors");
+    size_t at = 0;
+    std::vector<PreDesc> pre;
     for (auto& P : p->passes) {
-      P.d_params = p->d_params;
+      P.d_params = static_cast<char*>(p->d_params) + at;
+      if (p->params_apart) at += (((size_t)P.stride * h->batch * (h->esize / 2)) + 255) & ~(size_t)255;
       P.d_alpha = P.out_start[P.m + 1] > 0 ? p->d_alpha : nullptr;
+      pre.push_back(PreDesc{P.d_params, P.d_prods, P.d_contribs, P.stride, (int)P.prods.size(), (int)P.contribs.size(),
+                            P.num_dwin, P.num_dense, P.tab_entries, P.diag_off});
     }
+    if (st == QS_OK) st = upload(p, &p->d_pre, pre);
   }
   if (st == QS_OK && !p->passes.empty() &&
       cudaMalloc((void**)&p->d_fid, 2 * fid_slots_max * h->batch * sizeof(double)) != cudaSuccess)
@@ -2112,6 +2232,8 @@ void free_passes(qs_plan p) {
   if (p->d_params) cudaFree(p->d_params);
   if (p->d_alpha) cudaFree(p->d_alpha);
   if (p->d_fid) cudaFree(p->d_fid);
+  if (p->d_pre) cudaFree(p->d_pre);
+  p->d_pre = nullptr;
   if (p->d_start_c) cudaFree(p->d_start_c);
   if (p->d_start_v) cudaFree(p->d_start_v);
   p->d_start_c = p->d_start_v = nullptr;
@@ -2127,6 +2249,7 @@ void count_launches(qs_plan p) {
   p->kernels = p->launches;
   for (const Step& s : p->steps)
     if (s.kind == 0 && p->passes[s.pass].d_alpha) ++p->kernels;
+  if (p->params_apart && !p->passes.empty()) p->kernels -= (int)p->passes.size() - 1;   // one precompute
 }
 
 }  // namespace
