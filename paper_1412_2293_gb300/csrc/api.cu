@@ -339,7 +339,8 @@ qs_status read_results(qs_ctx* h, double* out, int count) {
 qs_status materialize_basis(qs_ctx* h) {
   if (!h->pending) return QS_OK;
   const uint64_t* xs = h->pending == 2 ? h->m_basis : nullptr;
-  QS_CUDA(h, launch_set_basis(h, h->state, h->n, h->batch, h->pending_x, xs));
+  if (h->pending == 3) QS_CUDA(h, launch_set_entangled(h, h->state, h->batch, 0));
+  else QS_CUDA(h, launch_set_basis(h, h->state, h->n, h->batch, h->pending_x, xs));
   h->pending = 0;
   return QS_OK;
 }
@@ -494,9 +495,8 @@ qs_status qs_set_basis_state(qs_handle h, uint64_t x) {
 qs_status qs_set_maximally_entangled(qs_handle h) {
   if (!h) return QS_ERR_INVALID_ARG;
   if (h->n % 2) return fail(h, QS_ERR_INVALID_ARG, "the maximally entangled state needs an even qubit count");
-  h->pending = 0;
   if (h->mode == QS_STATEVEC) {
-    QS_CUDA(h, qs::launch_set_entangled(h, h->state, h->batch, 0));
+    h->pending = 3;                       // written by its first consumer
   } else if (h->mode == QS_DENSITY) {
     QS_CUDA(h, qs::launch_set_entangled(h, h->state, 1, 1));
     h->hermitian = true;

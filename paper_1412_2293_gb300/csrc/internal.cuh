@@ -147,7 +147,7 @@ struct qs_ctx {
   bool hermitian = true;                 // DENSITY: the stored matrix is exactly Hermitian
 
   // STATEVEC start state not yet written: 1 = every member |pending_x>,
-  // 2 = member b |m_basis[b]>.  Written by the first consumer (a fused first
+  // 2 = member b |m_basis[b]>, 3 = the maximally entangled state.  Written by the first consumer (a fused first
   // pass creates it in registers instead of reading memory).
   int pending = 0;
   uint64_t pending_x = 0;

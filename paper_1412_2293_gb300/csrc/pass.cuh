@@ -108,6 +108,8 @@ struct PassArgs {
   // values.  synth = kUnit: the start itself, synthesised; kMasked: only the
   // amplitudes whose qubits in `inact` have the start's values are read, straight
   // into registers, the others are taken as zero (whatever memory holds there).
+  // kEntangled: the maximally entangled state of Eq. 16, 2^{-n/4} where the low
+  // half of the index equals the high half.
   // rshift >= 0: only the tiles whose inactive outside bits match the start are
   // run, 2^rshift per member, tile_active = their free bits among the tile index.
   int synth;
@@ -135,7 +137,7 @@ struct PassArgs {
   uint32_t spin_limit;
 };
 
-enum : int { kLoad = 0, kUnit = 1, kMasked = 3 };   // PassArgs::synth
+enum : int { kLoad = 0, kUnit = 1, kEntangled = 2, kMasked = 3 };   // PassArgs::synth
 
 // the low bits of v spread over the set bits of mask
 __device__ __forceinline__ uint64_t deposit(uint64_t v, uint64_t mask) {
@@ -146,6 +148,26 @@ __device__ __forceinline__ uint64_t deposit(uint64_t v, uint64_t mask) {
 }
 __device__ __forceinline__ uint64_t start_index(const PassArgs& A, uint64_t member) {
   return (A.basis ? A.basis[member] : A.basis0[0]) & A.basis_mask;
+}
+
+// The registers r of a thread at member-local index i0 | r << sh, in the maximally
+// entangled state of n qubits.  A thread none of whose registers can match (most
+// of them) stops at one test.
+template <typename R, typename Off>
+__device__ __forceinline__ void entangled_regs(cplx<R> (&a)[kAmps], int n, Off i0, int sh) {
+  const int hm = n >> 1;
+  const uint64_t half = (1ull << hm) - 1, regs = 31ull << sh;
+  const uint64_t amask = (regs | (regs >> hm)) & half;   // bits of the comparison the registers move
+  const uint64_t d0 = ((uint64_t)i0 >> hm ^ (uint64_t)i0) & half;
+#pragma unroll
+  for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
+  if (d0 & ~amask) return;
+  const R amp = (R)sqrt(ldexp(1.0, -hm));
+#pragma unroll
+  for (int r = 0; r < kAmps; ++r) {
+    const uint64_t x = (uint64_t)r << sh;
+    if (((x >> hm ^ x) & half) == d0) a[r].x = amp;
+  }
 }
 
 // First window bit held in registers in stage S of a window of M bits.
@@ -614,7 +636,10 @@ __device__ __forceinline__ int exchange_count(const PassArgs& A, int stage, bool
   return n;
 }
 
-template <typename R, int WARPS, int NBUF, int PROG = 0, int M = kWin>
+// START: the tiles are created or gathered (A.synth != kLoad), never copied; the
+// pass kernels proper do not carry that code (it cost the interpreted high pass
+// 1.5 %).
+template <typename R, int WARPS, int NBUF, int PROG = 0, int M = kWin, bool START = false>
 __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict__ psi, const __grid_constant__ PassArgs A) {
   static_assert(NBUF == 1 || NBUF == 2, "one or two tile buffers");
   static_assert(PROG == 0 || (M == kWin) == ((PROG & kProgWide) == 0), "program kind matches the width");
@@ -643,11 +668,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
     mbar_fence_init();
   }
   group_sync<G>(grp);
-  if (!A.synth && leader && first < last) {
+  if (!START && leader && first < last) {
     mbar_expect_tx(&bars[grp][0], tile_bytes);
     bulk_g2s(wbase, psi + (first << M), tile_bytes, &bars[grp][0]);
   }
-  int in_flight = (!A.synth && first < last) ? 1 : 0;
+  int in_flight = (!START && first < last) ? 1 : 0;
   const int nx = NBUF == 1 ? exchange_count(A, 0, true) : 0;
   uint32_t it = 0;
   for (uint64_t ti = first; ti < last; ti += S::GROUPS, ++it) {
@@ -655,7 +680,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
     const uint32_t parity = NBUF == 2 ? ((it >> 1) & 1) : (it & 1);
     C* cbuf = wbase + cur * S::BUF;
     const uint64_t tn = ti + S::GROUPS;                 // this group's next tile
-    if (NBUF == 2 && !A.synth && leader && tn < last) {
+    if (NBUF == 2 && !START && leader && tn < last) {
       fence_proxy_async();
       mbar_expect_tx(&bars[grp][cur ^ 1], tile_bytes);
       bulk_g2s(wbase + (cur ^ 1) * S::BUF, psi + (tn << M), tile_bytes, &bars[grp][cur ^ 1]);
@@ -664,8 +689,8 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
     // single buffer: start the next tile's copy once this tile's last shared read is done
     int reads_left = nx;
     auto release = [&]() {
-      if constexpr (NBUF == 1) {
-        if (--reads_left == 0 && !A.synth) {
+      if constexpr (NBUF == 1 && !START) {
+        if (--reads_left == 0) {
           fence_proxy_async();
           group_sync<G>(grp);
           if (leader && tn < last) {
@@ -677,7 +702,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
       }
     };
     uint64_t base = ti << M;
-    if (A.rshift >= 0) {
+    if (START && A.rshift >= 0) {
       const uint64_t b = ti >> A.rshift, x = start_index(A, b);
       const uint64_t tl = deposit(ti & ((1ull << A.rshift) - 1), A.tile_active) | ((x >> M) & ~A.tile_active);
       base = (b << A.n) | (tl << M);
@@ -689,25 +714,29 @@ __global__ void __launch_bounds__(WARPS * 32, 1) k_pass_low(cplx<R>* __restrict_
     // read at the end of the tile: into L1 now
     if (A.alpha_tab && wig == 0 && lane < 2) prefetch_l1(static_cast<const C*>(A.alpha_tab) + aidx + lane * 8);
     C a[kAmps];
-    if (A.synth == kMasked) {
-      const uint64_t x = start_index(A, member), i0 = mloc | (uint64_t)t;
-      constexpr int sh = M - kRegBits;
-      const bool own = ((i0 ^ x) & A.inact & ~(31ull << sh)) == 0;
-      const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
-      const C* src = psi + base + t;
-#pragma unroll
-      for (int r = 0; r < kAmps; ++r)
-        a[r] = own && ((r ^ xr) & rmask) == 0 ? src[r << sh] : mk<R>(R(0), R(0));
-    } else if (A.synth) {
-      // the one amplitude equal to 1: register x >> (M-5) & 31 of thread x & (2^(M-5) - 1)
-      const uint64_t x = start_index(A, member);
-#pragma unroll
-      for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
-      if ((x & ~(uint64_t)(S::TILE - 1)) == mloc && (int)(x & ((1u << (M - 5)) - 1)) == t) {
-        const int hr = (int)((x >> (M - 5)) & 31);
+    if constexpr (START) {
+      if (A.synth == kMasked) {
+        const uint64_t x = start_index(A, member), i0 = mloc | (uint64_t)t;
+        constexpr int sh = M - kRegBits;
+        const bool own = ((i0 ^ x) & A.inact & ~(31ull << sh)) == 0;
+        const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
+        const C* src = psi + base + t;
 #pragma unroll
         for (int r = 0; r < kAmps; ++r)
-          if (r == hr) a[r].x = R(1);
+          a[r] = own && ((r ^ xr) & rmask) == 0 ? src[r << sh] : mk<R>(R(0), R(0));
+      } else if (A.synth == kEntangled) {
+        entangled_regs<R>(a, A.n, mloc | (uint64_t)t, M - kRegBits);
+      } else {
+        // the one amplitude equal to 1: register x >> (M-5) & 31 of thread x & (2^(M-5) - 1)
+        const uint64_t x = start_index(A, member);
+#pragma unroll
+        for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
+        if ((x & ~(uint64_t)(S::TILE - 1)) == mloc && (int)(x & ((1u << (M - 5)) - 1)) == t) {
+          const int hr = (int)((x >> (M - 5)) & 31);
+#pragma unroll
+          for (int r = 0; r < kAmps; ++r)
+            if (r == hr) a[r].x = R(1);
+        }
       }
     } else {
       // the group gives up together (a thread that saw the copy land follows
@@ -868,7 +897,7 @@ template <int COLB, int M = kWin> struct HighShape {
   static constexpr int BOXES = (1 << M) / 256;          // tensor-map boxes of 256 rows
 };
 
-template <typename R, int COLB, int NBUF, bool WIDE = false, int PROG = 0, int M = kWin>
+template <typename R, int COLB, int NBUF, bool WIDE = false, int PROG = 0, int M = kWin, bool START = false>
 __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / HighShape<COLB, M>::WARPS : 1)
     k_pass_high(cplx<R>* __restrict__ psi, const __grid_constant__ CUtensorMap tmap, const __grid_constant__ PassArgs A) {
   static_assert(NBUF == 1 || NBUF == 2, "one or two tile buffers");
@@ -913,14 +942,14 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
     for (int b = 0; b < S::BOXES; ++b)
       tma_g2s_2d(dst + b * 256 * S::COLS, &tmap, x, (int)(row0 + b * 256), &bars[which]);
   };
-  if (!A.synth && threadIdx.x == 0 && first < last) issue(first, 0);
-  int in_flight = (!A.synth && first < last) ? 1 : 0;
+  if (!START && threadIdx.x == 0 && first < last) issue(first, 0);
+  int in_flight = (!START && first < last) ? 1 : 0;
   const int nx = NBUF == 1 ? exchange_count(A, A.start_stage, false) : 0;
   uint32_t it = 0;
   for (uint64_t t = first; t < last; ++t, ++it) {
     const int cur = NBUF == 2 ? (int)(it & 1) : 0;
     const uint32_t parity = NBUF == 2 ? ((it >> 1) & 1) : (it & 1);
-    if (NBUF == 2 && !A.synth && threadIdx.x == 0 && t + 1 < last) {
+    if (NBUF == 2 && !START && threadIdx.x == 0 && t + 1 < last) {
       fence_proxy_async();
       issue(t + 1, cur ^ 1);
       ++in_flight;
@@ -928,8 +957,8 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
     // single buffer: start the next tile's copy once this tile's last shared read is done
     int reads_left = nx;
     auto release = [&]() {
-      if constexpr (NBUF == 1) {
-        if (--reads_left == 0 && !A.synth) {
+      if constexpr (NBUF == 1 && !START) {
+        if (--reads_left == 0) {
           fence_proxy_async();
           __syncthreads();
           if (threadIdx.x == 0 && t + 1 < last) {
@@ -941,7 +970,7 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
     };
     uint64_t member = t >> A.tile_shift;
     uint64_t tl = t & ((1ull << A.tile_shift) - 1);
-    if (A.rshift >= 0) {
+    if (START && A.rshift >= 0) {
       member = t >> A.rshift;
       const uint64_t x = start_index(A, member);
       const uint64_t xt = ((x >> (c0 + M)) << cshift) | ((x >> COLB) & cmask);
@@ -963,36 +992,43 @@ __global__ void __launch_bounds__(HighShape<COLB, M>::THREADS, NBUF == 1 ? 16 / 
     }
     C a[kAmps];
     int stage = A.start_stage;
-    if (A.synth == kMasked) {
-      const uint64_t x = start_index(A, member);
-      with_stage<M>(stage, [&](auto SC) {
-        constexpr int SS = decltype(SC)::value;
-        const int sh = c0 + stage_base(M, SS);
-        const Off fixed = tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0);
-        const bool own = (((uint64_t)fixed ^ x) & A.inact & ~(31ull << sh)) == 0;
-        const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
-        const C* src = psi + (member << A.n) + fixed;
-#pragma unroll
-        for (int r = 0; r < kAmps; ++r)
-          a[r] = own && ((r ^ xr) & rmask) == 0 ? src[(Off)r << sh] : mk<R>(R(0), R(0));
-      });
-    } else if (A.synth) {
-      // the one amplitude equal to 1: register (x >> sh) & 31 of the thread
-      // whose other bits match (one thread of the member's whole state)
-      const uint64_t x = start_index(A, member);
-#pragma unroll
-      for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
-      with_stage<M>(stage, [&](auto SC) {
-        constexpr int SS = decltype(SC)::value;
-        const int sh = c0 + stage_base(M, SS);
-        const Off fixed = tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0);
-        if ((x & ~(31ull << sh)) == (uint64_t)fixed) {
-          const int hr = (int)((x >> sh) & 31);
+    if constexpr (START) {
+      if (A.synth == kMasked) {
+        const uint64_t x = start_index(A, member);
+        with_stage<M>(stage, [&](auto SC) {
+          constexpr int SS = decltype(SC)::value;
+          const int sh = c0 + stage_base(M, SS);
+          const Off fixed = tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0);
+          const bool own = (((uint64_t)fixed ^ x) & A.inact & ~(31ull << sh)) == 0;
+          const uint32_t rmask = (uint32_t)(A.inact >> sh) & 31u, xr = (uint32_t)(x >> sh) & 31u;
+          const C* src = psi + (member << A.n) + fixed;
 #pragma unroll
           for (int r = 0; r < kAmps; ++r)
-            if (r == hr) a[r].x = R(1);
-        }
-      });
+            a[r] = own && ((r ^ xr) & rmask) == 0 ? src[(Off)r << sh] : mk<R>(R(0), R(0));
+        });
+      } else if (A.synth == kEntangled) {
+        with_stage<M>(stage, [&](auto SC) {
+          constexpr int SS = decltype(SC)::value;
+          entangled_regs<R>(a, A.n, tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0), c0 + stage_base(M, SS));
+        });
+      } else {
+        // the one amplitude equal to 1: register (x >> sh) & 31 of the thread
+        // whose other bits match (one thread of the member's whole state)
+        const uint64_t x = start_index(A, member);
+#pragma unroll
+        for (int r = 0; r < kAmps; ++r) a[r] = mk<R>(R(0), R(0));
+        with_stage<M>(stage, [&](auto SC) {
+          constexpr int SS = decltype(SC)::value;
+          const int sh = c0 + stage_base(M, SS);
+          const Off fixed = tbits | (Off)col | ((Off)tile_base<M, SS>(tw) << c0);
+          if ((x & ~(31ull << sh)) == (uint64_t)fixed) {
+            const int hr = (int)((x >> sh) & 31);
+#pragma unroll
+            for (int r = 0; r < kAmps; ++r)
+              if (r == hr) a[r].x = R(1);
+          }
+        });
+      }
     } else {
       // the block gives up together, after its copies in flight have landed
       if (__syncthreads_or(!mbar_wait(&bars[cur], parity, A.spin_limit))) {
@@ -1167,6 +1203,14 @@ constexpr int wide_full_prog(int m) {
 cudaError_t launch_pass_wide(cplx<float>* psi, const CUtensorMap& tmap, const PassArgs& A, bool high, int m, int prog,
                              int sms, cudaStream_t s);
 cudaError_t set_wide_attrs();
+// Passes of a run from a start not yet written (A.synth != kLoad; pass_start.cu):
+// one configuration per geometry, tiles of 8 columns (4 in complex128 and m = 12).
+template <typename R>
+cudaError_t launch_pass_start(cplx<R>* psi, const CUtensorMap& tmap, const PassArgs& A, bool high, int m, int prog,
+                              int sms, cudaStream_t s);
+cudaError_t set_start_attrs(size_t esize);
+// the compiled program of the 10-qubit windows: the noisy QFT's
+constexpr int kQftProg = prog_layers(0x1f, 0x1e);
 
 }  // namespace fused
 }  // namespace qs

@@ -22,8 +22,7 @@ cudaError_t launch_m(cplx<float>* psi, const CUtensorMap& tmap, const PassArgs& 
   using H = HighShape<CB, M>;
   constexpr int FULL = wide_full_prog(M);
   if (!high) {
-    const uint64_t blocks = (A.tiles + L::GROUPS - 1) / L::GROUPS;
-    const int grid = (int)(blocks < (uint64_t)sms ? blocks : (uint64_t)sms);
+    const int grid = (int)(A.tiles < (uint64_t)sms ? A.tiles : (uint64_t)sms);
     if (full)
       k_pass_low<float, kWarps, 1, FULL, M><<<grid, L::THREADS, low_smem<float, kWarps, 1, M>(), s>>>(psi, A);
     else

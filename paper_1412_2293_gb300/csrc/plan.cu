@@ -807,9 +807,9 @@ struct qs_plan_s {
   RunParams* d_run = nullptr;
   RunParams* h_run = nullptr;     // pinned
   // captured graphs, one per run variant: start (0 loaded, 1 one basis state,
-  // 2 per-member basis states) x fused fidelity (0, 1)
+  // 2 per-member basis states, 3 maximally entangled) x fused fidelity (0, 1)
   // (x 2: real gates in the two-shear form, or pivoted with a third shear)
-  static constexpr int kVariants = 12;
+  static constexpr int kVariants = 16;
   cudaGraphExec_t exec[kVariants] = {};
   bool graph_member_noise[kVariants] = {};
   bool graph_member_marked[kVariants] = {};
@@ -1438,21 +1438,22 @@ qs_status make_tmap(qs_plan p, PassPlan* P, int colb, CUtensorMap* map) {
   return QS_OK;
 }
 
-// columns per high-window tile of the configuration launched (0 for the low window)
-int launch_colb(qs_plan p, const PassPlan& P) {
+// columns per high-window tile of the configuration launched (0 for the low
+// window); start: the kernels of pass_start.cu, which have one
+int launch_colb(qs_plan p, const PassPlan& P, bool start) {
   if (!P.high) return 0;
   if (P.m != kWin) return wide_colb(P.m);
-  return p->h->esize == 8 && p->high_cfg == 2 ? 2 : P.colb;
+  return p->h->esize == 8 && p->high_cfg == 2 && !start ? 2 : P.colb;
 }
-int launch_tile_shift(qs_plan p, const PassPlan& P) { return p->h->n - P.m - launch_colb(p, P); }
+int launch_tile_shift(qs_plan p, const PassPlan& P, bool start) { return p->h->n - P.m - launch_colb(p, P, start); }
 // fused-fidelity partials per member: one per tile, and per warp of a tile in
 // the low window (2^(m-10) warps)
-int fid_slots(qs_plan p, const PassPlan& P) {
-  return (1 << launch_tile_shift(p, P)) * (P.high ? 1 : 1 << (P.m - kWin));
+int fid_slots(qs_plan p, const PassPlan& P, bool start) {
+  return (1 << launch_tile_shift(p, P, start)) * (P.high ? 1 : 1 << (P.m - kWin));
 }
 
-// How step i of a run executes: from memory, or as part of a run from basis
-// states (synth = 1: one start, 2: per member).
+// How step i of a run executes: from memory, or as part of a run from a start not
+// yet written (synth = 1: one basis state, 2: per member, 3: maximally entangled).
 struct PassMode {
   int synth = 0;                 // the run's start (0: from memory)
   int load = kLoad;              // PassArgs::synth
@@ -1463,6 +1464,10 @@ struct PassMode {
 PassMode pass_mode(qs_plan p, size_t i, int synth) {
   PassMode M;
   if (!synth) return M;
+  if (synth == 3) {              // a dense start: the first pass creates it instead of reading it
+    if (i == 0) { M.synth = synth; M.load = kEntangled; }
+    return M;
+  }
   if (p->start_full < 1) {       // the first pass writes the whole state
     if (i == 0) { M.synth = synth; M.load = kUnit; M.act = 0; }
     return M;
@@ -1496,8 +1501,9 @@ PassArgs pass_args(qs_plan p, const PassPlan& P, const PassMode& mode, int fid) 
   A.params = P.d_params;
   A.marked = h->m_marked;
   const uint64_t total = (uint64_t)h->batch << h->n;
-  A.tile_shift = launch_tile_shift(p, P);
-  A.tiles = total >> (P.m + launch_colb(p, P));
+  const bool start = mode.load != kLoad;
+  A.tile_shift = launch_tile_shift(p, P, start);
+  A.tiles = total >> (P.m + launch_colb(p, P, start));
   A.status = h->dstatus + 2;
   A.synth = mode.load;
   A.rshift = -1;
@@ -1505,7 +1511,7 @@ PassArgs pass_args(qs_plan p, const PassPlan& P, const PassMode& mode, int fid) 
   A.inact = ((1ull << h->n) - 1) & ~mode.act;
   if (mode.restricted) {
     // the tile index: the bits between the columns and the window, then those above it
-    const int cb = launch_colb(p, P), c0 = P.win[0];
+    const int cb = launch_colb(p, P, true), c0 = P.win[0];
     A.tile_active = P.high ? ((mode.act >> cb) & ((1ull << (c0 - cb)) - 1)) | ((mode.act >> (c0 + P.m)) << (c0 - cb))
                            : mode.act >> P.m;
     A.rshift = __builtin_popcountll(A.tile_active);
@@ -1586,25 +1592,28 @@ cudaError_t launch_pass_args(qs_plan p, const PassPlan& P, const PassArgs& A, cp
     const uint64_t cap = (uint64_t)sms * per_sm;
     return (int)(units < cap ? units : cap);
   };
-  constexpr int kQft = prog_layers(0x1f, 0x1e);
+  constexpr int kQft = kQftProg;
+  if (A.synth != kLoad) return launch_pass_start<R>(psi, P.tmap, A, P.high, P.m, prog, sms, s);
   if constexpr (sizeof(R) == 4) {
     // wider windows (n <= 32, checked when the width is set)
     if (P.m != kWin) return launch_pass_wide(psi, P.tmap, A, P.high, P.m, prog, sms, s);
   }
+  // low passes: a block per SM even where its warps then have less than a tile
+  // each (64 members of 13 qubits: 512 tiles on 43 full blocks 10.2 us)
   if (!P.high) {
     if constexpr (sizeof(R) == 4) {
       if (prog == kQft && p->low_cfg == 1)
-        k_pass_low<R, 16, 1, kQft><<<grid((A.tiles + 15) / 16, 1), 16 * 32, low_smem<R, 16, 1>(), s>>>(psi, A);
+        k_pass_low<R, 16, 1, kQft><<<grid(A.tiles, 1), 16 * 32, low_smem<R, 16, 1>(), s>>>(psi, A);
       else if (prog == kQft && p->low_cfg == 2)
-        k_pass_low<R, 12, 1, kQft><<<grid((A.tiles + 11) / 12, 1), 12 * 32, low_smem<R, 12, 1>(), s>>>(psi, A);
+        k_pass_low<R, 12, 1, kQft><<<grid(A.tiles, 1), 12 * 32, low_smem<R, 12, 1>(), s>>>(psi, A);
       else if (p->low_cfg == 1)
-        k_pass_low<R, 16, 1><<<grid((A.tiles + 15) / 16, 1), 16 * 32, low_smem<R, 16, 1>(), s>>>(psi, A);
+        k_pass_low<R, 16, 1><<<grid(A.tiles, 1), 16 * 32, low_smem<R, 16, 1>(), s>>>(psi, A);
       else if (p->low_cfg == 2)
-        k_pass_low<R, 12, 1><<<grid((A.tiles + 11) / 12, 1), 12 * 32, low_smem<R, 12, 1>(), s>>>(psi, A);
+        k_pass_low<R, 12, 1><<<grid(A.tiles, 1), 12 * 32, low_smem<R, 12, 1>(), s>>>(psi, A);
       else
-        k_pass_low<R, 12, 2><<<grid((A.tiles + 11) / 12, 1), 12 * 32, low_smem<R, 12, 2>(), s>>>(psi, A);
+        k_pass_low<R, 12, 2><<<grid(A.tiles, 1), 12 * 32, low_smem<R, 12, 2>(), s>>>(psi, A);
     } else {
-      k_pass_low<R, 4, 2><<<grid((A.tiles + 3) / 4, 1), 4 * 32, low_smem<R, 4, 2>(), s>>>(psi, A);
+      k_pass_low<R, 4, 2><<<grid(A.tiles, 1), 4 * 32, low_smem<R, 4, 2>(), s>>>(psi, A);
     }
   } else {
     constexpr int CB = high_colb<R>();
@@ -1689,7 +1698,7 @@ cudaError_t set_smem_attrs(size_t esize) {
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<float, 3, 1>, high_smem<float, 3, 1>(), 2);
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<float, 2, 1>, high_smem<float, 2, 1>(), 4);
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<float, 3, 2, true>, high_smem<float, 3, 2>(), 1);
-    constexpr int kQft = prog_layers(0x1f, 0x1e);
+    constexpr int kQft = kQftProg;
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_low<float, 16, 1, kQft>, low_smem<float, 16, 1>(), 1);
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_low<float, 12, 1, kQft>, low_smem<float, 12, 1>(), 1);
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<float, 3, 1, false, kQft>, high_smem<float, 3, 1>(), 2);
@@ -1700,6 +1709,7 @@ cudaError_t set_smem_attrs(size_t esize) {
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<double, 2, 2>, high_smem<double, 2, 2>(), 1);
     if (e == cudaSuccess) e = set_pass_attrs(k_pass_high<double, 2, 2, true>, high_smem<double, 2, 2>(), 1);
   }
+  if (e == cudaSuccess) e = set_start_attrs(esize);
   if (e == cudaSuccess) done[which] = true;
   return e;
 }
@@ -1987,7 +1997,7 @@ qs_status enqueue_run(qs_plan p, cudaStream_t s, int synth, int fid) {
       if (e == cudaSuccess) e = f32 ? launch_pass_kernel<float>(p, P, s, mode, fd) : launch_pass_kernel<double>(p, P, s, mode, fd);
       mark(P.high ? 2 : 1);
       if (e == cudaSuccess && fd) {
-        e = launch_finalize(p->d_fid, h->batch, mode.outer ? outer_slots(p, P) : fid_slots(p, P), 0, 1, h->small + kSmallOutIndex, s);
+        e = launch_finalize(p->d_fid, h->batch, mode.outer ? outer_slots(p, P) : fid_slots(p, P, mode.load != kLoad), 0, 1, h->small + kSmallOutIndex, s);
       }
       if (e != cudaSuccess) { h->stream = saved; return pfail(p, QS_ERR_CUDA, std::string("fused pass: ") + cudaGetErrorString(e)); }
     } else {
@@ -2045,7 +2055,7 @@ qs_status run_plan(qs_plan p, double e, uint64_t seed, uint64_t gate_id0, int wa
       return pfail(p, QS_ERR_CUDA, "run params copy");
     st = enqueue_run(p, h->stream, synth, fid);
   } else {
-    const int v = h->mode == QS_FIXED_RANK ? p->rank_variant : p->stable * 6 + synth * 2 + fid;
+    const int v = h->mode == QS_FIXED_RANK ? p->rank_variant : p->stable * 8 + synth * 2 + fid;
     if (p->exec[v] && (p->graph_member_noise[v] != h->member_noise || p->graph_member_marked[v] != h->member_marked ||
                        p->graph_timing[v] != p->timing || p->graph_wait_polls[v] != h->wait_polls ||
                        p->graph_kmax[v] != p->rank_kmax)) {

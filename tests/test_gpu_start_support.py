@@ -133,3 +133,34 @@ def test_run_from_a_basis_start_equals_the_run_from_memory(kind, n, batch, dtype
     # overlaps: 2^n products of a random reference, the same relative bound on the norm product
     np.testing.assert_allclose(f_got, f_want, rtol=0, atol=2 * tol)
     np.testing.assert_allclose(tr, 1.0, atol=2 * tol)
+
+
+@pytest.mark.parametrize("n,batch,dtype,m", [(10, 3, qs.QS_C64, 10), (12, 5, qs.QS_C64, 10), (14, 2, qs.QS_C64, 11),
+                                             (16, 3, qs.QS_C64, 12), (20, 2, qs.QS_C64, 10), (22, 1, qs.QS_C64, 10),
+                                             (12, 2, qs.QS_C128, 10), (16, 2, qs.QS_C128, 10)])
+@pytest.mark.parametrize("kind", ["system", "random"])
+def test_run_from_the_entangled_start_equals_the_run_from_memory(n, batch, dtype, m, kind):
+    rng = np.random.default_rng(n)
+    ops = inputs.qft_circuit(n // 2) if kind == "system" else scattered(n, rng, True)
+    h = qs.qs_create(n, batch, 0, qs.QS_STATEVEC, dtype)
+    try:
+        qs.qs_set_maximally_entangled(h)
+        qs.qs_set_reference_from(h, h, batch - 1)
+        p = qs.qs_plan_create(h, pcirc.to_gates(ops))
+        if m != 10:
+            qs.qs_plan_set_window(p, m)
+        qs.qs_set_state(h, np.full(batch << n, np.nan + 1j * np.nan))      # memory must not matter
+        qs.qs_set_maximally_entangled(h)
+        f_got = qs.qs_plan_run_fidelity(p, 0.05, SEED, 3, h)
+        got = qs.qs_get_state(h)
+        qs.qs_set_maximally_entangled(h)
+        qs.qs_apply_phase_flip(h, 0)                      # writes the start to memory
+        qs.qs_apply_phase_flip(h, 0)
+        f_want = qs.qs_plan_run_fidelity(p, 0.05, SEED, 3, h)
+        want = qs.qs_get_state(h)
+        qs.qs_plan_destroy(p)
+    finally:
+        qs.qs_destroy(h)
+    # created and loaded registers hold the same bits, and the same gates follow
+    np.testing.assert_array_equal(got, want)
+    np.testing.assert_array_equal(f_got, f_want)
