@@ -600,10 +600,14 @@ qs_status qs_apply_noisy_gate(qs_handle h, const int* targets, int k, const doub
     const qs::NoiseSrc src = qs::noise_src(h, e, seed);
     const Targets tg = qs::make_targets(h->n, targets, k);
     const bool diag = noise == QS_NOISE_PHASE && is_diagonal(M, d);
+    uint32_t mask = 1u << (d - 1);
+    if (diag) for (int l = 0; l < d - 1; ++l) if (M[l * d + l] != cd(1.0, 0.0)) mask |= 1u << l;
+    if (qs::noisy_in_one_launch(h, k, diag)) {
+      QS_CUDA(h, qs::launch_apply_noisy(h, tg, U, noise, diag, src, gate_id, mask));
+      return QS_OK;
+    }
     QS_CUDA(h, qs::launch_noise_mats(h, h->mats, h->batch, k, U, noise, diag ? 1 : 0, src, gate_id));
     if (diag) {
-      uint32_t mask = 1u << (d - 1);
-      for (int l = 0; l < d - 1; ++l) if (M[l * d + l] != cd(1.0, 0.0)) mask |= 1u << l;
       QS_CUDA(h, qs::launch_apply_diag(h, h->state, h->n, h->batch, tg, h->mats, true, mask));
     } else if (k == 1) {
       QS_CUDA(h, qs::launch_apply_1q(h, h->state, h->n, h->batch, targets[0], nullptr, h->mats));

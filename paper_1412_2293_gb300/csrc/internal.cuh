@@ -168,6 +168,11 @@ cudaError_t launch_set_basis(qs_ctx* h, void* psi, int n, int members, uint64_t 
                              const uint64_t* xs_dev);
 cudaError_t launch_noise_mats(qs_ctx* h, void* mats, int members, int k, const double* U,
                               int noise, int diag_only, const NoiseSrc& src, uint64_t gate_id);
+// STATEVEC: a noisy gate with its draws in one launch, for small states (k = 1, or a
+// diagonal U under phase noise: mask = the local indices it changes).
+bool noisy_in_one_launch(const qs_ctx* h, int k, bool diag);
+cudaError_t launch_apply_noisy(qs_ctx* h, const Targets& tg, const double* U, int noise, bool diag, const NoiseSrc& src,
+                               uint64_t gate_id, uint32_t mask);
 cudaError_t launch_apply_1q(qs_ctx* h, void* psi, int n, int members, int t,
                             const double* U, const void* mats_dev);
 cudaError_t launch_apply_kq(qs_ctx* h, void* psi, int n, int members, const Targets& tg,

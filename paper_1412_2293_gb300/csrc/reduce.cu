@@ -45,10 +45,40 @@ __device__ __forceinline__ double2 block_sum2(double a, double b) {
   return r;
 }
 
+// Sums of products to more than FP64's input precision on the FP32 pipe: a
+// product of two floats as (rounded, exact remainder), the running sum as
+// (sum, what its roundings lost) -- the compensated dot product of Ogita, Rump
+// and Oishi (SIAM J. Sci. Comput. 26, 2005), as accurate as a 48-bit sum.  A
+// multiply-add takes 10 FP32 instructions; the FP64 one and its two
+// conversions hold a scheduler's FP64 unit for about 64 cycles each on GB300.
+struct Sum2 {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void plus(float p, float e) {   // += p + e
+    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
+    s = t;
+  }
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    plus(p, __fmaf_rn(a, b, -p));
+  }
+  __device__ __forceinline__ void add(float v) { plus(v, 0.f); }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+struct Sum1 {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <typename R> struct SumOf;
+template <> struct SumOf<float> { using T = Sum2; };
+template <> struct SumOf<double> { using T = Sum1; };
+
 // A thread's kPer amplitudes of a full chunk are read as 16-byte vectors
 // (two complex64 amplitudes or one complex128) before any of them is used:
 // the sweep is bound by HBM latency otherwise (one 8-byte load in flight per
-// thread and iteration read 1 GiB of members at 3.3 TB/s; see k_dot_partials).
+// thread and iteration read 1 GiB of members at 3.3 TB/s).
 constexpr int kPer = kChunk / kRBlock;   // 16 amplitudes per thread
 template <typename R> struct Vec;
 template <> struct Vec<float> { using T = float4; static constexpr int N = 2; };
@@ -82,20 +112,29 @@ __device__ __forceinline__ void chunk_each(const cplx<R>* __restrict__ p, const 
 }
 
 // partial[member][chunk] = sum over the chunk of conj(ref_i) psi_i.  Bound by
-// HBM (the members; the reference stays in L2): 64 members of 2^21 complex64
-// amplitudes 328 -> 175 us (6.1 TB/s) with the loads above.
+// HBM (the members; the reference stays in L2) and by the FP64 adds of the block
+// sums (20 warp instructions of 64 cycles a block), so from 20 qubits on a block
+// takes kRounds rounds of 4096 amplitudes, a thread's sums of 16 products added
+// up between rounds with their rounding errors (two floats).  64 members of 2^21
+// complex64 amplitudes: 328 us with neither, 259 with the wide loads, 171 with both
+// (6.3 TB/s).
 template <typename R>
 __global__ void __launch_bounds__(kRBlock) k_dot_partials(const cplx<R>* __restrict__ psi,
                                                           const cplx<R>* __restrict__ ref, int n,
-                                                          int chunks, double* partials) {
+                                                          int chunks, int rounds, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  R re = 0, im = 0;
-  chunk_each<R, true>(psi + (uint64_t)b * N, ref, (uint64_t)c * kChunk, N, [&](cplx<R> a, cplx<R> r) {
-    re += r.x * a.x + r.y * a.y;
-    im += r.x * a.y - r.y * a.x;
-  });
-  const double2 s = block_sum2((double)re, (double)im);
+  typename SumOf<R>::T sre, sim;
+  for (int k = 0; k < rounds; ++k) {
+    R re = 0, im = 0;
+    chunk_each<R, true>(psi + (uint64_t)b * N, ref, ((uint64_t)c * rounds + k) * kChunk, N, [&](cplx<R> a, cplx<R> r) {
+      re += r.x * a.x + r.y * a.y;
+      im += r.x * a.y - r.y * a.x;
+    });
+    sre.add(re);
+    sim.add(im);
+  }
+  const double2 s = block_sum2(sre.value(), sim.value());
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = s.x;
     partials[2 * ((uint64_t)b * chunks + c) + 1] = s.y;
@@ -105,13 +144,17 @@ __global__ void __launch_bounds__(kRBlock) k_dot_partials(const cplx<R>* __restr
 // partial[member][chunk] = sum |psi_i|^2 (stored in the .x slot)
 template <typename R>
 __global__ void __launch_bounds__(kRBlock) k_norm_partials(const cplx<R>* __restrict__ psi, int n,
-                                                           int chunks, double* partials) {
+                                                           int chunks, int rounds, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  R s = 0;
-  chunk_each<R, false>(psi + (uint64_t)b * N, psi, (uint64_t)c * kChunk, N,
-                       [&](cplx<R> a, cplx<R>) { s += a.x * a.x + a.y * a.y; });
-  const double2 t = block_sum2((double)s, 0.0);
+  typename SumOf<R>::T sum;
+  for (int k = 0; k < rounds; ++k) {
+    R s = 0;
+    chunk_each<R, false>(psi + (uint64_t)b * N, psi, ((uint64_t)c * rounds + k) * kChunk, N,
+                         [&](cplx<R> a, cplx<R>) { s += a.x * a.x + a.y * a.y; });
+    sum.add(s);
+  }
+  const double2 t = block_sum2(sum.value(), 0.0);
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = t.x;
     partials[2 * ((uint64_t)b * chunks + c) + 1] = 0.0;
@@ -127,8 +170,8 @@ __global__ void __launch_bounds__(kRBlock) k_norm_partials(const cplx<R>* __rest
 // their sums are added in warp order.  Either order is fixed by the shape.
 // The kernel is a chain of dependent loads, so the wide form is taken when an
 // output has more than 64 partials: one output of 16384 (a 14-qubit density
-// matrix) 247 -> 9 us, 27 of 8192 (fused passes at 23 qubits) 55 -> 6 us; with
-// fewer the narrow form starts fewer blocks and is as fast.
+// matrix) 247 -> 24 us, 40 of 4096 (fused passes at 22 qubits) 30 -> 10 us; with
+// fewer the narrow form starts fewer blocks and is as fast (4 us either way).
 template <int WIDE>
 __global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ partials, int members, int chunks, int mode,
                                                   int group, double* __restrict__ out) {
@@ -212,38 +255,13 @@ __global__ void __launch_bounds__(kRBlock) k_dm_trace_partials(const cplx<R>* rh
   if (threadIdx.x == 0) { partials[2 * blockIdx.x] = t.x; partials[2 * blockIdx.x + 1] = 0.0; }
 }
 
-// Sums of products to more than FP64's input precision on the FP32 pipe: a
-// product of two floats as (rounded, exact remainder), the running sum as
-// (sum, what its roundings lost) -- the compensated dot product of Ogita, Rump
-// and Oishi (SIAM J. Sci. Comput. 26, 2005), as accurate as a 48-bit sum.  A
-// multiply-add takes 10 FP32 instructions; the FP64 one and its two
-// conversions hold a scheduler's FP64 unit for about 64 cycles each on GB300.
-struct Sum2 {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-struct Sum1 {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <typename R> struct SumOf;
-template <> struct SumOf<float> { using T = Sum2; };
-template <> struct SumOf<double> { using T = Sum1; };
-
 // <phi|rho|phi> = sum_i conj(phi_i) sum_j rho[i][j] phi_j, one block per row.
 // HERM (an exactly Hermitian rho): the entries right of the diagonal only,
 // their real part counted twice, 2 Re sum_{i<j}, plus the real diagonal; the
 // part of a row that is summed starts at i, so blocks take rows from both
 // ends in turn.  Bound by the FP64 pipe in complex128, four multiply-adds an
-// entry (14 qubits 2.99 -> 0.95 ms for half the entries), and by HBM in
-// complex64 with Sum2 (13 qubits 1.28 -> 0.06 ms).
+// entry (14 qubits 2.99 -> 0.99 ms for half the entries); in complex64 with Sum2
+// 13 qubits take 0.11 ms (1.28 before; the half read is 0.04 ms of HBM).
 template <typename R, bool HERM>
 __global__ void __launch_bounds__(kRBlock) k_dm_expect_rows(const cplx<R>* __restrict__ rho,
                                                             const cplx<R>* __restrict__ phi, int n,
@@ -294,9 +312,12 @@ bool ensure_partials(qs_ctx* h, size_t doubles) {
   return true;
 }
 
+// rounds of a block (a function of n alone: a member's sum does not depend on the
+// batch; at 20 qubits one member still has 64 blocks) and blocks per member
+int chunk_rounds(int n) { return n >= 20 ? 4 : 1; }
 int chunk_count(int n) {
-  const uint64_t N = 1ull << n;
-  return (int)((N + kChunk - 1) / kChunk);
+  const uint64_t N = 1ull << n, per = (uint64_t)kChunk * chunk_rounds(n);
+  return (int)((N + per - 1) / per);
 }
 
 }  // namespace
@@ -318,9 +339,9 @@ cudaError_t launch_dot(qs_ctx* h, const void* psi, const void* ref, int n, int m
   if (!ensure_partials(h, (size_t)2 * chunks * members)) return cudaErrorMemoryAllocation;
   dim3 grid(chunks, members);
   if (h->dtype == QS_C64)
-    k_dot_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, (const float2*)ref, n, chunks, h->partials);
+    k_dot_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, (const float2*)ref, n, chunks, chunk_rounds(n), h->partials);
   else
-    k_dot_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, (const double2*)ref, n, chunks, h->partials);
+    k_dot_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, (const double2*)ref, n, chunks, chunk_rounds(n), h->partials);
   return launch_finalize(h->partials, members, chunks, 0, group, out, h->stream);
 }
 
@@ -329,9 +350,9 @@ cudaError_t launch_norm(qs_ctx* h, const void* psi, int n, int members, int grou
   if (!ensure_partials(h, (size_t)2 * chunks * members)) return cudaErrorMemoryAllocation;
   dim3 grid(chunks, members);
   if (h->dtype == QS_C64)
-    k_norm_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, n, chunks, h->partials);
+    k_norm_partials<float><<<grid, kRBlock, 0, h->stream>>>((const float2*)psi, n, chunks, chunk_rounds(n), h->partials);
   else
-    k_norm_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, n, chunks, h->partials);
+    k_norm_partials<double><<<grid, kRBlock, 0, h->stream>>>((const double2*)psi, n, chunks, chunk_rounds(n), h->partials);
   return launch_finalize(h->partials, members, chunks, 1, group, out, h->stream);
 }
 
@@ -346,7 +367,7 @@ cudaError_t launch_basis_prob(qs_ctx* h, const void* psi, int n, int members, ui
 }
 
 cudaError_t launch_dm_trace(qs_ctx* h, const void* rho, int n, double* out) {
-  const int chunks = chunk_count(n);
+  const int chunks = (int)(((1ull << n) + kChunk - 1) / kChunk);
   if (!ensure_partials(h, (size_t)2 * chunks)) return cudaErrorMemoryAllocation;
   if (h->dtype == QS_C64)
     k_dm_trace_partials<float><<<chunks, kRBlock, 0, h->stream>>>((const float2*)rho, n, chunks, kChunk, h->partials);

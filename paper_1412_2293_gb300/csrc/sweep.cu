@@ -69,14 +69,10 @@ __global__ void k_set_basis(cplx<R>* psi, int n, int members, uint64_t x, const 
 // 2^k diagonal entries (a diagonal U under phase noise stays diagonal).
 struct DMat { double v[2 * 16]; };
 
+// Member's matrix (2^k x 2^k, or its 2^k diagonal entries) into o.
 template <typename R>
-__global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int diag_only,
-                             NoiseSrc src, uint64_t gate_id) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= members) return;
-  const double e = src.e ? src.e[b] : src.e0;
-  const uint64_t seed = src.seed ? src.seed[b] : src.seed0;
-  const uint64_t traj = src.traj ? src.traj[b] : src.traj0 + (uint64_t)b;
+__device__ __forceinline__ void noise_matrix(R* o, int k, const DMat& U, int noise, int diag_only, double e, uint64_t seed,
+                                             uint64_t traj, uint64_t gate_id) {
   const double2 xi = noise_normals(seed, traj, gate_id);
   const int d = 1 << k;
   if (noise == QS_NOISE_ROTATION) {
@@ -87,7 +83,6 @@ __global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int 
     if (k == 2) sincos(e * xi.y, &sb, &cb);
     const double Va[2][2] = {{ca, sa}, {-sa, ca}};
     const double Vb[2][2] = {{cb, sb}, {-sb, cb}};
-    R* o = out + (size_t)b * 2 * d * d;
     for (int r = 0; r < d; ++r) {
       for (int c = 0; c < d; ++c) {
         double re = 0.0, im = 0.0;
@@ -107,7 +102,6 @@ __global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int 
     sincos(e * xi.x, &s, &c);
     const double pr = c, pi = -s;
     if (diag_only) {
-      R* o = out + (size_t)b * 2 * d;
       for (int r = 0; r < d; ++r) {
         double re = U.v[2 * (r * d + r)], im = U.v[2 * (r * d + r) + 1];
         if (r == d - 1) {
@@ -119,8 +113,7 @@ __global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int 
         o[2 * r + 1] = (R)im;
       }
     } else {
-      R* o = out + (size_t)b * 2 * d * d;
-      for (int r = 0; r < d; ++r) {
+        for (int r = 0; r < d; ++r) {
         for (int cc = 0; cc < d; ++cc) {
           double re = U.v[2 * (r * d + cc)], im = U.v[2 * (r * d + cc) + 1];
           if (cc == d - 1) {
@@ -134,6 +127,17 @@ __global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int 
       }
     }
   }
+}
+
+template <typename R>
+__global__ void k_noise_mats(R* out, int members, int k, DMat U, int noise, int diag_only,
+                             NoiseSrc src, uint64_t gate_id) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= members) return;
+  const double e = src.e ? src.e[b] : src.e0;
+  const uint64_t seed = src.seed ? src.seed[b] : src.seed0;
+  const uint64_t traj = src.traj ? src.traj[b] : src.traj0 + (uint64_t)b;
+  noise_matrix<R>(out + (size_t)b * 2 * (diag_only ? 1 << k : 1 << (2 * k)), k, U, noise, diag_only, e, seed, traj, gate_id);
 }
 
 template <typename R> struct Mat2 { cplx<R> m00, m01, m10, m11; };
@@ -251,6 +255,75 @@ __global__ void __launch_bounds__(kBlock) k_apply_diag(cplx<R>* __restrict__ psi
       }
     }
   }
+}
+
+// A noisy gate (one qubit, or diagonal on one or two) of a small state in one
+// launch: a block draws the noise of its members (one thread each) and then
+// applies the gate to its 256 groups.  The draw is a chain of FP64 latencies, 6 us
+// as a launch of its own for one member, and depends on nothing before it, so the
+// kernel is launched with programmatic stream serialization: it lets the next
+// launch start at once, draws, and only then waits for the launches before it
+// (each of which waited for its own).  55 gates on one member of 10 qubits in
+// complex128, read back: 12.3 us a gate in two launches, 9.5 in one.
+template <typename R, int K, bool DIAG>
+__global__ void __launch_bounds__(kBlock) k_apply_noisy(cplx<R>* __restrict__ psi, int n, uint64_t ngroups, Targets tg,
+                                                        const __grid_constant__ DMat U, int noise, NoiseSrc src,
+                                                        uint64_t gate_id, uint32_t active_mask) {
+  using C = cplx<R>;
+  constexpr int D = 1 << K, E = DIAG ? D : D * D;
+  extern __shared__ __align__(16) unsigned char noisy_sm[];
+  R* mats = reinterpret_cast<R*>(noisy_sm);              // [members of the block][E] complex
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const uint64_t g0 = (uint64_t)blockIdx.x * kBlock;
+  const uint64_t m0 = g0 >> (n - K), members = ((ngroups - 1) >> (n - K)) + 1;
+  const int count = n - K >= 8 ? 1 : kBlock >> (n - K);
+  if ((int)threadIdx.x < count && m0 + threadIdx.x < members) {
+    const uint64_t b = m0 + threadIdx.x;
+    noise_matrix<R>(mats + threadIdx.x * 2 * E, K, U, noise, DIAG ? 1 : 0, src.e ? src.e[b] : src.e0,
+                    src.seed ? src.seed[b] : src.seed0, src.traj ? src.traj[b] : src.traj0 + b, gate_id);
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint64_t g = g0 + threadIdx.x;
+  if (g >= ngroups) return;
+  uint64_t base = g;
+#pragma unroll
+  for (int j = 0; j < K; ++j) base = insert0(base, tg.sorted[j]);
+  const R* m = mats + ((g >> (n - K)) - m0) * 2 * E;
+  if constexpr (DIAG) {
+#pragma unroll
+    for (int l = 0; l < D; ++l)
+      if (active_mask & (1u << l)) psi[base + tg.off[l]] = cmul(mk<R>(m[2 * l], m[2 * l + 1]), psi[base + tg.off[l]]);
+  } else {
+    C a[D];
+#pragma unroll
+    for (int l = 0; l < D; ++l) a[l] = psi[base + tg.off[l]];
+#pragma unroll
+    for (int r = 0; r < D; ++r) {
+      C acc = cmul(mk<R>(m[2 * r * D], m[2 * r * D + 1]), a[0]);
+#pragma unroll
+      for (int c = 1; c < D; ++c) acc = cfma(mk<R>(m[2 * (r * D + c)], m[2 * (r * D + c) + 1]), a[c], acc);
+      psi[base + tg.off[r]] = acc;
+    }
+  }
+}
+
+template <typename R, int K, bool DIAG>
+cudaError_t apply_noisy(qs_ctx* h, int n, uint64_t ng, const Targets& tg, const DMat& U, int noise, const NoiseSrc& src,
+                        uint64_t gate_id, uint32_t mask) {
+  const int count = n - K >= 8 ? 1 : kBlock >> (n - K);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((ng + kBlock - 1) / kBlock));
+  cfg.blockDim = dim3(kBlock);
+  cfg.dynamicSmemBytes = (size_t)count * 2 * (DIAG ? 1 << K : 1 << (2 * K)) * sizeof(R);
+  cfg.stream = h->stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_apply_noisy<R, K, DIAG>, static_cast<cplx<R>*>(h->state), n, ng, tg, U, noise, src,
+                            gate_id, mask);
 }
 
 template <typename R>
@@ -605,6 +678,28 @@ cudaError_t launch_noise_mats(qs_ctx* h, void* mats, int members, int k, const d
   else
     k_noise_mats<double><<<g, 128, 0, h->stream>>>((double*)mats, members, k, m, noise, diag_only, src, gate_id);
   return cudaGetLastError();
+}
+
+// Blocks of the whole state at most for the one-launch form: two per SM, whose
+// draws (about 150 FP64 instructions of one warp) overlap; a grid of 16 blocks an SM
+// would take 20 us for them.
+bool noisy_in_one_launch(const qs_ctx* h, int k, bool diag) {
+  return (k == 1 || diag) && h->n >= k && (((uint64_t)h->batch << (h->n - k)) + kBlock - 1) / kBlock <= (uint64_t)num_sms() * 2;
+}
+
+cudaError_t launch_apply_noisy(qs_ctx* h, const Targets& tg, const double* U, int noise, bool diag, const NoiseSrc& src,
+                               uint64_t gate_id, uint32_t mask) {
+  DMat m{};
+  for (int i = 0; i < 2 << (2 * tg.k); ++i) m.v[i] = U[i];
+  const uint64_t ng = (uint64_t)h->batch << (h->n - tg.k);
+  if (h->dtype == QS_C64) {
+    if (!diag) return apply_noisy<float, 1, false>(h, h->n, ng, tg, m, noise, src, gate_id, mask);
+    return tg.k == 1 ? apply_noisy<float, 1, true>(h, h->n, ng, tg, m, noise, src, gate_id, mask)
+                     : apply_noisy<float, 2, true>(h, h->n, ng, tg, m, noise, src, gate_id, mask);
+  }
+  if (!diag) return apply_noisy<double, 1, false>(h, h->n, ng, tg, m, noise, src, gate_id, mask);
+  return tg.k == 1 ? apply_noisy<double, 1, true>(h, h->n, ng, tg, m, noise, src, gate_id, mask)
+                   : apply_noisy<double, 2, true>(h, h->n, ng, tg, m, noise, src, gate_id, mask);
 }
 
 cudaError_t launch_apply_1q(qs_ctx* h, void* psi, int n, int members, int t, const double* U,
