@@ -47,7 +47,13 @@ constexpr uint32_t kSpinLimit = 1u << 24;
 struct TcArgs {
   float2* psi;
   uint64_t tiles;                       // members * 2^(n - k - 7)
-  uint32_t off_j[32];                   // index offset of local index j (targets in caller order)
+  uint32_t off_j[32];                   // index offset of local index j, targets in ascending order
+  uint8_t perm[32];                     // j in the caller's order of targets (U's)
+  // kRows: the lowest `run_bits + 1` qubits are targets; thread t's s-th 16-byte
+  // vector of a tile sits step_off[s] amplitudes and step_sm[s] operand bytes from its
+  // first
+  int run_bits;
+  uint32_t step_off[16], step_sm[16];
   int pos[12];                          // ascending positions of the tile's k + 7 bits
   int free_pos[kTcFree];                // the 7 free bits, ascending (group index m)
   const float* U;                       // D x D interleaved complex, row-major
@@ -65,9 +71,12 @@ __device__ __forceinline__ uint64_t insert0(uint64_t v, int s) {
 
 // Byte offset of element (row, col) in a K-major operand without swizzle:
 // 8-row x 16-byte core matrices, the row direction fastest (SBO = 128 B),
-// the K direction every rows/8 core matrices (LBO = rows * 16 B).
-__device__ __forceinline__ uint32_t op_byte(int row, int col, int rows) {
-  return (uint32_t)(row * 16 + (col >> 2) * rows * 16 + (col & 3) * 4);
+// the K direction every LBO bytes.  A's LBO is 16 bytes more than its 128 rows
+// take, so that lanes writing one row's columns meet no bank twice (k = 5 on
+// scattered targets 0.45 -> 0.41 ms for 1 GiB, k = 3 0.44 -> 0.39).
+constexpr uint32_t kLboA = kTcRows * 16 + 16;
+__device__ __forceinline__ uint32_t op_byte(int row, int col, uint32_t lbo) {
+  return (uint32_t)(row * 16 + (col & 3) * 4) + (uint32_t)(col >> 2) * lbo;
 }
 
 // Shared-memory matrix descriptor (tcgen05): start, LBO, SBO in 16-byte
@@ -135,12 +144,26 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
-template <int K>
+// MODE: how a tile is read and written.
+//   kPlain  thread m moves row m, one amplitude at a time; the lanes' groups are
+//           neighbours in memory.
+//   kPairs  qubit 0 is a target: local indices 2i and 2i + 1 are neighbours and move
+//           as one 16-byte vector.
+//   kRows   qubits 0..2 (or more) are targets: a row is made of runs of 64 bytes and
+//           more, and lanes that each take a row would be 64 to 256 bytes apart (k =
+//           5 on qubits 0..4, 1 GiB: 1.20 ms with 8-byte accesses, which touched every
+//           sector four times with too little L1 to keep it, 0.76 with 16-byte ones).
+//           The threads take the tile's vectors in the order of memory instead and
+//           write each to its row of A; the results go back the same way through
+//           A's space once the MMAs are done: 0.42 ms, as scattered targets.
+enum : int { kPlain = 0, kPairs = 1, kRows = 2 };
+template <int K, int MODE>
 __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
+  constexpr bool VEC = MODE != kPlain;
   constexpr int D = 1 << K;             // amplitudes per group
   constexpr int KD = 2 * D;             // MMA K (real columns) and N (real rows of B)
   constexpr int kCols = KD < 32 ? 32 : KD;   // tensor-memory columns (power of two >= 32)
-  constexpr uint32_t kABytes = kTcRows * KD * 4;
+  constexpr uint32_t kABytes = KD / 4 * kLboA;
   constexpr uint32_t kBBytes = KD * KD * 4;
   constexpr uint32_t kIdesc = tf32_idesc(kTcRows, KD);
 
@@ -166,10 +189,11 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
   for (int e = tid; e < KD * KD; e += kTcThreads) {
     const int row = e / KD, col = e % KD;          // row 2i + c', column 2j + c
     const int i = row >> 1, cp = row & 1, j = col >> 1, c = col & 1;
-    const float ur = args.U[2 * (i * D + j)], ui = args.U[2 * (i * D + j) + 1];
+    const int at = args.perm[i] * D + args.perm[j];
+    const float ur = args.U[2 * at], ui = args.U[2 * at + 1];
     const float f = cp == 0 ? (c == 0 ? ur : -ui) : (c == 0 ? ui : ur);
     const float hi = tf32_hi(f);
-    const uint32_t b = op_byte(row, col, KD);
+    const uint32_t b = op_byte(row, col, KD * 16);
     *reinterpret_cast<float*>(b_hi + b) = hi;
     *reinterpret_cast<float*>(b_lo + b) = f - hi;
   }
@@ -179,15 +203,20 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
   const uint32_t tmem = tmem_base;
   const uint32_t mbar_a = smem_u32(&mbar);
 
-  // offset of this thread's group inside a tile
+  // offset of this thread's group (kRows: of its first vector) inside a tile, and
+  // that vector's place in A
   uint64_t off_m = 0;
+  const int row0 = MODE == kRows ? tid >> args.run_bits : tid;
+  const int chunk0 = MODE == kRows ? tid & ((1 << args.run_bits) - 1) : 0;
 #pragma unroll
-  for (int b = 0; b < kTcFree; ++b) off_m |= (uint64_t)((tid >> b) & 1) << args.free_pos[b];
+  for (int b = 0; b < kTcFree; ++b) off_m |= (uint64_t)((row0 >> b) & 1) << args.free_pos[b];
+  off_m += 2 * chunk0;
+  const uint32_t sm0 = (uint32_t)row0 * 16 + (uint32_t)chunk0 * kLboA;
 
   auto tile_base = [&](uint64_t t) {
 #pragma unroll
     for (int b = 0; b < K + kTcFree; ++b) t = insert0(t, args.pos[b]);
-    return t | off_m;
+    return t + off_m;                     // (disjoint bits)
   };
   uint32_t phase = 0;
   bool ok = true;
@@ -196,21 +225,26 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
   // two register sets in turn (k <= 4): while one tile is written, multiplied
   // and stored, the next tile's loads land in the other
   float2 xa[D], xb[D];
-  if (t < args.tiles) {
-    const float2* p = args.psi + base;
+  auto load = [&](float2 (&x)[D], const float2* p) {
 #pragma unroll
-    for (int j = 0; j < D; ++j) xa[j] = p[args.off_j[j]];
-  }
+    for (int j = 0; j < D; j += 2) {
+      if constexpr (VEC) {
+        const float4 v = *reinterpret_cast<const float4*>(p + (MODE == kRows ? args.step_off[j / 2] : args.off_j[j]));
+        x[j] = make_float2(v.x, v.y);
+        x[j + 1] = make_float2(v.z, v.w);
+      } else {
+        x[j] = p[args.off_j[j]];
+        x[j + 1] = p[args.off_j[j + 1]];
+      }
+    }
+  };
+  if (t < args.tiles) load(xa, args.psi + base);
   auto process = [&](float2 (&x)[D], float2 (&xn)[D]) -> bool {
     if (t >= args.tiles) return false;
     const uint64_t tn = t + gridDim.x;
     const uint64_t base_n = tile_base(tn);
     auto prefetch = [&]() {
-      if (tn < args.tiles) {
-        const float2* p = args.psi + base_n;
-#pragma unroll
-        for (int j = 0; j < D; ++j) xn[j] = p[args.off_j[j]];
-      }
+      if (tn < args.tiles) load(xn, args.psi + base_n);
     };
     // k <= 4: the next loads go out before this tile's operand writes; k = 5
     // (twice the registers per set) issues them after the MMAs
@@ -220,7 +254,7 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
     for (int j = 0; j < D; j += 2) {
       const float4 v = make_float4(x[j].x, x[j].y, x[j + 1].x, x[j + 1].y);
       const float4 h = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
-      const uint32_t b = op_byte(tid, 2 * j, kTcRows);
+      const uint32_t b = MODE == kRows ? sm0 + args.step_sm[j / 2] : op_byte(tid, 2 * j, kLboA);
       *reinterpret_cast<float4*>(a_hi + b) = h;
       *reinterpret_cast<float4*>(a_lo + b) = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
     }
@@ -229,7 +263,7 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
     if (tid == 0) {
       fence_after();
       const uint32_t ah = smem_u32(a_hi), al = smem_u32(a_lo), bh = smem_u32(b_hi), bl = smem_u32(b_lo);
-      constexpr uint32_t lbo_a = kTcRows * 16, lbo_b = KD * 16;
+      constexpr uint32_t lbo_a = kLboA, lbo_b = KD * 16;
       uint32_t acc = 0;
 #pragma unroll
       for (int s = 0; s < KD / 8; ++s) {          // K = 8 per instruction: two core matrices along K
@@ -258,7 +292,23 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
       tmem_load<kChunk>(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, d);
       tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < kChunk / 2; ++i) q[args.off_j[c0 / 2 + i]] = make_float2(d[2 * i], d[2 * i + 1]);
+      for (int i = 0; i < kChunk / 2; i += 2) {
+        if constexpr (MODE == kRows) {
+          *reinterpret_cast<float4*>(a_hi + op_byte(tid, c0 + 2 * i, kLboA)) =
+              make_float4(d[2 * i], d[2 * i + 1], d[2 * i + 2], d[2 * i + 3]);
+        } else if constexpr (VEC) {
+          *reinterpret_cast<float4*>(q + args.off_j[c0 / 2 + i]) = make_float4(d[2 * i], d[2 * i + 1], d[2 * i + 2], d[2 * i + 3]);
+        } else {
+          q[args.off_j[c0 / 2 + i]] = make_float2(d[2 * i], d[2 * i + 1]);
+          q[args.off_j[c0 / 2 + i + 1]] = make_float2(d[2 * i + 2], d[2 * i + 3]);
+        }
+      }
+    }
+    if constexpr (MODE == kRows) {
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < D; j += 2)
+        *reinterpret_cast<float4*>(q + args.step_off[j / 2]) = *reinterpret_cast<const float4*>(a_hi + sm0 + args.step_sm[j / 2]);
     }
     fence_before();
     __syncthreads();
@@ -285,25 +335,25 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
 
 template <int K>
 constexpr size_t tc_smem_bytes() {
-  return (size_t)2 * kTcRows * (2 << K) * 4 + (size_t)2 * (2 << K) * (2 << K) * 4;
+  return (size_t)2 * ((2 << K) / 4) * kLboA + (size_t)2 * (2 << K) * (2 << K) * 4;
 }
 
-template <int K>
+template <int K, int MODE>
 cudaError_t launch_k(const TcArgs& a, cudaStream_t s) {
   static std::atomic<int> grid_cache{0};
   const size_t smem = tc_smem_bytes<K>();
   int grid = grid_cache.load();
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_tc<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_dense_tc<K, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dense_tc<K>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(k_dense_tc<K, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     // resident CTAs per SM from the kernel's own needs (shared memory with the
     // per-block reserve, registers at warp granularity of 256, threads, and
     // tensor-memory columns so that no CTA waits in tcgen05.alloc)
     cudaFuncAttributes fa{};
-    e = cudaFuncGetAttributes(&fa, k_dense_tc<K>);
+    e = cudaFuncGetAttributes(&fa, k_dense_tc<K, MODE>);
     if (e != cudaSuccess) return e;
     int dev = 0, smem_sm = 0, reserve = 0, regs_sm = 0, threads_sm = 0;
     cudaGetDevice(&dev);
@@ -321,7 +371,7 @@ cudaError_t launch_k(const TcArgs& a, cudaStream_t s) {
     grid_cache.store(grid);
   }
   const uint64_t g = std::min<uint64_t>((uint64_t)grid, a.tiles);
-  k_dense_tc<K><<<(unsigned)g, kTcThreads, smem, s>>>(a);
+  k_dense_tc<K, MODE><<<(unsigned)g, kTcThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -339,10 +389,17 @@ cudaError_t launch_dense_tc(qs_ctx* h, void* psi, int n, int members, const int*
   a.status = h->dstatus + 3;
   uint32_t tmask = 0;
   for (int i = 0; i < k; ++i) tmask |= 1u << targets[i];
+  int order[5];
+  for (int i = 0; i < k; ++i) order[i] = i;
+  std::sort(order, order + k, [&](int x, int y) { return targets[x] < targets[y]; });
   for (int j = 0; j < (1 << k); ++j) {
-    uint32_t o = 0;
-    for (int i = 0; i < k; ++i) o |= (uint32_t)((j >> i) & 1) << targets[i];
+    uint32_t o = 0, c = 0;
+    for (int i = 0; i < k; ++i) {
+      o |= (uint32_t)((j >> i) & 1) << targets[order[i]];
+      c |= (uint32_t)((j >> i) & 1) << order[i];
+    }
     a.off_j[j] = o;
+    a.perm[j] = (uint8_t)c;
   }
   int nf = 0;
   for (int b = 0; b < n && nf < kTcFree; ++b)
@@ -351,10 +408,23 @@ cudaError_t launch_dense_tc(qs_ctx* h, void* psi, int n, int members, const int*
   for (int b = 0; b < n; ++b)
     if ((tmask >> b & 1) || (nf > 0 && b <= a.free_pos[kTcFree - 1] && !(tmask >> b & 1))) a.pos[np++] = b;
   if (np != k + kTcFree) return cudaErrorInvalidValue;
+  int r = 0;                              // consecutive targets from qubit 0 up
+  while (r < k && (tmask >> r & 1)) ++r;
+  if (r >= 3) {
+    const int run = r - 1, rows_per = kTcRows >> run;     // vectors of a run: 2^run; rows of one step
+    a.run_bits = run;
+    for (int s = 0; s < (1 << (k - 1)); ++s) {
+      const int m = (s & ((1 << run) - 1)) * rows_per, hi = s >> run;
+      uint64_t o = 0;
+      for (int b = 0; b < kTcFree; ++b) o |= (uint64_t)((m >> b) & 1) << a.free_pos[b];
+      a.step_off[s] = (uint32_t)o + a.off_j[(2 << run) * hi];
+      a.step_sm[s] = (uint32_t)m * 16 + (uint32_t)(hi << run) * kLboA;
+    }
+  }
   switch (k) {
-    case 3: return launch_k<3>(a, h->stream);
-    case 4: return launch_k<4>(a, h->stream);
-    default: return launch_k<5>(a, h->stream);
+    case 3: return r >= 3 ? launch_k<3, kRows>(a, h->stream) : (r ? launch_k<3, kPairs>(a, h->stream) : launch_k<3, kPlain>(a, h->stream));
+    case 4: return r >= 3 ? launch_k<4, kRows>(a, h->stream) : (r ? launch_k<4, kPairs>(a, h->stream) : launch_k<4, kPlain>(a, h->stream));
+    default: return r >= 3 ? launch_k<5, kRows>(a, h->stream) : (r ? launch_k<5, kPairs>(a, h->stream) : launch_k<5, kPlain>(a, h->stream));
   }
 }
 
