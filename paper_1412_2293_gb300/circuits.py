@@ -22,8 +22,13 @@ def hadamard() -> np.ndarray:
     return _H.copy()
 
 
+_CP = np.eye(4, dtype=np.complex128)
+
+
 def controlled_phase(theta: float) -> np.ndarray:
-    return np.diag([1.0, 1.0, 1.0, np.exp(-1j * theta)]).astype(np.complex128)
+    m = _CP.copy()
+    m[3, 3] = np.exp(-1j * theta)
+    return m
 
 
 def op_gate(op: Op, per_member_flip: bool = False):

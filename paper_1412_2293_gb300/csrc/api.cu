@@ -319,12 +319,32 @@ qs_status read_out(qs_handle h, double* out, int count) { return qs::read_result
 
 }  // namespace
 
+namespace {
+// h->hpinned: results (batch doubles at least one) and the status words, then the
+// members' noise (e, seed, traj, marked), then their basis states
+size_t stage_members(const qs_ctx* h) { return std::max<size_t>((size_t)h->batch, 1); }
+size_t stage_marked(const qs_ctx* h) { return stage_members(h) * (h->mode == QS_FIXED_RANK ? h->rank : 1); }
+size_t stage_noise_at(const qs_ctx* h) { return stage_members(h) + 2; }
+size_t stage_basis_at(const qs_ctx* h) { return stage_noise_at(h) + 3 * stage_members(h) + stage_marked(h); }
+size_t stage_doubles(const qs_ctx* h) { return stage_basis_at(h) + stage_members(h); }
+constexpr size_t kStageMax = 1u << 19;   // doubles (4 MB)
+}  // namespace
+
 namespace qs {
 qs_status read_results(qs_ctx* h, double* out, int count) {
-  QS_CUDA(h, cudaMemcpyAsync(out, h->small + kSmallOut, count * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  QS_CUDA(h, cudaStreamSynchronize(h->stream));
   int status[4] = {0, 0, 0, 0};
-  QS_CUDA(h, cudaMemcpy(status, h->dstatus, sizeof(status), cudaMemcpyDeviceToHost));
+  if (h->hpinned && (size_t)count <= stage_members(h)) {
+    // both copies into pinned memory, one wait
+    QS_CUDA(h, cudaMemcpyAsync(h->hpinned, h->small + kSmallOut, count * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    QS_CUDA(h, cudaMemcpyAsync(h->hpinned + stage_members(h), h->dstatus, sizeof(status), cudaMemcpyDeviceToHost, h->stream));
+    QS_CUDA(h, cudaStreamSynchronize(h->stream));
+    std::memcpy(out, h->hpinned, count * sizeof(double));
+    std::memcpy(status, h->hpinned + stage_members(h), sizeof(status));
+  } else {
+    QS_CUDA(h, cudaMemcpyAsync(out, h->small + kSmallOut, count * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    QS_CUDA(h, cudaStreamSynchronize(h->stream));
+    QS_CUDA(h, cudaMemcpy(status, h->dstatus, sizeof(status), cudaMemcpyDeviceToHost));
+  }
   if (status[2] != 0 || status[3] != 0) {
     // reported once: the words are cleared so the handle's next run starts clean
     QS_CUDA(h, cudaMemset(h->dstatus + 2, 0, 2 * sizeof(int)));
@@ -433,6 +453,14 @@ qs_status qs_create(int n, int batch, int rank, qs_mode mode, qs_dtype dtype, vo
   if (cudaMalloc(&h->mats, h->mats_cap) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
   h->small_cap = kSmallOut + std::max<size_t>((size_t)batch, 64);
   if (cudaMalloc((void**)&h->small, h->small_cap * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
+  if (mode != QS_DENSITY && stage_doubles(h) <= kStageMax) {
+    if (cudaMallocHost((void**)&h->hpinned, stage_doubles(h) * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      h->hpinned = nullptr;
+    }
+    for (auto& ev : h->stage_done)
+      if (h->hpinned && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return bail(QS_ERR_CUDA);
+  }
   if (cudaMalloc((void**)&h->dstatus, 4 * sizeof(int)) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
   if (cudaMemsetAsync(h->dstatus, 0, 4 * sizeof(int), h->stream) != cudaSuccess) return bail(QS_ERR_CUDA);
   h->cols = 1;
@@ -449,10 +477,10 @@ qs_status qs_create(int n, int batch, int rank, qs_mode mode, qs_dtype dtype, vo
 qs_status qs_destroy(qs_handle h) {
   if (!h) return QS_ERR_INVALID_ARG;
   cudaStreamSynchronize(h->stream);
-  void* ptrs[] = {h->state, h->work, h->partials, h->mats, h->small, h->dstatus, h->m_e,
-                  h->m_seed, h->m_traj, h->m_marked, h->ref, h->m_basis, h->rsmall, h->rc.cols, h->rcounters};
+  void* ptrs[] = {h->state, h->work, h->partials, h->mats, h->small, h->dstatus, h->m_e, h->ref, h->m_basis, h->rsmall, h->rc.cols, h->rcounters};
   for (void* p : ptrs) if (p) cudaFree(p);
   if (h->hpinned) cudaFreeHost(h->hpinned);
+  for (auto& ev : h->stage_done) if (ev) cudaEventDestroy(ev);
   delete h;
   return QS_OK;
 }
@@ -513,9 +541,18 @@ qs_status qs_set_basis_states(qs_handle h, const uint64_t* xs) {
     if (xs[b] >= (1ull << h->n)) return fail(h, QS_ERR_INVALID_ARG, "basis index out of range");
   if (h->mode == QS_FIXED_RANK) return rank_set_start(h, 0, 0, xs);
   if (!h->m_basis) QS_CUDA(h, cudaMalloc((void**)&h->m_basis, h->batch * sizeof(uint64_t)));
-  // an earlier run may still read m_basis
-  QS_CUDA(h, cudaStreamSynchronize(h->stream));
-  QS_CUDA(h, cudaMemcpy(h->m_basis, xs, h->batch * sizeof(uint64_t), cudaMemcpyHostToDevice));
+  const size_t bytes = h->batch * sizeof(uint64_t);
+  if (h->hpinned) {
+    // behind any run that still reads m_basis, without waiting for it
+    double* st = h->hpinned + stage_basis_at(h);
+    QS_CUDA(h, cudaEventSynchronize(h->stage_done[1]));
+    std::memcpy(st, xs, bytes);
+    QS_CUDA(h, cudaMemcpyAsync(h->m_basis, st, bytes, cudaMemcpyHostToDevice, h->stream));
+    QS_CUDA(h, cudaEventRecord(h->stage_done[1], h->stream));
+  } else {
+    QS_CUDA(h, cudaStreamSynchronize(h->stream));
+    QS_CUDA(h, cudaMemcpy(h->m_basis, xs, bytes, cudaMemcpyHostToDevice));
+  }
   h->pending = 2;                         // written by its first consumer
   return QS_OK;
 }
@@ -830,7 +867,7 @@ qs_status qs_fidelity_ref(qs_handle h, qs_handle ref, int first, int count, doub
   if (first < 0 || count < 1 || first + count > h->batch) return fail(h, QS_ERR_INVALID_ARG, "member range out of bounds");
   { const qs_status st = qs::materialize_basis(h); if (st != QS_OK) return st; }
   { const qs_status st = qs::materialize_basis(ref); if (st != QS_OK) return fail(h, st, ref->err); }
-  QS_CUDA(h, cudaStreamSynchronize(ref->stream));
+  if (ref->stream != h->stream) QS_CUDA(h, cudaStreamSynchronize(ref->stream));
   // FIXED_RANK: member b's columns, summed (sum_c |<ref|L_{b,c}>|^2)
   const size_t cols = h->mode == QS_FIXED_RANK ? (size_t)h->rank : 1;
   const char* psi = (const char*)h->state + (((size_t)first * cols) << h->n) * h->esize;
@@ -973,30 +1010,33 @@ qs_status qs_set_member_noise(qs_handle h, const double* e, const uint64_t* seed
     if (!(e[b] >= 0.0) || !std::isfinite(e[b])) return fail(h, QS_ERR_INVALID_ARG, "e must be finite and >= 0");
     e_max = std::max(e_max, e[b]);
   }
-  const size_t B = h->batch;
-  if (!h->m_e) QS_CUDA(h, cudaMalloc((void**)&h->m_e, B * sizeof(double)));
-  if (!h->m_seed) QS_CUDA(h, cudaMalloc((void**)&h->m_seed, B * sizeof(uint64_t)));
-  if (!h->m_traj) QS_CUDA(h, cudaMalloc((void**)&h->m_traj, B * sizeof(uint64_t)));
-  QS_CUDA(h, cudaMemcpyAsync(h->m_e, e, B * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-  QS_CUDA(h, cudaMemcpyAsync(h->m_seed, seed, B * sizeof(uint64_t), cudaMemcpyHostToDevice, h->stream));
-  QS_CUDA(h, cudaMemcpyAsync(h->m_traj, traj, B * sizeof(uint64_t), cudaMemcpyHostToDevice, h->stream));
-  h->member_noise = true;
-  h->m_e_max = e_max;
-  if (marked) {
+  if (marked)
     for (int b = 0; b < h->batch; ++b)
       if (marked[b] >= (1ull << h->n)) return fail(h, QS_ERR_INVALID_ARG, "marked index out of range");
-    // FIXED_RANK: one index per column (a member's columns share its index)
-    const size_t per = h->mode == QS_FIXED_RANK ? (size_t)h->rank : 1;
-    std::vector<uint64_t> cols(B * per);
-    for (size_t i = 0; i < cols.size(); ++i) cols[i] = marked[i / per];
-    if (!h->m_marked) QS_CUDA(h, cudaMalloc((void**)&h->m_marked, cols.size() * sizeof(uint64_t)));
-    QS_CUDA(h, cudaMemcpyAsync(h->m_marked, cols.data(), cols.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, h->stream));
-    h->member_marked = true;
-  } else {
-    h->member_marked = false;
+  const size_t B = h->batch, cols = stage_marked(h), per = cols / B;
+  if (!h->m_e) {
+    QS_CUDA(h, cudaMalloc((void**)&h->m_e, (3 * B + cols) * sizeof(double)));
+    h->m_seed = reinterpret_cast<uint64_t*>(h->m_e + B);
+    h->m_traj = h->m_seed + B;
+    h->m_marked = h->m_traj + B;
   }
-  // the host arrays are consumed by the time the stream reaches the copies
-  QS_CUDA(h, cudaStreamSynchronize(h->stream));
+  // one copy of the block, from pinned memory where there is some (the caller's
+  // arrays are consumed either way when the call returns)
+  std::vector<double> pageable;
+  double* st = h->hpinned ? h->hpinned + stage_noise_at(h) : nullptr;
+  if (st) QS_CUDA(h, cudaEventSynchronize(h->stage_done[0]));
+  else { pageable.resize(3 * B + cols); st = pageable.data(); }
+  std::memcpy(st, e, B * sizeof(double));
+  std::memcpy(st + B, seed, B * sizeof(uint64_t));
+  std::memcpy(st + 2 * B, traj, B * sizeof(uint64_t));
+  // FIXED_RANK: one index per column (a member's columns share its index)
+  if (marked) for (size_t i = 0; i < cols; ++i) std::memcpy(st + 3 * B + i, marked + i / per, sizeof(uint64_t));
+  QS_CUDA(h, cudaMemcpyAsync(h->m_e, st, (3 * B + (marked ? cols : 0)) * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  if (h->hpinned) QS_CUDA(h, cudaEventRecord(h->stage_done[0], h->stream));
+  else QS_CUDA(h, cudaStreamSynchronize(h->stream));
+  h->member_noise = true;
+  h->m_e_max = e_max;
+  h->member_marked = marked != nullptr;
   return QS_OK;
 }
 

@@ -126,12 +126,15 @@ struct qs_ctx {
   double* small = nullptr;               // Gram matrix, eigenvectors, results
   size_t small_cap = 0;                  // doubles
   int* dstatus = nullptr;                // device status words
-  double* hpinned = nullptr;             // pinned host staging for results
-  size_t hpinned_cap = 0;
+  // pinned host staging (null for very large batches: pageable copies then):
+  // results and status words, the members' noise, their basis states; an upload's
+  // block is written again only after its event
+  double* hpinned = nullptr;
+  cudaEvent_t stage_done[2] = {nullptr, nullptr};   // noise, basis states
 
   // per-member noise (continuous batching)
   uint64_t traj_offset = 0;
-  double* m_e = nullptr;
+  double* m_e = nullptr;                 // one block: e, seed, traj, marked
   uint64_t* m_seed = nullptr;
   uint64_t* m_traj = nullptr;
   uint64_t* m_marked = nullptr;

@@ -37,10 +37,11 @@ class qs_gate(ct.Structure):
 
 
 _lib = None
+# Array arguments are declared as plain addresses: an address (or None, or any
+# ctypes pointer or array) converts faster than numpy's pointer objects are made,
+# a fifth of a small gate call's time.
 _P = ct.c_void_p
-_D = ct.POINTER(ct.c_double)
-_U64 = ct.POINTER(ct.c_uint64)
-_I = ct.POINTER(ct.c_int)
+_D = _U64 = _I = ct.c_void_p
 
 _SIGS = {
     "qs_version": ([], ct.c_char_p),
@@ -94,7 +95,7 @@ _SIGS = {
     "qs_plan_get_window": ([_P, _I], ct.c_int),
     "qs_fidelity_noalloc": ([_P, _P, ct.c_int, ct.c_int, ct.c_int, _P, _D], ct.c_int),
     "qs_measure_peaks": ([_D, _D], ct.c_int),
-    "qs_debug_noise": ([ct.c_uint64, ct.c_uint64, ct.c_uint64, ct.c_int, ct.POINTER(ct.c_uint32), _D], ct.c_int),
+    "qs_debug_noise": ([ct.c_uint64, ct.c_uint64, ct.c_uint64, ct.c_int, _P, _D], ct.c_int),
 }
 
 
@@ -120,12 +121,14 @@ def _check(status, h=None):
 
 
 def _dptr(a):
-    return a.ctypes.data_as(_D)
+    return a.__array_interface__["data"][0]
 
 
 def _cplx_interleaved(M):
-    M = np.ascontiguousarray(np.asarray(M, dtype=np.complex128))
-    return np.ascontiguousarray(M.view(np.float64).reshape(-1))
+    """M's entries in order as interleaved doubles (its own memory where it already is that)."""
+    if type(M) is not np.ndarray or M.dtype != np.complex128 or not M.flags.c_contiguous or not M.ndim:
+        M = np.ascontiguousarray(np.asarray(M, dtype=np.complex128))
+    return M.reshape(-1).view(np.float64)
 
 
 def _targets(t):
@@ -169,7 +172,7 @@ def qs_set_basis_state(h, x):
 
 def qs_set_basis_states(h, xs):
     a = np.ascontiguousarray(np.asarray(xs, dtype=np.uint64))
-    _check(lib().qs_set_basis_states(h, a.ctypes.data_as(_U64)), h)
+    _check(lib().qs_set_basis_states(h, _dptr(a)), h)
 
 
 def qs_set_maximally_entangled(h):
@@ -304,12 +307,12 @@ def qs_set_rank_columns(h, m):
 
 def qs_set_member_ranks(h, ranks):
     r = np.ascontiguousarray(np.asarray(ranks, dtype=np.int32))
-    _check(lib().qs_set_member_ranks(h, r.ctypes.data_as(_I)), h)
+    _check(lib().qs_set_member_ranks(h, _dptr(r)), h)
 
 
 def qs_get_member_columns(h):
     out = np.zeros(qs_info(h)["batch"], dtype=np.int32)
-    _check(lib().qs_get_member_columns(h, out.ctypes.data_as(_I)), h)
+    _check(lib().qs_get_member_columns(h, _dptr(out)), h)
     return out
 
 
@@ -327,8 +330,8 @@ def qs_set_member_noise(h, e=None, seed=None, traj=None, marked=None):
     ea = None if e is None else np.ascontiguousarray(np.asarray(e, dtype=np.float64))
     sa, ta, ma = u64(seed), u64(traj), u64(marked)
     _check(lib().qs_set_member_noise(
-        h, None if ea is None else _dptr(ea), None if sa is None else sa.ctypes.data_as(_U64),
-        None if ta is None else ta.ctypes.data_as(_U64), None if ma is None else ma.ctypes.data_as(_U64)), h)
+        h, None if ea is None else _dptr(ea), None if sa is None else _dptr(sa),
+        None if ta is None else _dptr(ta), None if ma is None else _dptr(ma)), h)
 
 
 def make_gate(targets=(), U=None, noisy=False, noise=QS_NOISE_ROTATION, kind=QS_GATE_DENSE, index=0):
@@ -381,7 +384,7 @@ def qs_plan_profile(p, reps, e, seed, gate_id0=0, cap=4096, h=None):
     kinds = np.zeros(cap, dtype=np.int32)
     count = ct.c_int()
     _check(lib().qs_plan_profile(p, int(reps), float(e), int(seed), int(gate_id0), _dptr(ms),
-                                 kinds.ctypes.data_as(_I), cap, ct.byref(count)), h)
+                                 _dptr(kinds), cap, ct.byref(count)), h)
     c = min(count.value, cap)
     return ms[:c].copy(), [PROFILE_KINDS[int(k)] for k in kinds[:c]]
 
@@ -429,7 +432,7 @@ def qs_plan_last_times(p, cap=4096, h=None):
     ms = np.zeros(cap, dtype=np.float64)
     kinds = np.zeros(cap, dtype=np.int32)
     count = ct.c_int()
-    _check(lib().qs_plan_last_times(p, _dptr(ms), kinds.ctypes.data_as(_I), cap, ct.byref(count)), h)
+    _check(lib().qs_plan_last_times(p, _dptr(ms), _dptr(kinds), cap, ct.byref(count)), h)
     c = min(count.value, cap)
     return ms[:c].copy(), [PROFILE_KINDS[int(k)] for k in kinds[:c]]
 
@@ -467,5 +470,5 @@ def qs_debug_noise(seed, traj, gate_id, count):
     words = np.zeros(4 * count, dtype=np.uint32)
     normals = np.zeros(2 * count, dtype=np.float64)
     _check(lib().qs_debug_noise(int(seed), int(traj), int(gate_id), int(count),
-                                words.ctypes.data_as(ct.POINTER(ct.c_uint32)), _dptr(normals)))
+                                _dptr(words), _dptr(normals)))
     return words.reshape(count, 4), normals.reshape(count, 2)
