@@ -453,7 +453,7 @@ qs_status qs_create(int n, int batch, int rank, qs_mode mode, qs_dtype dtype, vo
   if (cudaMalloc(&h->mats, h->mats_cap) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
   h->small_cap = kSmallOut + std::max<size_t>((size_t)batch, 64);
   if (cudaMalloc((void**)&h->small, h->small_cap * sizeof(double)) != cudaSuccess) { cudaGetLastError(); return bail(QS_ERR_OUT_OF_MEMORY); }
-  if (mode != QS_DENSITY && stage_doubles(h) <= kStageMax) {
+  if (stage_doubles(h) <= kStageMax) {
     if (cudaMallocHost((void**)&h->hpinned, stage_doubles(h) * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       h->hpinned = nullptr;
