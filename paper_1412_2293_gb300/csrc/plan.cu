@@ -174,6 +174,19 @@ __device__ __forceinline__ void noisy_matrix(const DGate& g, double e, uint64_t 
 // entry, far below the precision of R (intermediate values stay in range).
 template <typename R> __device__ __forceinline__ double min_pivot() { return sizeof(R) == 4 ? 0x1p-30 : 0x1p-300; }
 
+// 1 / x for the factors of complex64 runs, which are rounded to FP32: the FP32
+// reciprocal and one third-order step, y (1 + err + err^2) with err = 1 - x y of
+// about 2^-22, in three FP64 instructions and two conversions.  An FP64 division is
+// about a dozen, and one warp's FP64 instruction holds its scheduler for 64
+// cycles: with four divisions a gate and a square root the factoring bound the
+// launch (serving Grover, 17 passes x 500 members: 364 -> 285 us).  |x| >= 2^-30
+// (min_pivot), so the seed is a normal number.
+__device__ __forceinline__ double recip64(double x) {
+  const double y = __frcp_rn((float)x);
+  const double err = fma(-x, y, 1.0);
+  return fma(y, fma(err, err, err), y);
+}
+
 constexpr int kSmallBits = 5;        // table levels the precompute runs for all parts together
 
 // What k_precompute builds for one pass.
@@ -294,23 +307,42 @@ __global__ void __launch_bounds__(128) k_precompute(const PreDesc* __restrict__ 
         const double2* slot = dmat + p.contrib_start * 4;
         if (p.real) {
           const double mp = min_pivot<R>();
-          auto clamp = [mp](double x) { return fabs(x) < mp ? (x < 0.0 ? -mp : mp) : x; };
+          const long long mpb = __double_as_longlong(mp);
+          auto clamp = [mp, mpb](double x) {            // compared as bits, off the FP64 pipe
+            const long long b = __double_as_longlong(x), a = b & 0x7fffffffffffffffll;
+            return a < mpb ? (b < 0 && a != 0 ? -mp : mp) : x;
+          };
           const double a = slot[0].x, bb = slot[0].y * rho, c = slot[1].x, d = slot[1].y * rho;
           const double det = a * d - bb * c;
           double fp, fq, fw, d0, d1;
-          if (!stable || fabs(a) >= 0.25 * sqrt(a * a + c * c)) {
-            d0 = clamp(a);
-            d1 = clamp(det / d0);
-            fp = bb / d0;
-            fq = c / d1;
-            fw = 0.0;
+          const bool first = !stable || 15.0 * (a * a) >= c * c;      // |a| >= |(a, c)| / 4
+          double rho_next;
+          if constexpr (sizeof(R) == 4) {
+            // the pivot x and y = det' / x
+            const double x = clamp(first ? a : c), rx = recip64(x);
+            const double y = clamp(det * rx), ry = recip64(y);
+            fp = first ? bb * rx : fma(d, rx, -1.0);
+            fq = first ? c * ry : 1.0;
+            fw = first ? 0.0 : fma(a, ry, -1.0);
+            d0 = first ? x : y;
+            d1 = first ? y : x;
+            rho_next = first ? y * rx : x * ry;
           } else {
-            d1 = clamp(c);
-            const double dt = clamp(det);
-            fp = d / d1 - 1.0;
-            d0 = dt / d1;
-            fq = 1.0;
-            fw = a * d1 / dt - 1.0;
+            if (first) {
+              d0 = clamp(a);
+              d1 = clamp(det / d0);
+              fp = bb / d0;
+              fq = c / d1;
+              fw = 0.0;
+            } else {
+              d1 = clamp(c);
+              const double dt = clamp(det);
+              fp = d / d1 - 1.0;
+              d0 = dt / d1;
+              fq = 1.0;
+              fw = a * d1 / dt - 1.0;
+            }
+            rho_next = d1 / d0;
           }
           out[p.off] = (R)fp;                           // (p, p, q, q, w, w)
           out[p.off + 1] = (R)fp;
@@ -319,7 +351,7 @@ __global__ void __launch_bounds__(128) k_precompute(const PreDesc* __restrict__ 
           out[p.off + 4] = (R)fw;
           out[p.off + 5] = (R)fw;
           pa *= d0;
-          rho = d1 / d0;
+          rho = rho_next;
         } else {
           const double pd = rho * pa;
           for (int q = 0; q < 4; ++q) {
