@@ -246,14 +246,12 @@ void advance_counts(qs_handle h, int K, int trunc_r, int* max_M, int* max_keep) 
   h->cols = *std::max_element(h->m_cols.begin(), h->m_cols.end());
 }
 
-// FIXED_RANK: L'_b = [E_1 L_b | ..], then truncation when K > 1.  ks: one
-// Kraus set for every member, or (per_member) `batch` sets of K operators.
-qs_status rank_apply_kraus(qs_handle h, const int* targets, int k, const std::vector<std::vector<cd>>& ks,
-                           int per_member = 0) {
+// FIXED_RANK: L'_b = [E_1 L_b | ..], then truncation when K > 1.
+qs_status rank_apply_kraus(qs_handle h, const int* targets, int k, const std::vector<std::vector<cd>>& ks) {
   const int d = 1 << k;
-  const int K = per_member ? (int)ks.size() / h->batch : (int)ks.size();
+  const int K = (int)ks.size();
   for (const auto& E : ks) if (!all_real(E)) h->real_factor = false;
-  if (K == 1 && !per_member) return apply_uniform(h, h->state, h->n, rank_swept(h), targets, k, ks[0]);
+  if (K == 1) return apply_uniform(h, h->state, h->n, rank_swept(h), targets, k, ks[0]);
   int max_cols = 0;
   for (int b = 0; b < h->batch; ++b) {
     if (K * h->m_cols[b] > std::min(qs::kMaxGramDim, h->mcap))
@@ -264,19 +262,13 @@ qs_status rank_apply_kraus(qs_handle h, const int* targets, int k, const std::ve
   for (const auto& E : ks) { auto v = to_interleaved(E); e.insert(e.end(), v.begin(), v.end()); }
   const size_t set_bytes = (size_t)K * d * d * 2 * sizeof(double);
   double* Edev = h->rsmall + qs::kSmallE;
-  if (per_member) {
-    QS_CUDA(h, cudaMemcpy2DAsync(Edev, qs::kRankStride * sizeof(double), e.data(), set_bytes, set_bytes, h->batch,
-                                 cudaMemcpyHostToDevice, h->stream));
-  } else {
-    QS_CUDA(h, cudaMemcpyAsync(Edev, e.data(), set_bytes, cudaMemcpyHostToDevice, h->stream));
-  }
+  QS_CUDA(h, cudaMemcpyAsync(Edev, e.data(), set_bytes, cudaMemcpyHostToDevice, h->stream));
   const Targets tg = qs::make_targets(h->n, targets, k);
   bool diag = true;
   for (const auto& E : ks) diag &= is_diagonal(E, d);
   int max_M, max_keep;
   advance_counts(h, K, 0, &max_M, &max_keep);
-  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, Edev, K, per_member ? qs::kRankStride : 0,
-                                     qs::KrausGate{}, max_cols, max_keep, h->normalize));
+  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, Edev, K, 0, qs::KrausGate{}, max_cols, max_keep, h->normalize));
   return QS_OK;
 }
 

@@ -241,23 +241,18 @@ cudaError_t launch_finalize(const double* partials, int members, int chunks, int
                             cudaStream_t s);
 cudaError_t launch_convert_ref(qs_ctx* h, const double* src_dev, void* dst, size_t count);
 
-// fixed rank, every member of the handle (counts in h->rc): expansion of the
-// factors into L' with K Kraus operators (member b's at E + b e_stride,
-// e_stride = 0: shared), FP64 Gram matrices, eigensolver and truncation (to
-// the members' ranks, or to trunc_r > 0), projection back into the factors.
-// max_* are the largest counts over the members (launch sizes).
-cudaError_t launch_kraus_expand(qs_ctx* h, const Targets& tg, bool real, const double* E_dev, int K, int e_stride,
-                                int max_cols);
-// the same with the Kraus set of a noisy gate built on the device per member
-cudaError_t launch_kraus_expand_gate(qs_ctx* h, const Targets& tg, bool real, const KrausGate& g, int max_cols);
+// fixed rank, every member of the handle (counts in h->rc): FP64 Gram matrices of
+// L', eigensolver and truncation (to the members' ranks, or to trunc_r > 0),
+// projection back into the factors.  max_* are the largest counts over the
+// members (launch sizes).
 // Kraus operators of a noisy gate's averaged channel (2 for k = 1 or phase
 // noise, 4 for k = 2 rotation noise)
 inline int kraus_count(int k, int noise) { return noise == QS_NOISE_ROTATION && k == 2 ? 4 : 2; }
 cudaError_t launch_gram(qs_ctx* h, bool real, int max_M);
 cudaError_t launch_eig_truncate(qs_ctx* h, int trunc_r, int normalize);
 cudaError_t launch_project(qs_ctx* h, bool real, int K, int max_keep);
-// A whole channel (Kraus operators E as above, or g's averaged set when g.k >
-// 0) with truncation to the members' ranks.  diag: every operator is diagonal.
+// A whole channel (K Kraus operators, member b's at E + b e_stride, e_stride = 0:
+// shared; or g's averaged set when g.k > 0) with truncation to the members' ranks.  diag: every operator is diagonal.
 // One-qubit and diagonal channels never form L' (k_moments, k_project_fused).
 cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool diag, const double* E_dev, int K,
                                 int e_stride, const KrausGate& g, int max_cols, int max_keep, int normalize);

@@ -41,10 +41,6 @@ __device__ __forceinline__ uint64_t insert0(uint64_t v, int s) {
   return ((v >> s) << (s + 1)) | (v & ((1ull << s) - 1));
 }
 
-// Lp_b[a m_b + c] = E_a L_b[c] for member b = blockIdx.y; one thread per
-// (group, column).  The member's Kraus operators are E + b e_stride (e_stride
-// = 0: one set for every member).  Block (0, b) records M_b = K m_b.  REAL: L
-// and the E_a are real (imaginary parts zero), real arithmetic.
 // Entry (row, col) of operator `op` of the xi-averaged Kraus set of a noisy
 // gate U (Eqs. 5-6 and 8-9) at noise level e: rotation noise -> U N with N
 // the tensor product over the targets (target 0 the low local bit) of
@@ -79,13 +75,17 @@ __device__ double2 kraus_entry(const KrausGate& g, double e, int op, int row, in
   return make_double2(re, im);
 }
 
-template <typename R, int K_Q, bool REAL, bool DIAG = false>
+// Lp_b[a m_b + c] = E_a L_b[c] for member b = blockIdx.y; one thread per
+// (group, column) of a two-qubit channel.  The member's Kraus operators are E + b e_stride (e_stride
+// = 0: one set for every member).  Block (0, b) records M_b = K m_b.  REAL: L
+// and the E_a are real (imaginary parts zero), real arithmetic.
+template <typename R, bool REAL>
 __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __restrict__ L,
                                                             cplx<R>* __restrict__ Lp, int n, int rcap, int mcap,
                                                             Targets tg, const double* __restrict__ E, int K,
                                                             int e_stride, RankCounts rc, const KrausGate g) {
   using C = cplx<R>;
-  constexpr int D = 1 << K_Q;
+  constexpr int D = 4;
   __shared__ C sE[8 * D * D];
   const int b = blockIdx.y;
   if (g.k > 0) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __res
   if (blockIdx.x == 0 && threadIdx.x == 0) rc.M[b] = K * m;
   __syncthreads();
   const uint64_t N = 1ull << n;
-  const uint64_t groups = N >> K_Q;
+  const uint64_t groups = N >> 2;
   const uint64_t total = groups * (uint64_t)m;
   const C* Lb = L + (uint64_t)b * rcap * N;
   C* Lpb = Lp + (uint64_t)b * mcap * N;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __res
     const uint64_t g = w - (uint64_t)c * groups;
     uint64_t base = g;
 #pragma unroll
-    for (int j = 0; j < K_Q; ++j) base = insert0(base, tg.sorted[j]);
+    for (int j = 0; j < 2; ++j) base = insert0(base, tg.sorted[j]);
     if constexpr (REAL) {
       R v[D];
 #pragma unroll
@@ -123,12 +123,8 @@ __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __res
 #pragma unroll
         for (int r = 0; r < D; ++r) {
           R acc = R(0);
-          if constexpr (DIAG) {
-            acc = sE[(a * D + r) * D + r].x * v[r];
-          } else {
 #pragma unroll
-            for (int q = 0; q < D; ++q) acc = fma(sE[(a * D + r) * D + q].x, v[q], acc);
-          }
+          for (int q = 0; q < D; ++q) acc = fma(sE[(a * D + r) * D + q].x, v[q], acc);
           out[tg.off[r]] = mk<R>(acc, R(0));
         }
       }
@@ -141,12 +137,8 @@ __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __res
 #pragma unroll
         for (int r = 0; r < D; ++r) {
           C acc = mk<R>(R(0), R(0));
-          if constexpr (DIAG) {
-            acc = cmul(sE[(a * D + r) * D + r], v[r]);
-          } else {
 #pragma unroll
-            for (int q = 0; q < D; ++q) acc = cfma(sE[(a * D + r) * D + q], v[q], acc);
-          }
+          for (int q = 0; q < D; ++q) acc = cfma(sE[(a * D + r) * D + q], v[q], acc);
           out[tg.off[r]] = acc;
         }
       }
@@ -340,7 +332,6 @@ template <> __device__ __forceinline__ double tscal<double>(double v) { return v
 template <> __device__ __forceinline__ double2 tscal<double2>(double v) { return make_double2(v, 0.0); }
 __device__ __forceinline__ double tscale(double a, double v) { return a * v; }
 __device__ __forceinline__ double2 tscale(double2 a, double v) { return make_double2(a.x * v, a.y * v); }
-__device__ __forceinline__ double trsqrt(double a) { return rsqrt(a); }
 // the same for the FP32 pre-pass (float / float2)
 __device__ __forceinline__ float tmul(float a, float b) { return a * b; }
 __device__ __forceinline__ float2 tmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
@@ -356,7 +347,6 @@ template <> __device__ __forceinline__ float tscal<float>(double v) { return (fl
 template <> __device__ __forceinline__ float2 tscal<float2>(double v) { return make_float2((float)v, 0.f); }
 __device__ __forceinline__ float tscale(float a, float v) { return a * v; }
 __device__ __forceinline__ float2 tscale(float2 a, float v) { return make_float2(a.x * v, a.y * v); }
-__device__ __forceinline__ float trsqrt(float a) { return rsqrtf(a); }
 // e^{-i arg a} for a != 0: the sign of a real a, conj(a) / |a| for a complex
 // one (FP64 unit modulus: an FP32 reciprocal square root refined by two
 // Newton steps in FP64)
@@ -1731,25 +1721,14 @@ unsigned rows_blocks(uint64_t rows, int members) {
 }
 
 template <typename R>
-cudaError_t expand_dispatch(qs_ctx* h, const Targets& tg, bool real, const double* E, int K, int e_stride,
+cudaError_t expand_launch(qs_ctx* h, const Targets& tg, bool real, const double* E, int K, int e_stride,
                             int max_cols, const KrausGate& g) {
-  const uint64_t work = ((1ull << h->n) >> tg.k) * (uint64_t)max_cols;
+  const uint64_t work = ((1ull << h->n) >> 2) * (uint64_t)max_cols;
   const dim3 grid(rows_blocks(work, h->batch), h->batch);
   auto* l = static_cast<const cplx<R>*>(h->state);
   auto* lp = static_cast<cplx<R>*>(h->work);
-  const int n = h->n, rcap = h->rank, mcap = h->mcap;
-  // a diagonal gate with phase noise has diagonal Kraus operators: one product per output
-  bool diag = g.k == 2 && g.noise == QS_NOISE_PHASE;
-  for (int r = 0; diag && r < 4; ++r)
-    for (int c = 0; c < 4; ++c)
-      if (r != c && (g.U[2 * (r * 4 + c)] != 0.0 || g.U[2 * (r * 4 + c) + 1] != 0.0)) diag = false;
-  if (diag && real) k_kraus_expand<R, 2, true, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else if (diag) k_kraus_expand<R, 2, false, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else if (tg.k == 1 && real) k_kraus_expand<R, 1, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else if (tg.k == 1) k_kraus_expand<R, 1, false><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else if (tg.k == 2 && real) k_kraus_expand<R, 2, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else if (tg.k == 2) k_kraus_expand<R, 2, false><<<grid, kExpBlock, 0, h->stream>>>(l, lp, n, rcap, mcap, tg, E, K, e_stride, h->rc, g);
-  else return cudaErrorInvalidValue;
+  if (real) k_kraus_expand<R, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, e_stride, h->rc, g);
+  else k_kraus_expand<R, false><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, e_stride, h->rc, g);
   return cudaGetLastError();
 }
 
@@ -1785,19 +1764,6 @@ size_t gram_partials_doubles(int n, int members, int rank) {
   return (size_t)members * std::max<size_t>(blocks * 2 * kTriMax, mom * mom_stride(rank));
 }
 int rank_counters() { return kMomGroups; }
-
-cudaError_t launch_kraus_expand(qs_ctx* h, const Targets& tg, bool real, const double* E, int K, int e_stride,
-                                int max_cols) {
-  KrausGate none{};
-  if (h->dtype == QS_C64) return expand_dispatch<float>(h, tg, real, E, K, e_stride, max_cols, none);
-  return expand_dispatch<double>(h, tg, real, E, K, e_stride, max_cols, none);
-}
-
-cudaError_t launch_kraus_expand_gate(qs_ctx* h, const Targets& tg, bool real, const KrausGate& g, int max_cols) {
-  const int K = kraus_count(g.k, g.noise);
-  if (h->dtype == QS_C64) return expand_dispatch<float>(h, tg, real, nullptr, K, 0, max_cols, g);
-  return expand_dispatch<double>(h, tg, real, nullptr, K, 0, max_cols, g);
-}
 
 cudaError_t launch_gram(qs_ctx* h, bool real, int max_M) {
   const uint64_t N = 1ull << h->n;
@@ -1887,8 +1853,8 @@ cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool di
                                 const KrausGate& g, int max_cols, int max_keep, int normalize) {
   if (tg.k == 2 && !diag) {                              // through L'
     const int max_M = std::min(kMaxGramDim, K * max_cols);
-    cudaError_t e = g.k > 0 ? launch_kraus_expand_gate(h, tg, real, g, max_cols)
-                            : launch_kraus_expand(h, tg, real, E, K, e_stride, max_cols);
+    cudaError_t e = h->dtype == QS_C64 ? expand_launch<float>(h, tg, real, E, K, e_stride, max_cols, g)
+                                       : expand_launch<double>(h, tg, real, E, K, e_stride, max_cols, g);
     if (e == cudaSuccess) e = launch_gram(h, real, max_M);
     if (e == cudaSuccess) e = launch_eig_truncate(h, 0, normalize);
     if (e == cudaSuccess) e = launch_project(h, real, K, max_keep);
