@@ -342,8 +342,10 @@ qs_status qs_plan_run(qs_plan p, double e, uint64_t seed, uint64_t gate_id0);
  * reference (qs_set_reference / qs_set_reference_from) in out[batch]: when
  * the plan ends with a fused pass, that pass also reduces <phi|psi_b> (FP64
  * across blocks) instead of a separate read of the state.  A start state set
- * by qs_set_basis_state(s) is created by the first fused pass instead of being
- * written to memory first.  STATEVEC only.  Synchronises. */
+ * by qs_set_basis_state(s) or qs_set_maximally_entangled is created by the first
+ * fused pass instead of being written to memory first; from a basis state the
+ * passes follow which qubits can be non-zero and write only what the last one
+ * must.  STATEVEC only.  Synchronises. */
 qs_status qs_plan_run_fidelity(qs_plan p, double e, uint64_t seed, uint64_t gate_id0, double* out);
 
 /* Number of passes over the state one run makes, and kernels it launches. */

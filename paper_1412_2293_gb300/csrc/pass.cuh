@@ -36,7 +36,6 @@ constexpr int kWin = 10;                   // the default window width M
 constexpr int kMaxWin = 12;                // the widest window (complex64)
 constexpr int kRegBits = 5;
 constexpr int kAmps = 32;
-constexpr int kMaxOther = 48;
 constexpr uint32_t kSpinLimit = 1u << 22;
 constexpr int kStatusTimeout = 0x51;       // value written to the status word on a timed-out wait
 constexpr int kMaxPassOps = 256;           // ops of one pass before segmentation

@@ -199,10 +199,10 @@ struct PreDesc {
 
 // Members' parameters of the passes of a run, one block of 128 threads per pass
 // and member (pass-major): the blocks of a pass alone are a chain of FP64 and
-// barrier latencies (31 us for 500 members of a Grover pass, 18 times a run), so
-// all passes' are launched together: the
-// noisy matrices of the dense gates in their factored forms, the phase
-// tables, the out factors.  The producer list holds the dense gates, then the
+// barrier latencies (31 us for 500 members of a Grover pass, 18 times a run: 571),
+// so all passes' are launched together (364 us; 285 with recip64): the noisy
+// matrices of the dense gates in their factored forms, the phase tables, the out
+// factors.  The producer list holds the dense gates, then the
 // tables, then the out terms (the order build_pass writes).  Every draw and
 // product is independent of the others except two chains: the dense gates of
 // one window bit (the diagonal carried from gate to gate) and the doubling of
@@ -986,7 +986,9 @@ int choose_window(const std::vector<PGate>& G, const std::vector<int>& rem, int 
 // order allows (an exchange is a write and a read of the whole tile in shared
 // memory): commuting ops of the current stage run first.  A layer of Hadamards, a
 // flip and another layer (two windows' worth of Grover's search) take two
-// exchanges instead of four.  partners: the lower window bits of each phase table;
+// exchanges instead of four (with the one parameter launch, serving Grover on 16
+// qubits 3.69 -> 3.21 ms, 27 trajectories of the 23-qubit QFT 523 -> 485 us).
+// partners: the lower window bits of each phase table;
 // end_stage: the stage the given order ends in.
 void order_stages(PassPlan* P, const std::vector<uint32_t>& partners, int end_stage) {
   std::vector<FOp> ops;

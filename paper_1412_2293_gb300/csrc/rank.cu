@@ -35,7 +35,6 @@ constexpr double kGsAccept = 1e-3;       // residual norm to accept a projection
 constexpr double kGsFallback = 1e-8;
 constexpr double kRotTol = 4e-16;        // rotate while |a_pq| > kRotTol * max|a_ii|
 constexpr int kJacobiSweeps32 = 12;      // bound on the FP32 pre-pass
-constexpr double kRotTol32 = 1e-6;       // FP32 pre-pass: rotate while |a_pq| > this * max|a_ii|
 
 __device__ __forceinline__ uint64_t insert0(uint64_t v, int s) {
   return ((v >> s) << (s + 1)) | (v & ((1ull << s) - 1));
@@ -450,7 +449,8 @@ __host__ __device__ inline MomSplit mom_split(int n, int kq) {
 // eight sums of an entry meet in shared memory (32 threads an entry would cost 31
 // FP64 additions there, as much as a quarter of the products at 15 qubits; blocks
 // of 512 threads, one per SM, left the pipe idle between their phases: five jobs
-// of ranks 1..8 at 15 qubits 54 us).  The last block of every kMomGroup adds the
+// of ranks 1..8 at 15 qubits 54 us, 43 as it is; the Gram matrix of L' took 99 and
+// its reduction 11, after 20 to write L').  The last block of every kMomGroup adds the
 // group's sums in block order, so the eigensolver's block has kMomGroups values
 // per entry left to add, not one per row block (its single SM would need 5 us
 // and more for those).
@@ -599,7 +599,8 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const cplx<R>* __restri
 // a row; a thread per row and column run rather than per group, and small blocks
 // (one per 128 / runs rows, no grid stride) share the FP64 work out over the SMs:
 // with 256 threads and two blocks of a rank-8 member on some SMs, one on others,
-// the pipe was busy 100 % on the first and 51 % on average.
+// the pipe was busy 100 % on the first and 51 % on average.  Five jobs of ranks
+// 1..8 at 15 qubits, one-qubit channel: 37 us, 105 from L' (which has K m columns).
 constexpr int kProjThreads = 128;
 template <typename R, bool REAL, int KQ, bool DIAG, int CB>
 __global__ void __launch_bounds__(kProjThreads) k_project_fused(cplx<R>* __restrict__ L, int n, int rcap, Targets tg, int K,
