@@ -164,3 +164,18 @@ def test_run_from_the_entangled_start_equals_the_run_from_memory(n, batch, dtype
     # created and loaded registers hold the same bits, and the same gates follow
     np.testing.assert_array_equal(got, want)
     np.testing.assert_array_equal(f_got, f_want)
+
+
+@pytest.mark.parametrize("n", [12, 20])
+def test_autotune_keeps_default_of_passes_without_a_choice(n):
+    """Every pass of the QFT from a pending basis start has one form, so timing
+    configurations there chooses nothing."""
+    h = qs.qs_create(n, 2, 0, qs.QS_STATEVEC, qs.QS_C64)
+    p = qs.qs_plan_create(h, pcirc.to_gates(inputs.qft_circuit(n)))
+    try:
+        qs.qs_set_basis_state(h, 3)
+        qs.qs_plan_autotune(p, 1, 0.01, SEED, h)
+        assert tuple(qs.qs_plan_get_config(p, h)) == ((2, 1) if qs.qs_plan_get_window(p, h) == 10 else (0, 0))
+    finally:
+        qs.qs_plan_destroy(p)
+        qs.qs_destroy(h)
