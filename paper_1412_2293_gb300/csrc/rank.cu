@@ -687,36 +687,29 @@ constexpr int kEigThreads = 256;                        // two warps per schedul
 // ---------------------------------------------------------------------------
 // Parallel cyclic Jacobi on the Hermitian (or real symmetric) A (M x M, pitch
 // kJP), accumulating V (V <- V R, from a unitary start).  Each step applies Mp / 2
-// disjoint rotations of the round-robin schedule: pair 0 = (s, Mp - 1), pair i =
-// ((s + i) mod (Mp - 1), (s - i) mod (Mp - 1)).  Most of the work is done in FP32
-// (a warp's FP64 instruction holds its scheduler for about 64 cycles on this GPU);
-// FP64 takes the matrices refine() declines, from a basis in which A is nearly
-// diagonal.
-// FP32, jacobi32: a step is a chain of latencies, so one warp walks it without
-// block barriers: lane i reads pair i's 2 x 2 block, finds its rotation with two
-// reciprocal square roots in sequence (c^2 = (1 + |th| / h) / 2, sigma = b / (2 h c),
-// h^2 = th^2 + |b|^2, R = [[c, sigma], [-conj(sigma), c]]) and writes it to a log in
-// shared memory; every lane then takes one off-diagonal 2 x 2 block (rows of pair i,
-// columns of pair j > i; 28 of them for M = 16), which it has read meanwhile, and
-// writes it and its conjugate transpose.  V needs only the log: the other warps
-// apply a sweep's rotations to it while warp 0 is in the next sweep (a warp owns
-// whole rows).  A pair rotates while |a_pq| > tol sqrt(a_pp a_qq) (G is a Gram
-// matrix: its small eigenvalues are graded, and the refinement needs their vectors
-// as well separated as the large ones') and above kFloor32 of the largest diagonal
-// entry; a sweep whose sines were all below 2e-4 ends the loop, what it leaves is
-// below their square.  A 16 x 16 real matrix takes 1.2 thousand cycles a rotating
-// step with everything around it (three warps on A, the rest on V and two block
-// barriers a step: 1.2-1.7); a 16-qubit Grover circuit at rank 8, 80 channels, went
-// from 7.56 to 7.31 ms with it.
+// disjoint rotations of the round-robin schedule: pair 0 = (Mp - 1, s), pair i =
+// ((s + i) mod (Mp - 1), (s - i) mod (Mp - 1)).  T is float / float2, where most of
+// the work is done (a warp's FP64 instruction holds its scheduler for about 64
+// cycles on this GPU), or double / double2, for matrices refine() declines, from a
+// basis in which A is nearly diagonal.
 //
-// FP64, jacobi: every warp tests the step's pairs (and all go on to the next step
-// when none rotates), warp 0 finds the rotations (the tangent in FP32 -- any tangent
-// gives an exactly unitary rotation, the next sweep removes what is left -- cos, sin
-// and the phase refined by Newton steps), the first warps update A, the others V, in
-// place.  Of A only the 2 x 2 blocks on and above the diagonal are computed, one of
-// their two columns a thread, and written below it as conjugates; what no rotating
-// pair touches is skipped.  A pair rotates while |a_pq| > tol * max |a_ii|; the loop
-// ends with a sweep without rotations.  Returns false if the sweep bound was reached.
+// A step is a chain of latencies: every warp tests the step's pairs (and all go
+// on to the next step when none rotates), warp 0 finds the rotations (lane =
+// pair: a phase makes a_pq real, then the classical angle; in FP64 the tangent is
+// found in FP32 -- any tangent gives an exactly unitary rotation, the next sweep
+// removes what is left -- and cos, sin and the phase are refined by Newton steps),
+// the first warps update A, the others V, in place.  Of A only the 2 x 2 blocks
+// (rows of pair i, columns of pair j >= i) are computed, one of their two columns
+// a thread, and written below the diagonal as conjugates; what no rotating pair
+// touches is skipped.
+//
+// FP32: a pair rotates while |a_pq| > tol sqrt(a_pp a_qq) (G is a Gram matrix:
+// its small eigenvalues are graded, and the refinement needs their vectors as
+// well separated as the large ones') and above kFloor32 of the largest
+// diagonal entry; a sweep whose tangents were all below 2e-4 ends the loop, what
+// it leaves is below their square.  FP64: while |a_pq| > tol * max |a_ii|; the
+// loop ends with a sweep without rotations.  Returns false if the sweep bound was
+// reached.
 constexpr float kFloor32 = 1e-13f;
 template <typename T> struct Rot {
   decltype(tre(T{})) c, s;               // R = [[c, s], [-s ph, c ph]]
@@ -743,169 +736,18 @@ __device__ __forceinline__ double2 tneg(double2 a) { return make_double2(-a.x, -
 // |a| > thr (a part's magnitude, thr >= 0 as bits) without the FP64 pipe
 __device__ __forceinline__ bool above(double a, long long thr) { return (__double_as_longlong(a) & 0x7fffffffffffffffll) > thr; }
 __device__ __forceinline__ bool above(double2 a, long long thr) { return above(a.x, thr) || above(a.y, thr); }
-__device__ __forceinline__ bool nonzero(double a) { return (__double_as_longlong(a) << 1) != 0; }
-__device__ __forceinline__ bool nonzero(double2 a) { return nonzero(a.x) || nonzero(a.y); }
-
-__device__ __forceinline__ void jacobi_pair(int st, int i, int m1, int* p, int* q) {
-  int a = st + i, c = st - i;
-  if (a >= m1) a -= m1;
-  if (c < 0) c += m1;
-  *p = a;
-  *q = i == 0 ? m1 : c;
-}
-// c x + g w, g = (gx, gy)
-__device__ __forceinline__ float rot_mix(float c, float x, float gx, float, float w) { return fmaf(c, x, gx * w); }
-__device__ __forceinline__ float2 rot_mix(float c, float2 x, float gx, float gy, float2 w) {
-  return make_float2(fmaf(c, x.x, fmaf(gx, w.x, -gy * w.y)), fmaf(c, x.y, fmaf(gx, w.y, gy * w.x)));
-}
-__device__ __forceinline__ float part_x(float a) { return a; }
-__device__ __forceinline__ float part_x(float2 a) { return a.x; }
-__device__ __forceinline__ float part_y(float) { return 0.f; }
-__device__ __forceinline__ float part_y(float2 a) { return a.y; }
-
-// log: 2 x (kMaxGramDim - 1) x kMaxGramDim / 2 rotations (c, Re sigma, Im sigma).  A and V: index M
-// of an odd M is padding, zeroed by the caller.
-constexpr int kLogPairs = kMaxGramDim / 2;
-constexpr int kLogSweep = (kMaxGramDim - 1) * kLogPairs;
-template <typename T>
-__device__ void jacobi32(T* A, T* V, float4* log, int M, float tol, int max_sweeps) {
-  __shared__ unsigned steps[2];          // steps of a sweep with rotations
-  __shared__ int more[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Mp = M + (M & 1), nb = Mp / 2, m1 = Mp - 1;
-  constexpr int kItems = (kLogPairs * (kLogPairs - 1) / 2 + 31) / 32;
-  const int nblocks = nb * (nb - 1) / 2;
-  int bi[kItems], bj[kItems];
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      bi[k] = bj[k] = 0;
-      // the strict upper triangle of nb x nb
-      int w = lane + 32 * k;
-      if (w < nblocks) {
-        int i = 0;
-        while (w >= nb - 1 - i) { w -= nb - 1 - i; ++i; }
-        bi[k] = i;
-        bj[k] = i + 1 + w;
-      }
-    }
-  }
-  auto rotate_v = [&](int sweep, int w, int nw) {
-    int nbp = 1;
-    while (nbp < nb) nbp *= 2;
-    const float4* lg = log + (sweep & 1) * kLogSweep;
-    const unsigned act = steps[sweep & 1];
-    const int j = lane & (nbp - 1);
-    for (int r0 = w * (32 / nbp); r0 < M; r0 += nw * (32 / nbp)) {
-      const int k = r0 + lane / nbp;
-      const bool on = k < M && j < nb;
-      for (unsigned left = act; left; left &= left - 1) {
-        const int st = __ffs(left) - 1;
-        if (on) {
-          int p, q;
-          jacobi_pair(st, j, m1, &p, &q);
-          const float4 r = lg[st * kLogPairs + j];
-          const T x = V[k * kJP + p], y = V[k * kJP + q];
-          V[k * kJP + p] = rot_mix(r.x, x, -r.y, r.z, y);
-          V[k * kJP + q] = rot_mix(r.x, y, r.y, r.z, x);
-        }
-        __syncwarp();
-      }
-    }
-  };
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (warp == 0) {
-      float4* lg = log + (sweep & 1) * kLogSweep;
-      float dmax = lane < M ? fabsf(tre(A[lane * kJP + lane])) : 0.f;
-#pragma unroll
-      for (int o = 16; o; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      const float floor2 = kFloor32 * dmax * kFloor32 * dmax, tol2 = tol * tol;
-      bool big = false;
-      unsigned act = 0;
-      for (int st = 0; st < m1; ++st) {
-        bool rotates = false;
-        float a = 0.f, d = 0.f, a2 = 0.f;
-        T b = tscal<T>(0.0);
-        int p = 0, q = 0;
-        if (lane < nb) {
-          jacobi_pair(st, lane, m1, &p, &q);
-          b = A[p * kJP + q];
-          a = tre(A[p * kJP + p]);
-          d = tre(A[q * kJP + q]);
-          a2 = tabs2(b);
-          rotates = a2 > tol2 * fabsf(a * d) && a2 > floor2;
-        }
-        if (!__any_sync(0xffffffffu, rotates)) continue;
-        act |= 1u << st;
-        if (lane < nb) {
-          float4 r = make_float4(1.f, 0.f, 0.f, 0.f);
-          if (rotates) {
-            const float th = 0.5f * (d - a), x = fmaf(th, th, a2);
-            const float rh = rsqrtf(x);
-            const float c2 = fmaf(0.5f * fabsf(th), rh, 0.5f);
-            const float rc = rsqrtf(c2);
-            const float k = copysignf(0.5f * rh * rc, th);
-            r = make_float4(c2 * rc, k * part_x(b), k * part_y(b), 0.f);
-            big |= k * k * a2 > 4e-8f;
-            const float tb = copysignf(__fdividef(a2, fmaf(x, rh, fabsf(th))), th);
-            A[p * kJP + p] = tscal<T>(a - tb);
-            A[q * kJP + q] = tscal<T>(d + tb);
-            A[p * kJP + q] = A[q * kJP + p] = tscal<T>(0.0);   // zero by construction
-          }
-          lg[st * kLogPairs + lane] = r;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-          if (32 * k >= nblocks) break;                  // the same on every lane
-          if (lane + 32 * k < nblocks) {
-            int i0, i1, j0, j1;
-            jacobi_pair(st, bi[k], m1, &i0, &i1);
-            jacobi_pair(st, bj[k], m1, &j0, &j1);
-            const T x00 = A[i0 * kJP + j0], x01 = A[i0 * kJP + j1], x10 = A[i1 * kJP + j0], x11 = A[i1 * kJP + j1];
-            const float4 ri = lg[st * kLogPairs + bi[k]], rj = lg[st * kLogPairs + bj[k]];
-            // X R_j, then R_i^H of it
-            const T y00 = rot_mix(rj.x, x00, -rj.y, rj.z, x01), y01 = rot_mix(rj.x, x01, rj.y, rj.z, x00);
-            const T y10 = rot_mix(rj.x, x10, -rj.y, rj.z, x11), y11 = rot_mix(rj.x, x11, rj.y, rj.z, x10);
-            const T z00 = rot_mix(ri.x, y00, -ri.y, -ri.z, y10), z10 = rot_mix(ri.x, y10, ri.y, -ri.z, y00);
-            const T z01 = rot_mix(ri.x, y01, -ri.y, -ri.z, y11), z11 = rot_mix(ri.x, y11, ri.y, -ri.z, y01);
-            A[i0 * kJP + j0] = z00;
-            A[i0 * kJP + j1] = z01;
-            A[i1 * kJP + j0] = z10;
-            A[i1 * kJP + j1] = z11;
-            A[j0 * kJP + i0] = tconj(z00);
-            A[j1 * kJP + i0] = tconj(z01);
-            A[j0 * kJP + i1] = tconj(z10);
-            A[j1 * kJP + i1] = tconj(z11);
-          }
-        }
-        __syncwarp();
-      }
-      const bool go = __any_sync(0xffffffffu, big);
-      if (lane == 0) {
-        steps[sweep & 1] = act;
-        more[sweep & 1] = go;
-      }
-    } else if (sweep > 0) {
-      rotate_v(sweep - 1, warp - 1, kEigThreads / 32 - 1);
-    }
-    __syncthreads();
-    if (!more[sweep & 1]) break;                         // the same on every thread
-  }
-  rotate_v(min(sweep, max_sweeps - 1), warp, kEigThreads / 32);
-  __syncthreads();
-}
 
 template <typename T>
 __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
   using RT = decltype(tre(T{}));
+  constexpr bool F64 = sizeof(RT) == 8;
   constexpr int kABlocks = (kMaxGramDim / 2) * (kMaxGramDim / 2 + 1);   // half blocks of A at most
   constexpr int kAThreads = 96;
   constexpr int kAItems = (kABlocks + kAThreads - 1) / kAThreads;
   constexpr int kVThreads = kEigThreads - kAThreads;
   constexpr int kVItems = (kMaxGramDim / 2 * kMaxGramDim + kVThreads - 1) / kVThreads;
   __shared__ Rot<T> rot[kMaxGramDim / 2];
+  __shared__ int more;
   const int tid = threadIdx.x, lane = tid & 31;
   const int Mp = M + (M & 1), nb = Mp / 2;
   const int na = nb * (nb + 1), nv = nb * M;
@@ -925,8 +767,13 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
     }
   }
   auto pair_of = [&](int st, int i, int* p, int* q) {
-    int a, c;
-    jacobi_pair(st, i, Mp - 1, &a, &c);
+    int a = st, c = Mp - 1;
+    if (i > 0) {
+      a = st + i;
+      if (a >= Mp - 1) a -= Mp - 1;
+      c = st - i;
+      if (c < 0) c += Mp - 1;
+    }
     *p = a < c ? a : c;
     *q = a < c ? c : a;
   };
@@ -934,8 +781,9 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
     float dmax = lane < M ? fabsf((float)tre(A[lane * kJP + lane])) : 0.f;
 #pragma unroll
     for (int o = 16; o; o >>= 1) dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    const float floor2 = kFloor32 * dmax * kFloor32 * dmax;
     const long long thr = __double_as_longlong((double)(tol * dmax));
-    bool did = false;
+    bool did = false, big = false;
     for (int st = 0; st < Mp - 1; ++st) {
       bool rotates = false;
       T apq = tscal<T>(0.0);
@@ -945,8 +793,15 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
         pair_of(st, lane, &p, &q);
         if (q < M) {
           apq = A[p * kJP + q];
-          rotates = above(apq, thr);
-          if (rotates && tid < 32) { app = tre(A[p * kJP + p]); aqq = tre(A[q * kJP + q]); }
+          if constexpr (F64) {
+            rotates = above(apq, thr);
+            if (rotates && tid < 32) { app = tre(A[p * kJP + p]); aqq = tre(A[q * kJP + q]); }
+          } else {
+            app = tre(A[p * kJP + p]);
+            aqq = tre(A[q * kJP + q]);
+            const float a2 = tabs2(apq);
+            rotates = a2 > tol * tol * fabsf(app * aqq) && a2 > floor2;
+          }
         }
       }
       const unsigned any = __ballot_sync(0xffffffffu, rotates);
@@ -958,14 +813,22 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
         const float th = 0.5f * (float)(aqq - app) * inv;
         const float h2 = 1.f + th * th;
         const float tf = copysignf(__fdividef(1.f, fabsf(th) + h2 * rsqrtf(h2)), th);
+        big |= fabsf(tf) > 2e-4f;
         Rot<T> r;
-        // 1 / sqrt(h) from an FP32 seed: y + y err (1 / 2 + 3 / 8 err), err = 1 - h y^2 (third order)
-        const double t = tf, h = fma(t, t, 1.0), y0 = rsqrtf(fmaf(tf, tf, 1.f));
-        const double err = fma(-(h * y0), y0, 1.0);
-        const double y = fma(y0 * err, fma(0.375, err, 0.5), y0);
-        r.c = y;
-        r.s = t * y;
-        const T ph = unit_phase(apq);
+        T ph;
+        if constexpr (F64) {
+          const double t = tf, h = fma(t, t, 1.0), hh = -0.5 * h;
+          double y = rsqrtf(fmaf(tf, tf, 1.f));          // 1 / sqrt(h): two Newton steps in FP64
+          y = y * fma(hh * y, y, 1.5);
+          y = y * fma(hh * y, y, 1.5);
+          r.c = y;
+          r.s = t * y;
+          ph = unit_phase(apq);
+        } else {
+          r.c = rsqrtf(1.f + tf * tf);
+          r.s = tf * r.c;
+          ph = tscale(tconj(apq), inv);
+        }
         r.sp = tscale(ph, r.s);
         r.cp = tscale(ph, r.c);
         rot[lane] = r;
@@ -1019,6 +882,7 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
           } else if (col == 0) {
             A[p * kJP + p] = tscal<T>(tre(x0));
           } else {
+            if (!F64) x0 = z;                            // the rotated pair: zero by construction
             A[p * kJP + q] = x0;
             A[q * kJP + p] = tconj(x0);
             A[q * kJP + q] = tscal<T>(tre(x1));
@@ -1041,6 +905,14 @@ __device__ bool jacobi(T* A, T* V, int M, float tol, int max_sweeps) {
       __syncthreads();
     }
     if (!did) return true;                               // no rotation in the whole sweep (the same on every thread)
+    if constexpr (!F64) {
+      if (tid < 32) {
+        const bool b = __any_sync(0xffffffffu, big);
+        if (lane == 0) more = b;
+      }
+      __syncthreads();
+      if (!more) return true;
+    }
   }
   return false;
 }
@@ -1244,8 +1116,7 @@ __device__ bool refine(const double2* G, const T* Q, T* Y, T* P, T* Z, T32* f32,
 // cluster's accepted vectors q_t; as the q_t lie in range(P),
 // <q_t, P e_j> = conj(q_t[j]) and |P e_j - ...|^2 = P_jj - sum_t |q_t[j]|^2,
 // so the projections need no dot products.  An accepted vector is
-// normalised by its norm: its residual, or the computed norm where the residual has
-// lost digits to the subtractions.  A cluster fills its own columns of the
+// normalised by its computed norm.  A cluster fills its own columns of the
 // basis (from the index of its first eigenvalue on), so the clusters are shared
 // out over the warps (lane = row).
 template <typename T>
@@ -1254,50 +1125,30 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
                            int* status) {
   __shared__ int order[kMaxGramDim + 1], start[kMaxGramDim + 1], nclusters;
   __shared__ double lam[kMaxGramDim];
-  __shared__ long long key[kMaxGramDim];
-  __shared__ unsigned near_[kMaxGramDim];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = kEigThreads / 32;
-  // descending, ties in index order: position of i = how many come before it,
-  // compared as integers that order like the doubles (off the FP64 pipe)
-  if (tid < M) {
-    const long long k = __double_as_longlong(lam_in[tid] + 0.0);
-    key[tid] = k ^ ((k >> 63) & 0x7fffffffffffffffll);
-  }
-  __syncthreads();
-  if (tid < M) {
+  // descending, ties in index order: position of i = how many come before it
+  for (int i = tid; i < M; i += blockDim.x) {
     int pos = 0;
-    for (int j = 0; j < M; ++j) pos += key[j] > key[tid] || (key[j] == key[tid] && j < tid);
-    order[pos] = tid;
-    lam[pos] = lam_in[tid];
+    for (int j = 0; j < M; ++j) pos += lam_in[j] > lam_in[i] || (lam_in[j] == lam_in[i] && j < i);
+    order[pos] = i;
+    lam[pos] = lam_in[i];
   }
   const int keep = r < M ? r : M;
   for (int i = tid; i < M * kJP; i += blockDim.x) basis[i] = tscal<T>(0.0);
   __syncthreads();
   const double lam1 = lam[0] > 0.0 ? lam[0] : 0.0;
-  for (int i = warp; i < keep; i += warps) {              // who is within the tolerance of i
-    const unsigned w = __ballot_sync(0xffffffffu, lane < M && lam[i] - lam[lane] <= kTieTol * lam1);
-    if (lane == 0) near_[i] = w;
-  }
-  __syncthreads();
   if (tid == 0) {
     int nc = 0, i0 = 0;
     while (i0 < keep) {
       start[nc++] = i0;
       int i1 = i0 + 1;
-      while (i1 < M && ((near_[i0] >> i1) & 1)) ++i1;
+      while (i1 < M && lam[i0] - lam[i1] <= kTieTol * lam1) ++i1;
       i0 = i1;
     }
     start[nc] = i0;
     nclusters = nc;
   }
   __syncthreads();
-  // the kept weight, while the other warps have the clusters
-  if (tid == 32 * (warps - 1)) {
-    double kept = 0.0;
-    for (int i = 0; i < keep; ++i) kept += lam[i] * unscale;
-    keep_out[0] = keep;
-    scale_out[0] = normalize ? 1.0 / sqrt(kept) : 1.0;
-  }
   for (int cl = warp; cl < nclusters; cl += warps) {
     const int i0 = start[cl], i1 = start[cl + 1];
     const int s = i1 - i0;
@@ -1315,63 +1166,42 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
       }
     }
     // P = S S^dagger; GS of P e_j, j = 0..M-1, thresholds kGsAccept then
-    // kGsFallback, as far as the kept vectors go.  Lane j holds candidate j's
-    // residual, P_jj - sum_t |q_t[j]|^2; it only falls, so the next accepted one is
-    // the first after the last that passes now.
+    // kGsFallback, as far as the kept vectors go
     const int need = i1 < keep ? i1 : keep;
-    double n2 = 0.0;
-    if (lane < M)
-      for (int c = i0; c < i1; ++c) {
-        const T v = V[lane * kJP + order[c]];
-        if (nonzero(v)) n2 += tabs2(v);
-      }
-    const float whole = (float)n2;                       // P_jj
     for (int pass = 0; pass < 2 && found < need; ++pass) {
       const double thr = pass == 0 ? kGsAccept : kGsFallback;
-      const long long thr2 = __double_as_longlong(thr * thr);
-      unsigned later = 0xffffffffu;
-      while (found < need) {
-        // (positive numbers' bits order like they do; no NaN)
-        const long long res = __double_as_longlong(n2);
-        const unsigned ok = __ballot_sync(0xffffffffu, lane < M && res > thr2 && res <= 0x7ff0000000000000ll) & later;
-        if (!ok) break;
-        const int j = __ffs(ok) - 1;
-        later = j == 31 ? 0u : 0xffffffffu << (j + 1);
-        // row `lane` of P e_j less the accepted vectors' parts; the coefficients
-        // are the same on every lane, and many are zero (eigenvectors of a
-        // circuit's early channels touch few rows)
+      for (int j = 0; j < M && found < need; ++j) {
+        // row `lane` of P e_j and of the accepted vectors' parts, and this lane's
+        // share of P_jj - sum_t |q_t[j]|^2 (lane = member of the cluster)
+        double n2 = lane < s ? tabs2(V[j * kJP + order[i0 + lane]]) : 0.0;
+        if (lane < found - i0) n2 -= tabs2(basis[j * kJP + i0 + lane]);
         T v0 = tscal<T>(0.0), v1 = tscal<T>(0.0);
-        for (int c = i0; c < i1; ++c) {
-          const T f = tconj(V[j * kJP + order[c]]);
-          if (!nonzero(f)) continue;
-          const T w = lane < M ? V[lane * kJP + order[c]] : tscal<T>(0.0);
-          if (c & 1) v1 = cmacc(w, f, v1);
-          else v0 = cmacc(w, f, v0);
-        }
-        for (int t = i0; t < found; ++t) {
-          const T f = tneg(tconj(basis[j * kJP + t]));
-          if (!nonzero(f)) continue;
-          const T w = lane < M ? basis[lane * kJP + t] : tscal<T>(0.0);
-          if (t & 1) v1 = cmacc(w, f, v1);
-          else v0 = cmacc(w, f, v0);
+        if (lane < M) {
+          for (int c = 0; c < s; c += 2) {
+            const int ca = order[i0 + c];
+            v0 = cmacc(V[lane * kJP + ca], tconj(V[j * kJP + ca]), v0);
+            if (c + 1 < s) {
+              const int cb = order[i0 + c + 1];
+              v1 = cmacc(V[lane * kJP + cb], tconj(V[j * kJP + cb]), v1);
+            }
+          }
+          for (int t = i0; t < found; t += 2) {
+            v0 = cmacc(basis[lane * kJP + t], tneg(tconj(basis[j * kJP + t])), v0);
+            if (t + 1 < found) v1 = cmacc(basis[lane * kJP + t + 1], tneg(tconj(basis[j * kJP + t + 1])), v1);
+          }
         }
         const T v = tadd(v0, v1);
-        // |v|^2 is the residual; summed anew where that has lost digits
-        double nv = __shfl_sync(0xffffffffu, n2, j);
-        if (!((float)nv > 0.5f * __shfl_sync(0xffffffffu, whole, j))) {
-          nv = tabs2(v);
+        double nv = lane < M ? tabs2(v) : 0.0;
 #pragma unroll
-          for (int o = 16; o; o >>= 1)
-            if (o < M) nv += __shfl_xor_sync(0xffffffffu, nv, o);   // lanes from M on hold zeros
+        for (int o = 16; o; o >>= 1) {
+          n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+          nv += __shfl_xor_sync(0xffffffffu, nv, o);
         }
-        T q = v;
-        if (__double_as_longlong(nv) != __double_as_longlong(1.0)) q = tscale(v, rsqrt(nv));
-        if (lane < M) {
-          basis[lane * kJP + found] = q;
-          n2 = lane == j ? 0.0 : n2 - tabs2(q);
+        if (n2 > thr * thr) {
+          if (lane < M) basis[lane * kJP + found] = tscale(v, rsqrt(nv));
+          ++found;
+          __syncwarp();
         }
-        ++found;
-        __syncwarp();
       }
     }
     if (found < need && lane == 0) status[0] = 2;      // incomplete cluster
@@ -1390,13 +1220,18 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
     }
   }
   for (int i = tid; i < M; i += blockDim.x) lam_out[i] = lam[i] * unscale;
+  if (tid == 0) {
+    double kept = 0.0;
+    for (int i = 0; i < keep; ++i) kept += lam[i] * unscale;
+    keep_out[0] = keep;
+    scale_out[0] = normalize ? 1.0 / sqrt(kept) : 1.0;
+  }
 }
 
 // Shared memory of the eigensolver: G, four FP64 matrices, five FP32 ones
 constexpr size_t kEigMat = (size_t)kMaxGramDim * kJP;
 constexpr int kEigSmem = (int)(kEigMat * (5 * sizeof(double2) + 5 * sizeof(float2)));
 constexpr float kTol32 = 3e-7f;
-static_assert(2 * kLogSweep * sizeof(float4) <= 3 * kEigMat * sizeof(float2), "the rotation log takes the last three");
 
 // Eigenvalues lam and eigenvectors (columns of *Qp) of G; see eig_member.
 template <typename T, typename T32>
@@ -1404,16 +1239,13 @@ __device__ void eig_vectors(const double2* G, T** Qp, T** Yp, T* P, T* Z, T32* f
   T32 *A32 = f32, *V32 = f32 + kEigMat;
   T *Q = *Qp, *Y = *Yp;
   const int tid = threadIdx.x, MM = M * M;
-  const int Mp = M + (M & 1);                            // an odd M is padded with a zero row and column
-  for (int i = tid; i < Mp * Mp; i += kEigThreads) {
-    const int p = i / Mp, q = i % Mp;
-    A32[p * kJP + q] = p < M && q < M ? to32(gsm<T>(G[p * kJP + q])) : tscal<T32>(0.0);
+  for (int i = tid; i < MM; i += kEigThreads) {
+    const int p = i / M, q = i % M;
+    A32[p * kJP + q] = to32(gsm<T>(G[p * kJP + q]));
     V32[p * kJP + q] = tscal<T32>(p == q ? 1.0 : 0.0);
   }
   __syncthreads();
-  // not converging here only costs FP64 sweeps
-  jacobi32<T32>(A32, V32, reinterpret_cast<float4*>(reinterpret_cast<float2*>(f32) + 2 * kEigMat), M, kTol32,
-                kJacobiSweeps32);
+  jacobi<T32>(A32, V32, M, kTol32, kJacobiSweeps32);    // not converging here only costs FP64 sweeps
   for (int i = tid; i < MM; i += kEigThreads) Q[(i / M) * kJP + i % M] = to64(V32[(i / M) * kJP + i % M]);
   __syncthreads();
   if (refine<T, T32>(G, Q, Y, P, Z, f32, M, lam)) {
@@ -1514,13 +1346,9 @@ extern __shared__ double2 eig_sm[];
 // One block per member: G_b, its eigendecomposition (real arithmetic when G_b
 // is real), truncation to r_b (or to trunc_r > 0 for an explicit truncation),
 // keep_b recorded; with moments, also the matrices V_ij of the projection.
-// One SM works while the others wait, so it is latency that counts: chains of FP64
-// instructions (100 cycles and more each) and instruction fetches of code that runs
-// once.  A real 16 x 16 matrix (rank 8, two Kraus operators) took 126 us with 256
-// threads, an FP64 Jacobi after the FP32 one and three block barriers a step; now
-// 60 thousand cycles (30 us) where refine() takes it -- 11 to load the moments and
-// form G, 10 for the FP32 Jacobi, 18 to refine, 21 to finish -- and 165 thousand with
-// the FP64 Jacobi (22 steps, 78).
+// One SM works while the others wait, so it is latency that counts.  A real 16 x
+// 16 matrix (rank 8, two Kraus operators) took 126 us with 256 threads, an FP64
+// Jacobi after the FP32 one and three block barriers a step.
 __global__ void __launch_bounds__(kEigThreads) k_eig_truncate(double* __restrict__ small, int sstride, RankCounts rc,
                                                               int trunc_r, int normalize, int* status,
                                                               const __grid_constant__ EigSource src) {
