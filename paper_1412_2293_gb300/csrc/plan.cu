@@ -607,9 +607,14 @@ __global__ void __launch_bounds__(256) k_out_entries(cplx<R>* __restrict__ tab, 
 // of V of MB members in registers and takes a run of tiles y, so the reference's
 // entries are read once for MB members.  Each member's overlap is summed over a
 // tile's 4 entries per thread in R and over the tiles by compensated sums in R
-// (two floats; FP64 for complex128), then in FP64 across the block.
+// (two floats; FP64 for complex128), then in FP64 across the block: the values of
+// its MB members are folded into one per lane group (9 or 6 additions a warp, 40
+// or 20 one by one), so a run can be short.
+// A run is 16 tiles (4 in complex128): one member of 20 (18) qubits has 64 blocks
+// then, 32 tiles gave it 32 (8) and took 84 us for 73 (263 for 184); 1024 members of
+// 20 qubits take 1.40 ms either way (1.44 with 32 tiles and no folding).
 constexpr int kOuterThreads = 256;
-constexpr int kOuterTiles = 32;          // tiles of a block
+template <typename R> constexpr int kOuterTiles = sizeof(R) == 4 ? 16 : 4;      // tiles of a block
 template <typename R> struct Acc2 {      // running sum with its rounding errors
   R s = R(0), c = R(0);
   __device__ __forceinline__ void add(R v) {
@@ -634,10 +639,11 @@ __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ p
   struct alignas(16) Vec { C v[W]; };
   const uint64_t tiles = 1ull << (n - m);
   const int slices = 1 << (m - 10);                      // 1024-amplitude slices of a tile
-  const unsigned runs = (unsigned)((tiles + kOuterTiles - 1) / kOuterTiles);
+  constexpr int T = kOuterTiles<R>;
+  const unsigned runs = (unsigned)((tiles + T - 1) / T);
   const unsigned run = blockIdx.x % runs;                // grid: runs of tiles, groups of members
-  const uint64_t y0 = (uint64_t)run * kOuterTiles;
-  const uint64_t y1 = y0 + kOuterTiles < tiles ? y0 + kOuterTiles : tiles;
+  const uint64_t y0 = (uint64_t)run * T;
+  const uint64_t y1 = y0 + T < tiles ? y0 + T : tiles;
   const int slice = blockIdx.y;
   const int b0 = (int)(blockIdx.x / runs) * MB;
   const uint64_t off = (uint64_t)slice * 1024;
@@ -680,25 +686,33 @@ __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ p
     }
   }
   if constexpr (FID) {
-    __shared__ double red[2][kOuterThreads / 32];
+    // value 2b + part of the 2 MB: each exchange over a lane bit halves what a lane
+    // keeps (the high half where its bit is set), then the lanes of a value meet
+    constexpr int NV = 2 * MB;
+    __shared__ double red[kOuterThreads / 32][NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int b = 0; b < MB && b0 + b < members; ++b) {
-      double re = 0.0, im = 0.0;
+    double w[NV];
 #pragma unroll
-      for (int k = 0; k < MB; ++k)
-        if (k == b) { re = ar[k].value(); im = ai[k].value(); }
-      re = warp_sum_d(re);
-      im = warp_sum_d(im);
-      __syncthreads();
-      if (lane == 0) { red[0][warp] = re; red[1][warp] = im; }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double sr = 0.0, si = 0.0;
-        for (int w = 0; w < kOuterThreads / 32; ++w) { sr += red[0][w]; si += red[1][w]; }
-        const uint64_t slot = ((uint64_t)(b0 + b) * runs + run) * slices + slice;
-        fid[2 * slot] = sr;
-        fid[2 * slot + 1] = si;
+    for (int b = 0; b < MB; ++b) { w[2 * b] = ar[b].value(); w[2 * b + 1] = ai[b].value(); }
+    int o = 16;
+#pragma unroll
+    for (int h = NV / 2; h; h >>= 1, o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int k = 0; k < h; ++k) {
+        const double give = up ? w[k] : w[k + h], own = up ? w[k + h] : w[k];
+        w[k] = own + __shfl_xor_sync(0xffffffffu, give, o);
       }
+    }
+#pragma unroll
+    for (int q = 16 / NV; q; q >>= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], q);
+    if ((lane & (32 / NV - 1)) == 0) red[warp][lane / (32 / NV)] = w[0];
+    __syncthreads();
+    if (threadIdx.x < NV && b0 + (int)(threadIdx.x >> 1) < members) {
+      double sum = 0.0;
+      for (int k = 0; k < kOuterThreads / 32; ++k) sum += red[k][threadIdx.x];
+      const uint64_t slot = ((uint64_t)(b0 + (threadIdx.x >> 1)) * runs + run) * slices + slice;
+      fid[2 * slot + (threadIdx.x & 1)] = sum;
     }
   }
 }
@@ -870,10 +884,11 @@ struct qs_plan_s {
   // Runs from basis states: the support grows by the qubits each pass's dense
   // gates act on.  start_full = the first step that completes it (all steps up to it
   // fused passes; -1: none, the first pass then writes the whole state);
-  // start_outer: that pass runs as one window and an outer product (k_outer), with
-  // these buffers.
+  // start_outer: that pass runs as one window and an outer product (k_outer),
+  // start_members members at a time in these buffers.
   int start_full = -1;
   bool start_outer = false;
+  int start_members = 0;
   void* d_start_c = nullptr;
   void* d_start_v = nullptr;
   std::vector<cudaEvent_t> events;     // launches + 1 when timing
@@ -1511,12 +1526,7 @@ PassMode pass_mode(qs_plan p, size_t i, int synth) {
   for (size_t j = 0; j < i; ++j) M.act |= p->passes[p->steps[j].pass].dense;
   M.load = i == 0 ? kUnit : kMasked;
   M.restricted = (int)i < p->start_full;
-  // the outer product adds two launches (about 9 us) and saves the pass's
-  // arithmetic, 3 ps an amplitude in complex64 and 80 in complex128: 2^22 (2^18)
-  // amplitudes is where that is 12 us (21 us); 64 members of 13 qubits, 2^19, took
-  // 182 us a launch with it and 172 without
-  const uint64_t amps = (uint64_t)p->h->batch << p->h->n;
-  M.outer = (int)i == p->start_full && p->start_outer && p->d_start_v && amps >= (p->h->esize == 8 ? 1ull << 22 : 1ull << 18);
+  M.outer = (int)i == p->start_full && p->start_outer;
   return M;
 }
 
@@ -1679,34 +1689,45 @@ cudaError_t launch_pass_args(qs_plan p, const PassPlan& P, const PassArgs& A, cp
 // fidelity slots per member of the outer product
 int outer_slots(qs_plan p, const PassPlan& P) {
   const uint64_t tiles = 1ull << (p->h->n - P.m);
-  return (int)((tiles + kOuterTiles - 1) / kOuterTiles) << (P.m - kWin);
+  const uint64_t per = p->h->esize == 8 ? kOuterTiles<float> : kOuterTiles<double>;
+  return (int)((tiles + per - 1) / per) << (P.m - kWin);
 }
 
 // The pass on the start's window state alone, one tile per member, then the
-// outer product with the amplitudes it starts from (see k_outer).
+// outer product with the amplitudes it starts from (see k_outer); start_members
+// members at a time, which changes no result.
 template <typename R>
 cudaError_t launch_outer(qs_plan p, const PassPlan& P, const PassMode& mode, int fid, cudaStream_t s) {
   using C = cplx<R>;
   qs_ctx* h = p->h;
-  PassArgs A = pass_args(p, P, mode, 0);
-  const uint64_t total = (uint64_t)h->batch << (h->n - P.m);
-  const unsigned g = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16);
-  k_gather_start<R><<<g, 256, 0, s>>>((const C*)h->state, (C*)p->d_start_c, h->n, P.m, total, A.basis, A.basis0);
-  A.synth = kUnit;
-  A.n = P.m;
-  A.tile_shift = 0;
-  A.tiles = (uint64_t)h->batch;
-  A.basis_mask = (1ull << P.m) - 1;
-  cudaError_t e = launch_pass_args<R>(p, P, A, (C*)p->d_start_v, s);
-  if (e != cudaSuccess) return e;
   constexpr int MB = sizeof(R) == 4 ? 4 : 2;
-  const unsigned runs = (unsigned)(((1ull << (h->n - P.m)) + kOuterTiles - 1) / kOuterTiles);
-  const dim3 grid(runs * (unsigned)((h->batch + MB - 1) / MB), 1u << (P.m - kWin));
-  auto* psi = (C*)h->state;
-  auto *v = (const C*)p->d_start_v, *c = (const C*)p->d_start_c, *ref = (const C*)h->ref;
-  if (fid) k_outer<R, MB, true><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, p->d_fid, h->n, P.m, h->batch);
-  else k_outer<R, MB, false><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, p->d_fid, h->n, P.m, h->batch);
-  return cudaGetLastError();
+  const int slots = outer_slots(p, P);
+  auto *v = (C*)p->d_start_v, *c = (C*)p->d_start_c;
+  auto* ref = (const C*)h->ref;
+  for (int b0 = 0; b0 < h->batch; b0 += p->start_members) {
+    const int count = std::min(p->start_members, h->batch - b0);
+    PassArgs A = pass_args(p, P, mode, 0);
+    A.synth = kUnit;
+    A.n = P.m;
+    A.tile_shift = 0;
+    A.tiles = (uint64_t)count;
+    A.basis_mask = (1ull << P.m) - 1;
+    A.params = static_cast<const R*>(A.params) + (size_t)b0 * P.stride;
+    if (A.basis) A.basis += b0;
+    C* psi = (C*)h->state + ((size_t)b0 << h->n);
+    const uint64_t total = (uint64_t)count << (h->n - P.m);
+    const unsigned g = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16);
+    k_gather_start<R><<<g, 256, 0, s>>>(psi, c, h->n, P.m, total, A.basis, A.basis0);
+    cudaError_t e = launch_pass_args<R>(p, P, A, v, s);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)(slots >> (P.m - kWin)) * (unsigned)((count + MB - 1) / MB), 1u << (P.m - kWin));
+    double* f = p->d_fid + 2 * (size_t)b0 * slots;
+    if (fid) k_outer<R, MB, true><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, f, h->n, P.m, count);
+    else k_outer<R, MB, false><<<grid, kOuterThreads, 0, s>>>(psi, v, c, ref, f, h->n, P.m, count);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 template <typename R>
@@ -2123,7 +2144,16 @@ qs_status run_plan(qs_plan p, double e, uint64_t seed, uint64_t gate_id0, int wa
 }
 
 // Where the support of a run from basis states becomes the whole state, and
-// whether that pass can run as an outer product (see k_outer).
+// whether that pass runs as an outer product (see k_outer): c (U e) and U (c e)
+// round differently, so this is a rule on the plan alone, and a trajectory's
+// result does not depend on how many share its launch.  The outer product adds
+// two launches (about 10 us) and saves the pass's arithmetic, 3 ps an amplitude in
+// complex64 and 80 in complex128, and the pass's chain of FP64 latencies on tiles
+// beyond one a warp.  From 17 (14) qubits: QFT of 17, 1024 complex64 members 555 ->
+// 359 us, one 72 -> 77, four 71 -> 85; 14, 75 complex128 members 207 -> 170, one 148 ->
+// 159; at 16, 1024 members 354 -> 308 but four 63 -> 85, at 13 complex128, 75 members
+// 148 -> 171.
+int outer_qubits(size_t esize) { return esize == 8 ? 17 : 14; }
 void find_start(qs_plan p) {
   p->start_full = -1;
   p->start_outer = false;
@@ -2134,7 +2164,8 @@ void find_start(qs_plan p) {
     if ((act | P.dense) == all) {
       p->start_full = (int)i;
       const uint64_t win = (1ull << P.m) - 1;
-      p->start_outer = i > 0 && !P.high && (act & win) == 0 && P.out_start[P.m + 1] == 0 && P.flips.empty();
+      p->start_outer = i > 0 && !P.high && (act & win) == 0 && P.out_start[P.m + 1] == 0 && P.flips.empty() &&
+                       p->h->n >= outer_qubits(p->h->esize);
       return;
     }
     act |= P.dense;
@@ -2255,13 +2286,19 @@ qs_status alloc_passes(qs_plan p) {
       cudaMalloc((void**)&p->d_fid, 2 * fid_slots_max * h->batch * sizeof(double)) != cudaSuccess)
     st = pfail(p, QS_ERR_OUT_OF_MEMORY, "fidelity partials");
   if (st == QS_OK && p->start_outer) {
-    // without room for these the pass runs on every tile instead
+    // window states of up to 16 MB (2048 complex64 members of 10 qubits: more
+    // members take turns, a few launches beside a millisecond and more of writes),
+    // and fewer where there is no room for these
     const PassPlan& P = p->passes[p->steps[p->start_full].pass];
-    if (cudaMalloc(&p->d_start_c, ((size_t)h->batch << (h->n - P.m)) * h->esize) != cudaSuccess ||
-        cudaMalloc(&p->d_start_v, ((size_t)h->batch << P.m) * h->esize) != cudaSuccess) {
+    p->start_members = (int)std::min<size_t>((size_t)h->batch, ((size_t)16 << 20 >> P.m) / h->esize);
+    for (;; p->start_members /= 2) {
+      if (cudaMalloc(&p->d_start_c, ((size_t)p->start_members << (h->n - P.m)) * h->esize) == cudaSuccess &&
+          cudaMalloc(&p->d_start_v, ((size_t)p->start_members << P.m) * h->esize) == cudaSuccess)
+        break;
       cudaGetLastError();
       if (p->d_start_c) cudaFree(p->d_start_c);
-      p->d_start_c = p->d_start_v = nullptr;
+      p->d_start_c = nullptr;
+      if (p->start_members == 1) { st = pfail(p, QS_ERR_OUT_OF_MEMORY, "plan start buffers"); break; }
     }
   }
   return st;
@@ -2805,8 +2842,9 @@ qs_status qs_plan_info(qs_plan p, int* passes, int* launches) {
   if (passes) *passes = (int)p->steps.size();
   if (launches) {
     *launches = p->kernels;
-    // the gather and the outer product beside the pass they run
-    if (p->h->pending && p->start_full > 0 && pass_mode(p, (size_t)p->start_full, p->h->pending).outer) *launches += 2;
+    // the gather and the outer product beside the pass they run, for start_members members at a time
+    if (p->h->pending && p->start_full > 0 && pass_mode(p, (size_t)p->start_full, p->h->pending).outer)
+      *launches += 3 * ((p->h->batch + p->start_members - 1) / p->start_members) - 1;
   }
   return QS_OK;
 }
