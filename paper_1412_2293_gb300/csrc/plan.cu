@@ -2320,6 +2320,9 @@ void free_passes(qs_plan p) {
   p->d_start_c = p->d_start_v = nullptr;
   p->d_params = p->d_alpha = nullptr;
   p->d_fid = nullptr;
+  p->start_full = -1;                    // (they name steps that are gone)
+  p->start_outer = false;
+  p->start_members = 0;
 }
 
 // timing slots (precompute + pass, or one single step) and kernels of one run

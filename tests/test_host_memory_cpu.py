@@ -1,0 +1,70 @@
+"""Host code of the library on a fake CUDA runtime (tests/fake_cudart.cc): the
+device memory a handle and its plans take against the server's admission bound,
+and plans after an allocation failed."""
+import glob
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_1412_2293_gb300 import build
+
+ROOT = build.ROOT
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """Path of the library linked against the fake runtime."""
+    objs = sorted(glob.glob(os.path.join(build.OUT_DIR, "obj", "*.o")))
+    if not build.up_to_date() or len(objs) != len(build.sources()):
+        build.build(force=True)
+        objs = sorted(glob.glob(os.path.join(build.OUT_DIR, "obj", "*.o")))
+    out = str(tmp_path_factory.mktemp("fake") / "libqsim_fake.so")
+    subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-o", out, os.path.join(ROOT, "tests", "fake_cudart.cc"), *objs,
+                    "-Wl,--no-undefined"], check=True, capture_output=True)
+    return out
+
+
+PRELUDE = """
+import sys, ctypes as ct
+sys.path.insert(0, {root!r})
+from paper_1412_2293_gb300 import circuits, inputs, qs, server
+qs.LIB_PATH = {lib!r}
+L = qs.lib()
+L.fake_device_bytes.restype = ct.c_size_t
+L.fake_pinned_blocks.restype = ct.c_size_t
+L.fake_pinned_calls.restype = ct.c_long
+L.fake_fail_after.argtypes = [ct.c_long]
+def circuit(name, n, it):
+    return circuits.to_gates(inputs.qft_circuit(n) if name == "qft" else inputs.grover_circuit(n, it, 1), per_member_flip=True)
+"""
+
+
+def run(lib, body):
+    """The body in an interpreter of its own (a fault in host code ends that one only)."""
+    r = subprocess.run([sys.executable, "-c", PRELUDE.format(root=ROOT, lib=lib) + body], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout[-2000:], r.stderr[-2000:])
+
+
+def test_plan_stays_usable_after_a_window_width_found_no_memory(fake):
+    run(fake, """
+for fail in range(24):
+    h = qs.qs_create(20, 4, 0, qs.QS_STATEVEC, qs.QS_C64)
+    p = qs.qs_plan_create(h, circuit("qft", 20, 0))
+    qs.qs_set_basis_state(h, 3)
+    L.fake_fail_after(fail)
+    try:
+        qs.qs_plan_set_window(p, 12, h)
+        L.fake_fail_after(-1)
+        passes, launches = qs.qs_plan_info(p)
+        assert passes == 2 and launches >= 5, (fail, passes, launches)
+    except qs.QSError as err:
+        assert err.status == qs.QS_ERR_OUT_OF_MEMORY, err
+        assert qs.qs_plan_info(p) == (0, 0), (fail, qs.qs_plan_info(p))
+        qs.qs_plan_set_window(p, 10, h)
+        assert qs.qs_plan_info(p)[0] == 2
+    qs.qs_plan_destroy(p)
+    qs.qs_destroy(h)
+assert L.fake_device_bytes() == 0
+""")
