@@ -2231,10 +2231,12 @@ void plan_passes(qs_plan p, const std::vector<int>& rem) {
   find_start(p);
 }
 
-// Device copies of the passes' op lists, their tensor maps, and the buffers
-// every pass shares: one parameter block and one out-factor table (a pass's
-// precompute runs on the same stream right before the pass itself) and the
-// fused-fidelity partials.
+// Device copies of the passes' op lists, their tensor maps, the passes' parameter
+// blocks (see k_precompute; one block that they share, each filled right before its
+// pass, where all of them would be too large) and the buffers every pass shares:
+// one out-factor table, filled before the pass on the same stream, and the
+// fused-fidelity partials; and the buffers of an outer product.  server.member_bytes
+// bounds the sum of all this for a member.
 qs_status alloc_passes(qs_plan p) {
   qs_ctx* h = p->h;
   qs_status st = QS_OK;
@@ -2259,9 +2261,9 @@ qs_status alloc_passes(qs_plan p) {
   // the most fidelity partials any configuration writes: 2^(n-10) per member
   const size_t fid_slots_max = (size_t)1 << (h->n - kWin);
   if (st == QS_OK && !p->passes.empty()) {
-    // a parameter block per pass, computed in one launch, while all of them take
-    // less than 1/64 of the state (or 64 MB)
-    p->params_apart = params_sum <= std::max<size_t>(h->state_elems * h->esize / 64, 64u << 20) &&
+    // a parameter block per pass, computed in one launch, while all of them take at
+    // most 512 KiB a member (8 MiB for fewer than 16 members)
+    p->params_apart = params_sum <= (size_t)std::max(h->batch, 16) << 19 &&
                       (uint64_t)h->batch * p->passes.size() < (1ull << 31);
     if (p->params_apart && cudaMalloc(&p->d_params, std::max<size_t>(params_sum, 16)) != cudaSuccess) {
       cudaGetLastError();

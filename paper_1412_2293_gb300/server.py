@@ -95,11 +95,15 @@ RANK_MEMBERS = 16                     # most fixed-rank jobs in one launch
 
 
 def member_bytes(n: int) -> int:
-    """Device bytes of one complex64 trajectory (upper bound): its amplitudes,
-    reduction partials (1/64 of the state), the out-of-window factors of the
-    fused passes (11 complex per 1024 amplitudes) and at most 512 KiB of
-    per-member gate parameters and phase tables."""
-    return (1 << n) * C64_BYTES + (1 << n) // 64 + (11 * C64_BYTES << max(n - 10, 0)) + (1 << 19)
+    """Device bytes of one complex64 trajectory (upper bound) in a launch of at
+    least 16: its amplitudes, reduction partials (the fused fidelity's, 1/64 of
+    the amplitude count, and the handle's, 1/256), the out-of-window factors of
+    the fused passes (11 complex per 1024 amplitudes), the buffers of the outer
+    product (one complex per 1024 amplitudes and a window of at most 4096), at
+    most 512 KiB of gate parameters and phase tables of all passes, and 1 KiB
+    of its inputs and matrices."""
+    return (1 << n) * C64_BYTES + (1 << n) // 64 + (1 << n) // 256 + (12 * C64_BYTES << max(n - 10, 0)) + \
+        (C64_BYTES << 12) + (1 << 19) + (1 << 10)
 
 
 def rank_bytes(n: int, r: int = RANK_MAX) -> int:

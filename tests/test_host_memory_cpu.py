@@ -68,3 +68,25 @@ for fail in range(24):
     qs.qs_destroy(h)
 assert L.fake_device_bytes() == 0
 """)
+
+
+# what the server runs: its smallest launch and larger ones, all widths, circuits of few and of thousands of passes
+@pytest.mark.parametrize("name,n,it,members,m", [
+    ("qft", 8, 0, 16, 10), ("qft", 13, 0, 64, 10), ("qft", 17, 0, 16, 10), ("qft", 20, 0, 256, 10), ("qft", 21, 0, 16, 11),
+    ("qft", 24, 0, 16, 12), ("qft", 26, 0, 16, 10), ("grover", 10, 25, 16, 10), ("grover", 16, 201, 16, 10),
+    ("grover", 12, 900, 16, 10), ("grover", 12, 900, 128, 10),
+])
+def test_admission_bound_covers_what_a_launch_allocates(fake, name, n, it, members, m):
+    run(fake, f"""
+name, n, it, B, m = {name!r}, {n}, {it}, {members}, {m}
+h = qs.qs_create(n, B, 0, qs.QS_STATEVEC, qs.QS_C64)
+p = qs.qs_plan_create(h, circuit(name, n, it))
+qs.qs_plan_set_window(p, m, h)
+qs.qs_set_member_noise(h, [0.01] * B, [1] * B, range(B), [1] * B)
+qs.qs_set_basis_states(h, [0] * B)
+used, bound = L.fake_device_bytes(), B * server.member_bytes(n)
+assert used <= bound, (used / B, bound / B)
+qs.qs_plan_destroy(p)
+qs.qs_destroy(h)
+assert L.fake_device_bytes() == 0
+""")
