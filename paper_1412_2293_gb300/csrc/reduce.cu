@@ -11,6 +11,7 @@
 #include <algorithm>
 
 #include "internal.cuh"
+#include "sums.cuh"
 
 namespace qs {
 
@@ -45,29 +46,19 @@ __device__ __forceinline__ double2 block_sum2(double a, double b) {
   return r;
 }
 
-// Sums of products to more than FP64's input precision on the FP32 pipe: a
-// product of two floats as (rounded, exact remainder), the running sum as
-// (sum, what its roundings lost) -- the compensated dot product of Ogita, Rump
-// and Oishi (SIAM J. Sci. Comput. 26, 2005), as accurate as a 48-bit sum.  A
-// multiply-add takes 10 FP32 instructions; the FP64 one and its two
-// conversions hold a scheduler's FP64 unit for about 64 cycles each on GB300.
+// A sum of a few values in two floats: the running sum and what its roundings
+// lost (48 bits).
 struct Sum2 {
   float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void plus(float p, float e) {   // += p + e
+  __device__ __forceinline__ void add(float p) {
     const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)), e));
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)));
     s = t;
   }
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    plus(p, __fmaf_rn(a, b, -p));
-  }
-  __device__ __forceinline__ void add(float v) { plus(v, 0.f); }
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 struct Sum1 {
   double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ double value() const { return s; }
 };
@@ -260,8 +251,15 @@ __global__ void __launch_bounds__(kRBlock) k_dm_trace_partials(const cplx<R>* rh
 // their real part counted twice, 2 Re sum_{i<j}, plus the real diagonal; the
 // part of a row that is summed starts at i, so blocks take rows from both
 // ends in turn.  Bound by the FP64 pipe in complex128, four multiply-adds an
-// entry (14 qubits 2.99 -> 0.99 ms for half the entries); in complex64 with Sum2
-// 13 qubits take 0.11 ms (1.28 before; the half read is 0.04 ms of HBM).
+// entry (14 qubits 2.99 -> 0.99 ms for half the entries).
+// complex64: the products and their sum in three floats (Sum3), phi scaled by
+// 2^100 so that of the remainders only what is below 2^-249 is lost.  A row whose sum
+// leaves FP32's range, or is so small (2^-172) that those could matter, is summed
+// again in FP64: the result carries FP64's bits whatever the magnitudes (a row all
+// of whose products are below 2^-249 is zero).  13 qubits, the call with its
+// read-back: 1.44 ms with FP64 sums over the whole matrix, 0.18 so; two floats
+// (48 bits) took 0.14.
+constexpr float kExpectScale = 0x1p100f;
 template <typename R, bool HERM>
 __global__ void __launch_bounds__(kRBlock) k_dm_expect_rows(const cplx<R>* __restrict__ rho,
                                                             const cplx<R>* __restrict__ phi, int n,
@@ -270,19 +268,50 @@ __global__ void __launch_bounds__(kRBlock) k_dm_expect_rows(const cplx<R>* __res
   const uint64_t bi = blockIdx.x;
   const uint64_t i = HERM ? ((bi & 1) ? N - 1 - (bi >> 1) : bi >> 1) : bi;
   const cplx<R>* row = rho + i * N;
-  typename SumOf<R>::T re, im;
   // whole aligned steps of the block from the one that holds column i + 1
   const uint64_t j0 = HERM ? ((i + 1) & ~(uint64_t)(kRBlock - 1)) : 0;
+  auto each = [&](auto&& f) {
 #pragma unroll 4
-  for (uint64_t j = j0 + threadIdx.x; j < N; j += kRBlock) {
-    if (HERM && j <= i) continue;
-    const cplx<R> a = row[j], f = phi[j];
-    re.add(a.x, f.x);
-    re.add(-a.y, f.y);
-    im.add(a.x, f.y);
-    im.add(a.y, f.x);
+    for (uint64_t j = j0 + threadIdx.x; j < N; j += kRBlock) {
+      if (HERM && j <= i) continue;
+      f(row[j], phi[j]);
+    }
+  };
+  auto in64 = [&]() {
+    double re = 0.0, im = 0.0;
+    each([&](cplx<R> a, cplx<R> f) {
+      re = fma((double)a.x, (double)f.x, re);
+      re = fma(-(double)a.y, (double)f.y, re);
+      im = fma((double)a.x, (double)f.y, im);
+      im = fma((double)a.y, (double)f.x, im);
+    });
+    return block_sum2(re, im);
+  };
+  double2 v;
+  if constexpr (sizeof(R) == 8) {
+    v = in64();
+  } else {
+    Sum3 re, im;
+    bool any = false;                    // a product that is not zero
+    each([&](cplx<R> a, cplx<R> f) {
+      f.x *= kExpectScale;
+      f.y *= kExpectScale;
+      re.add(a.x, f.x);
+      re.add(-a.y, f.y);
+      im.add(a.x, f.y);
+      im.add(a.y, f.x);
+      any |= re.s != 0.f || im.s != 0.f;
+    });
+    v = block_sum2(re.value(), im.value());
+    any = __syncthreads_or(any);
+    const double most = fmax(fabs(v.x), fabs(v.y));
+    if (__syncthreads_or(threadIdx.x == 0 && any && !(most >= 0x1p-72 && most < 0x1p126))) {
+      v = in64();
+    } else {
+      v.x *= 1.0 / (double)kExpectScale;
+      v.y *= 1.0 / (double)kExpectScale;
+    }
   }
-  const double2 v = block_sum2(re.value(), im.value());
   if (threadIdx.x == 0) {
     const cplx<R> f = phi[i];
     double r = (double)f.x * v.x + (double)f.y * v.y;                  // Re(conj(f) v)
