@@ -46,26 +46,6 @@ __device__ __forceinline__ double2 block_sum2(double a, double b) {
   return r;
 }
 
-// A sum of a few values in two floats: the running sum and what its roundings
-// lost (48 bits).
-struct Sum2 {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float p) {
-    const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z)));
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-struct Sum1 {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <typename R> struct SumOf;
-template <> struct SumOf<float> { using T = Sum2; };
-template <> struct SumOf<double> { using T = Sum1; };
-
 // A thread's kPer amplitudes of a full chunk are read as 16-byte vectors
 // (two complex64 amplitudes or one complex128) before any of them is used:
 // the sweep is bound by HBM latency otherwise (one 8-byte load in flight per
@@ -105,27 +85,27 @@ __device__ __forceinline__ void chunk_each(const cplx<R>* __restrict__ p, const 
 // partial[member][chunk] = sum over the chunk of conj(ref_i) psi_i.  Bound by
 // HBM (the members; the reference stays in L2) and by the FP64 adds of the block
 // sums (20 warp instructions of 64 cycles a block), so from 20 qubits on a block
-// takes kRounds rounds of 4096 amplitudes, a thread's sums of 16 products added
-// up between rounds with their rounding errors (two floats).  64 members of 2^21
-// complex64 amplitudes: 328 us with neither, 259 with the wide loads, 171 with both
-// (6.3 TB/s).
+// takes four rounds of 4096 amplitudes (chunk_rounds), a thread's sums of 16
+// products added up in FP64 between rounds.  64 members of 2^20 complex64
+// amplitudes, the call with its read-back: 209 -> 123 us, half of it the wide loads
+// (two floats between rounds took 119, and were 48 bits with FP32's exponents).
 template <typename R>
 __global__ void __launch_bounds__(kRBlock) k_dot_partials(const cplx<R>* __restrict__ psi,
                                                           const cplx<R>* __restrict__ ref, int n,
                                                           int chunks, int rounds, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  typename SumOf<R>::T sre, sim;
+  double sre = 0.0, sim = 0.0;
   for (int k = 0; k < rounds; ++k) {
     R re = 0, im = 0;
     chunk_each<R, true>(psi + (uint64_t)b * N, ref, ((uint64_t)c * rounds + k) * kChunk, N, [&](cplx<R> a, cplx<R> r) {
       re += r.x * a.x + r.y * a.y;
       im += r.x * a.y - r.y * a.x;
     });
-    sre.add(re);
-    sim.add(im);
+    sre += (double)re;
+    sim += (double)im;
   }
-  const double2 s = block_sum2(sre.value(), sim.value());
+  const double2 s = block_sum2(sre, sim);
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = s.x;
     partials[2 * ((uint64_t)b * chunks + c) + 1] = s.y;
@@ -138,14 +118,14 @@ __global__ void __launch_bounds__(kRBlock) k_norm_partials(const cplx<R>* __rest
                                                            int chunks, int rounds, double* partials) {
   const int c = blockIdx.x, b = blockIdx.y;
   const uint64_t N = 1ull << n;
-  typename SumOf<R>::T sum;
+  double sum = 0.0;
   for (int k = 0; k < rounds; ++k) {
     R s = 0;
     chunk_each<R, false>(psi + (uint64_t)b * N, psi, ((uint64_t)c * rounds + k) * kChunk, N,
                          [&](cplx<R> a, cplx<R>) { s += a.x * a.x + a.y * a.y; });
-    sum.add(s);
+    sum += (double)s;
   }
-  const double2 t = block_sum2(sum.value(), 0.0);
+  const double2 t = block_sum2(sum, 0.0);
   if (threadIdx.x == 0) {
     partials[2 * ((uint64_t)b * chunks + c)] = t.x;
     partials[2 * ((uint64_t)b * chunks + c) + 1] = 0.0;
