@@ -605,30 +605,16 @@ __global__ void __launch_bounds__(256) k_out_entries(cplx<R>* __restrict__ tab, 
 // member), the c_y are gathered, and this kernel writes the product (and reduces
 // <ref|psi>): bound by the HBM write of the state.  A block keeps 1024 entries
 // of V of MB members in registers and takes a run of tiles y, so the reference's
-// entries are read once for MB members.  Each member's overlap is summed over a
-// tile's 4 entries per thread in R and over the tiles by compensated sums in R
-// (two floats; FP64 for complex128), then in FP64 across the block: the values of
-// its MB members are folded into one per lane group (9 or 6 additions a warp, 40
-// or 20 one by one), so a run can be short.
+// entries are read once for MB members.  Each member's overlap is summed in R over
+// a thread's 4 entries of 4 tiles, as many products as the other reductions take,
+// and in FP64 from there: across the block the values of its MB members are folded
+// into one per lane group (9 or 6 additions a warp, 40 or 20 one by one), so a run
+// can be short.
 // A run is 16 tiles (4 in complex128): one member of 20 (18) qubits has 64 blocks
 // then, 32 tiles gave it 32 (8) and took 84 us for 73 (263 for 184); 1024 members of
 // 20 qubits take 1.40 ms either way (1.44 with 32 tiles and no folding).
 constexpr int kOuterThreads = 256;
 template <typename R> constexpr int kOuterTiles = sizeof(R) == 4 ? 16 : 4;      // tiles of a block
-template <typename R> struct Acc2 {      // running sum with its rounding errors
-  R s = R(0), c = R(0);
-  __device__ __forceinline__ void add(R v) {
-    if constexpr (sizeof(R) == 4) {
-      const float t = __fadd_rn(s, v), z = __fadd_rn(t, -s);
-      c = __fadd_rn(c, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(v, -z)));
-      s = t;
-    } else {
-      s += v;
-    }
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-
 template <typename R, int MB, bool FID>
 __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ psi, const cplx<R>* __restrict__ V,
                                                          const cplx<R>* __restrict__ cs, const cplx<R>* __restrict__ ref,
@@ -648,13 +634,17 @@ __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ p
   const int b0 = (int)(blockIdx.x / runs) * MB;
   const uint64_t off = (uint64_t)slice * 1024;
   Vec v[MB][L];
-  Acc2<R> ar[MB], ai[MB];
+  C d[MB];                                               // running products
+  double w[2 * MB];                                      // (re, im) of each member, as far as summed
 #pragma unroll
-  for (int b = 0; b < MB; ++b)
+  for (int b = 0; b < MB; ++b) {
+    d[b] = mk<R>(R(0), R(0));
+    w[2 * b] = w[2 * b + 1] = 0.0;
 #pragma unroll
     for (int l = 0; l < L; ++l)
       if (b0 + b < members)
         v[b][l] = *reinterpret_cast<const Vec*>(V + (((uint64_t)(b0 + b)) << m) + off + (l * kOuterThreads + threadIdx.x) * W);
+  }
   for (uint64_t y = y0; y < y1; ++y) {
     Vec r[L];
     if constexpr (FID) {
@@ -667,21 +657,24 @@ __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ p
       if (b0 + b >= members) break;
       const C c = cs[((uint64_t)(b0 + b) << (n - m)) + y];
       C* out = psi + ((uint64_t)(b0 + b) << n) + (y << m) + off;
-      C d = mk<R>(R(0), R(0));
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         Vec o;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-          o.v[w] = pmul<R>(c, v[b][l].v[w]);
-          if constexpr (FID) d = pdot<R>(d, r[l].v[w], o.v[w]);
+        for (int k = 0; k < W; ++k) {
+          o.v[k] = pmul<R>(c, v[b][l].v[k]);
+          if constexpr (FID) d[b] = pdot<R>(d[b], r[l].v[k], o.v[k]);
         }
         __stcs(reinterpret_cast<typename std::conditional<sizeof(R) == 4, float4, double2>::type*>(out + (l * kOuterThreads + threadIdx.x) * W),
                *reinterpret_cast<typename std::conditional<sizeof(R) == 4, float4, double2>::type*>(&o));
       }
-      if constexpr (FID) {
-        ar[b].add(d.x);
-        ai[b].add(d.y);
+    }
+    if (FID && ((y - y0) % 4 == 3 || y + 1 == y1)) {
+#pragma unroll
+      for (int b = 0; b < MB; ++b) {
+        w[2 * b] += (double)d[b].x;
+        w[2 * b + 1] += (double)d[b].y;
+        d[b] = mk<R>(R(0), R(0));
       }
     }
   }
@@ -691,9 +684,6 @@ __global__ void __launch_bounds__(kOuterThreads) k_outer(cplx<R>* __restrict__ p
     constexpr int NV = 2 * MB;
     __shared__ double red[kOuterThreads / 32][NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double w[NV];
-#pragma unroll
-    for (int b = 0; b < MB; ++b) { w[2 * b] = ar[b].value(); w[2 * b + 1] = ai[b].value(); }
     int o = 16;
 #pragma unroll
     for (int h = NV / 2; h; h >>= 1, o >>= 1) {
