@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <string>
 
 namespace {
 std::map<void*, size_t> blocks, pinned;
@@ -12,6 +13,12 @@ size_t live = 0, limit = (size_t)1 << 42;
 long countdown = -1;                     // allocations left before one fails (-1: none does)
 long pinned_calls = 0;
 int last = 0;
+// A clock for tests of what the library times: each launch advances it by the cost
+// of its kernel, the sum over the set patterns that the mangled name contains.  With
+// no cost set every interval is 1 ms.
+std::map<const void*, std::string> kernels;
+std::map<std::string, double> costs;
+double now = 0.0;
 
 int grab(std::map<void*, size_t>& m, void** p, size_t n) {
   *p = nullptr;
@@ -36,6 +43,7 @@ void fake_fail_after(long n) { countdown = n; }
 size_t fake_device_bytes() { return live; }
 size_t fake_pinned_blocks() { return pinned.size(); }
 long fake_pinned_calls() { return pinned_calls; }
+void fake_cost(const char* pattern, double ms) { costs[pattern] = ms; }
 
 int cudaMalloc(void** p, size_t n) {
   if (live + n > limit) { *p = nullptr; return last = 2; }
@@ -73,11 +81,14 @@ int cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned l
   *q = 0;
   return 0;
 }
-int cudaEventCreate(void** e) { *e = &last; return 0; }
-int cudaEventCreateWithFlags(void** e, unsigned) { *e = &last; return 0; }
-int cudaEventDestroy(void*) { return 0; }
-int cudaEventElapsedTime(float* ms, void*, void*) { *ms = 1.f; return 0; }
-int cudaEventRecord(void*, void*) { return 0; }
+int cudaEventCreate(void** e) { *e = new double(0.0); return 0; }
+int cudaEventCreateWithFlags(void** e, unsigned) { return cudaEventCreate(e); }
+int cudaEventDestroy(void* e) { delete static_cast<double*>(e); return 0; }
+int cudaEventElapsedTime(float* ms, void* a, void* b) {
+  *ms = costs.empty() ? 1.f : (float)(*static_cast<double*>(b) - *static_cast<double*>(a));
+  return 0;
+}
+int cudaEventRecord(void* e, void*) { *static_cast<double*>(e) = now; return 0; }
 int cudaEventRecordWithFlags(void*, void*, unsigned) { return 0; }
 int cudaEventSynchronize(void*) { return 0; }
 int cudaGraphDestroy(void*) { return 0; }
@@ -91,13 +102,18 @@ int cudaStreamDestroy(void*) { return 0; }
 int cudaStreamIsCapturing(void*, int* c) { *c = 0; return 0; }
 int cudaStreamSynchronize(void*) { return 0; }
 int cudaLaunchKernelExC(const void*, const void*, void**) { return 0; }
-int __cudaLaunchKernel(void*, Dim3, Dim3, void**, size_t, void*) { return 0; }
-int __cudaGetKernel(void** k, const void*) { *k = &last; return 0; }
+int __cudaLaunchKernel(void* k, Dim3, Dim3, void**, size_t, void*) {
+  for (const auto& c : costs) if (kernels[k].find(c.first) != std::string::npos) now += c.second;
+  return 0;
+}
+int __cudaGetKernel(void** k, const void* f) { *k = const_cast<void*>(f); return 0; }
 unsigned __cudaPushCallConfiguration(Dim3, Dim3, size_t, void*) { return 0; }
 int __cudaPopCallConfiguration(void*, void*, size_t* n, void*) { *n = 0; return 0; }
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
-void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*, void*, int*) {}
+void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, void*, void*, void*, void*, int*) {
+  kernels[f] = name;
+}
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 }

@@ -1,6 +1,6 @@
 """Host code of the library on a fake CUDA runtime (tests/fake_cudart.cc): the
 device memory a handle and its plans take against the server's admission bound,
-and plans after an allocation failed."""
+plans after an allocation failed, and what the autotuner picks from given times."""
 import glob
 import os
 import subprocess
@@ -36,6 +36,7 @@ L.fake_device_bytes.restype = ct.c_size_t
 L.fake_pinned_blocks.restype = ct.c_size_t
 L.fake_pinned_calls.restype = ct.c_long
 L.fake_fail_after.argtypes = [ct.c_long]
+L.fake_cost.argtypes = [ct.c_char_p, ct.c_double]
 def circuit(name, n, it):
     return circuits.to_gates(inputs.qft_circuit(n) if name == "qft" else inputs.grover_circuit(n, it, 1), per_member_flip=True)
 """
@@ -89,4 +90,30 @@ assert used <= bound, (used / B, bound / B)
 qs.qs_plan_destroy(p)
 qs.qs_destroy(h)
 assert L.fake_device_bytes() == 0
+""")
+
+
+# ms per pass by window width, from a start not yet written and from memory -> the width picked with a start pending
+# and without: start times within 1/16 of each other are decided by the others
+@pytest.mark.parametrize("start,memory,pending,loaded", [
+    ((1.0, 0.98, 0.99), (3.5, 4.5, 5.0), 10, 10),
+    ((1.0, 0.95, 0.99), (3.5, 4.5, 3.0), 12, 12),
+    ((1.0, 0.9, 0.8), (3.5, 4.5, 5.0), 12, 10),
+    ((1.0, 1.1, 1.2), (3.5, 3.0, 2.5), 10, 12),
+])
+def test_autotuned_width_from_a_pending_start(fake, start, memory, pending, loaded):
+    run(fake, f"""
+for m, s, d in zip((10, 11, 12), {start!r}, {memory!r}):
+    L.fake_cost(b"Li%dELb1EE" % m, s)                 # the pass kernels, M = m, START
+    L.fake_cost(b"Li%dELb0EE" % m, d)
+h = qs.qs_create(24, 2, 0, qs.QS_STATEVEC, qs.QS_C64)
+for start, want in ((True, {pending}), (False, {loaded})):
+    p = qs.qs_plan_create(h, circuit("qft", 24, 0)[:1])   # one pass at every width
+    if start:
+        qs.qs_set_basis_state(h, 5)
+    qs.qs_plan_autotune(p, 2, 0.01, 1, h)
+    assert qs.qs_plan_get_window(p, h) == want, (want, qs.qs_plan_get_window(p, h))
+    qs.qs_plan_run(p, 0.01, 1, 0, h)                  # no start is pending from here on
+    qs.qs_plan_destroy(p)
+qs.qs_destroy(h)
 """)
