@@ -112,25 +112,40 @@ def measured_peaks():
 
 
 def plan_source_hash():
+    """The sources of the kernels whose traffic is recorded: the passes, their starts, and k_outer."""
     h = hashlib.sha256()
-    for f in ("pass.cuh", "philox.cuh"):
+    for f in ("pass.cuh", "pass_start.cu", "plan.cu", "philox.cuh"):
         with open(os.path.join(ROOT, "paper_1412_2293_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def ncu_traffic(kind):
-    """DRAM bytes per launch from the committed ncu summary, if the kernel is unchanged."""
+def ncu_traffic(kind, workload, window):
+    """DRAM bytes per launch from the committed ncu summary, if that is of this workload and its kernels are unchanged."""
     path = os.path.join(ROOT, "profiles", "traffic.txt")
     try:
         with open(path) as f:
             t = json.load(f)
     except Exception:
         return None
-    if t.get("source_hash") != plan_source_hash():
+    if t.get("source_hash") != plan_source_hash() or t.get("workload") != workload or t.get("window") != window:
         return None
     v = t.get("kernels", {}).get(kind)
     return None if v is None else float(v)
+
+
+def dominant_pass(kinds, ms, outer):
+    """(kind, kernel, state writes) of the pass with the most time in a run from a basis start.
+
+    kinds: the run's launches in order; ms: their times by kind; outer: its last pass is the outer
+    product.  State writes: how often the pass moves the state, known where it creates all of it
+    (the outer product, or the only pass); None for a pass on part of the state or a dense one."""
+    passes = [k for k in kinds if k.startswith("pass")]
+    dom = max(set(passes), key=lambda k: sum(ms[k]))
+    alone = passes.count(dom) == 1 and passes[-1] == dom
+    if alone and outer:
+        return dom, "k_outer (with the window pass and the gather)", 1
+    return dom, "k_" + dom, 1 if len(passes) == 1 else None
 
 
 def workload_setup(name):
@@ -258,22 +273,22 @@ def run_ours(args, rank, world, local_rank):
     ev1.record(stream)
     torch.cuda.synchronize()
     ms_from_memory = ev0.elapsed_time(ev1) / 3
+    outer = launches > qs.qs_plan_info(p, h)[1]          # the gather and the outer product beside the pass
 
     # roofline of the dominant kernel (the fused pass with the most time).
     # Algorithmic bytes: a run from a basis start writes the state once, in the
-    # pass that completes its support; the passes before it touch 1 / 2^m of it.
+    # pass that completes its support.
     peaks, peak_src = measured_peaks()
     state_bytes = T * (1 << n) * esize
-    dom = max((k for k in kern if k.startswith("pass")), key=lambda k: sum(kern[k]))
+    dom, kernel, writes = dominant_pass(kinds, kern, outer)
     per_launch = {k: statistics.mean(v) for k, v in kern.items()}
-    bytes_per_pass = state_bytes
     avg_ms = statistics.mean(kern[dom])
-    achieved = bytes_per_pass / (avg_ms / 1e3) / 1e9
-    traffic = ncu_traffic(dom)
-    roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": round(achieved / peaks["hbm_gbs"], 4), "traffic": traffic,
-                "kernel": "k_pass_high" if dom == "pass_high" else "k_outer (with the window pass and the gather)",
-                "algorithmic_bytes_per_launch": bytes_per_pass, "avg_launch_ms": round(avg_ms, 4),
+    achieved = None if writes is None else writes * state_bytes / (avg_ms / 1e3) / 1e9
+    roofline = {"bound": "hbm", "achieved": None if achieved is None else round(achieved, 1), "peak": peaks["hbm_gbs"],
+                "unit": "GB/s", "frac": None if achieved is None else round(achieved / peaks["hbm_gbs"], 4),
+                "traffic": ncu_traffic(dom, args.workload, window), "kernel": kernel,
+                "algorithmic_bytes_per_launch": None if writes is None else writes * state_bytes,
+                "avg_launch_ms": round(avg_ms, 4),
                 "peak_source": f"{peak_src} hbm_gbs (copy bandwidth)",
                 "launch_ms_by_kind": {k: round(v, 4) for k, v in per_launch.items()}}
 
