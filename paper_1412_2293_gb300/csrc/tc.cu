@@ -157,8 +157,15 @@ __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__flo
 //           write each to its row of A; the results go back the same way through
 //           A's space once the MMAs are done: 0.42 ms, as scattered targets.
 enum : int { kPlain = 0, kPairs = 1, kRows = 2 };
+// Blocks per SM the registers are limited for (0: the compiler's choice).  Left to
+// itself it took 64 registers for k = 3 and 128 for k = 4 kPlain and spilled, for an
+// eighth and a fourth block that HBM has no use for: scattered targets of 8 GiB, k =
+// 3 3.15-3.21 ms for 3.03-3.07 with 7 blocks (3.03-3.18 before this kernel had
+// modes), k = 4 3.13-3.25 for 3.04-3.14 with 3.  kPairs at k = 4 is faster with four blocks (3.17
+// for 3.25), k = 5 (two blocks by shared memory) with the compiler's registers.
+constexpr int tc_blocks(int k, int mode) { return k == 3 ? 7 : (k == 4 && mode != kPairs ? 3 : 0); }
 template <int K, int MODE>
-__global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
+__global__ void __launch_bounds__(kTcThreads, tc_blocks(K, MODE)) k_dense_tc(TcArgs args) {
   constexpr bool VEC = MODE != kPlain;
   constexpr int D = 1 << K;             // amplitudes per group
   constexpr int KD = 2 * D;             // MMA K (real columns) and N (real rows of B)
@@ -226,16 +233,16 @@ __global__ void __launch_bounds__(kTcThreads) k_dense_tc(TcArgs args) {
   // and stored, the next tile's loads land in the other
   float2 xa[D], xb[D];
   auto load = [&](float2 (&x)[D], const float2* p) {
+    if constexpr (VEC) {
 #pragma unroll
-    for (int j = 0; j < D; j += 2) {
-      if constexpr (VEC) {
+      for (int j = 0; j < D; j += 2) {
         const float4 v = *reinterpret_cast<const float4*>(p + (MODE == kRows ? args.step_off[j / 2] : args.off_j[j]));
         x[j] = make_float2(v.x, v.y);
         x[j + 1] = make_float2(v.z, v.w);
-      } else {
-        x[j] = p[args.off_j[j]];
-        x[j + 1] = p[args.off_j[j + 1]];
       }
+    } else {
+#pragma unroll
+      for (int j = 0; j < D; ++j) x[j] = p[args.off_j[j]];
     }
   };
   if (t < args.tiles) load(xa, args.psi + base);
