@@ -934,8 +934,10 @@ constexpr float kRefined = 3e-5f;        // largest |Z| (Frobenius) refine() tak
 // Q - I) when the correction is not small, |Z| >= kRefined, or the
 // couplings left in tie clusters are not small against the other gaps: delta
 // converges by those two ratios.
-// Buffers: Q -> the refined basis in Y (swapped by the caller), P, Z FP64; f32 five
-// M x kJP FP32 matrices.  lam: the eigenvalues.
+// Q's entries are multiples of 2^-26 (quantum), so R is exact, and the refined
+// basis is left as Q and the correction Q Z in Y, 2^-53 of which is at most 2^-68:
+// a rounding of it in FP64 would be the same for every row of L.
+// Buffers: P, Z FP64; f32 five M x kJP FP32 matrices.  lam: the eigenvalues.
 template <typename T, typename T32>
 __device__ bool refine(const double2* G, const T* Q, T* Y, T* P, T* Z, T32* f32, int M, double* lam) {
   __shared__ double dD[kMaxGramDim], dR[kMaxGramDim];
@@ -1098,19 +1100,39 @@ __device__ bool refine(const double2* G, const T* Q, T* Y, T* P, T* Z, T32* f32,
     }
     __syncthreads();
   }
-  for (int i = tid; i < MM; i += kEigThreads) {           // Y = Q + Q Z
+  for (int i = tid; i < MM; i += kEigThreads) {           // Y = Q Z
     const int r = i / M, c = i % M;
-    T acc = Q[r * kJP + c];
+    T acc = tscal<T>(0.0);
     for (int k = 0; k < M; ++k) acc = cmacc(Q[r * kJP + k], Z[k * kJP + c], acc);
     Y[r * kJP + c] = acc;
   }
   __syncthreads();
   return true;
 }
+
+// The nearest multiple of 2^-26 (|x| < 2^25): products of two such numbers of at
+// most 1 are multiples of 2^-52, and so are their sums: exact in FP64.
+__device__ __forceinline__ double quantum(double x) { return __dadd_rn(__dadd_rn(x, 0x1.8p26), -0x1.8p26); }
+__device__ __forceinline__ double2 quantum(double2 x) { return make_double2(quantum(x.x), quantum(x.y)); }
+
+// An eigenbasis in columns (pitch kJP): hi, or hi + lo with hi in multiples of 2^-26
+// (lo null: hi alone); sum: rounded to FP64.  unit: the columns' norms are off by
+// the roundings of the FP64 Jacobi.
+template <typename T> struct Basis { T *hi, *lo, *sum; bool unit; };
+
+// (hi + lo) u for the phase u, unit to FP64's rounding: u too is split at 2^-26, its
+// norm's error, found exactly, goes into the low part.
+__device__ __forceinline__ void turn(double hi, double lo, double u, double* bh, double* bl) { *bh = hi * u; *bl = lo * u; }
+__device__ __forceinline__ void turn(double2 hi, double2 lo, double2 u, double2* bh, double2* bl) {
+  const double2 uq = quantum(u), ul = make_double2(u.x - uq.x, u.y - uq.y);
+  const double off = fma(uq.x, uq.x, fma(uq.y, uq.y, -1.0)) + fma(2.0 * uq.x + ul.x, ul.x, (2.0 * uq.y + ul.y) * ul.y);
+  *bh = cmacc(hi, uq, make_double2(0.0, 0.0));
+  *bl = cmacc(hi, ul, cmacc(lo, u, make_double2(-0.5 * off * bh->x, -0.5 * off * bh->y)));
+}
 // After the eigensolver: eigenvalues lam sorted descending (ties keep index
 // order), clusters of ties given a canonical basis, and the outputs W = first
-// keep canonical eigenvectors (in `basis`, columns, pitch kJP; M x keep complex
-// in Wout), lam_out (sorted), keep and the scale.  T is double (real G: real
+// keep canonical eigenvectors (basis + low, columns, pitch kJP; rounded, M x keep
+// complex, in W), lam_out (sorted), keep and the scale.  T is double (real G: real
 // eigenvectors, real arithmetic) or double2.  Candidate j of a cluster with
 // eigenvectors S is P e_j, P = S S^dagger, minus its components along the
 // cluster's accepted vectors q_t; as the q_t lie in range(P),
@@ -1120,12 +1142,13 @@ __device__ bool refine(const double2* G, const T* Q, T* Y, T* P, T* Z, T32* f32,
 // basis (from the index of its first eigenvalue on), so the clusters are shared
 // out over the warps (lane = row).
 template <typename T>
-__device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, int r, int normalize, double unscale,
+__device__ void eig_finish(const Basis<T> Q, T* basis, T* low, const double* lam_in, int M, int r, int normalize, double unscale,
                            double* __restrict__ W, double* __restrict__ lam_out, int* keep_out, double* scale_out,
                            int* status) {
   __shared__ int order[kMaxGramDim + 1], start[kMaxGramDim + 1], nclusters;
   __shared__ double lam[kMaxGramDim];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = kEigThreads / 32;
+  const T* V = Q.sum;
   // descending, ties in index order: position of i = how many come before it
   for (int i = tid; i < M; i += blockDim.x) {
     int pos = 0;
@@ -1134,7 +1157,7 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
     lam[pos] = lam_in[i];
   }
   const int keep = r < M ? r : M;
-  for (int i = tid; i < M * kJP; i += blockDim.x) basis[i] = tscal<T>(0.0);
+  for (int i = tid; i < M * kJP; i += blockDim.x) basis[i] = low[i] = tscal<T>(0.0);
   __syncthreads();
   const double lam1 = lam[0] > 0.0 ? lam[0] : 0.0;
   if (tid == 0) {
@@ -1161,7 +1184,22 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
       const unsigned ok = __ballot_sync(0xffffffffu, lane < M && tabs2(vl) > kGsAccept * kGsAccept);
       if (ok) {
         const T ph = unit_phase(V[(__ffs(ok) - 1) * kJP + col]);
-        if (lane < M) basis[lane * kJP + i0] = tmul(vl, ph);
+        T b = tscal<T>(0.0), bl = b;
+        if (lane < M) {
+          if (Q.lo) turn(Q.hi[lane * kJP + col], Q.lo[lane * kJP + col], ph, &b, &bl);
+          else b = tmul(vl, ph);
+        }
+        if (Q.unit) {                                      // the norm's error into the low part
+          double n2 = lane < M ? tabs2(b) : 0.0;
+          if (lane == 0) n2 -= 1.0;
+#pragma unroll
+          for (int o = 16; o; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+          bl = tscale(b, -0.5 * n2);
+        }
+        if (lane < M) {
+          basis[lane * kJP + i0] = b;
+          low[lane * kJP + i0] = bl;
+        }
         continue;
       }
     }
@@ -1210,7 +1248,7 @@ __device__ void eig_finish(const T* V, T* basis, const double* lam_in, int M, in
   // outputs
   for (int i = tid; i < M * keep; i += blockDim.x) {
     const int p = i / keep, c = i % keep;
-    const T v = basis[p * kJP + c];
+    const T v = tadd(basis[p * kJP + c], low[p * kJP + c]);
     if constexpr (sizeof(T) == 16) {
       W[2 * (p * keep + c)] = v.x;
       W[2 * (p * keep + c) + 1] = v.y;
@@ -1233,11 +1271,11 @@ constexpr size_t kEigMat = (size_t)kMaxGramDim * kJP;
 constexpr int kEigSmem = (int)(kEigMat * (5 * sizeof(double2) + 5 * sizeof(float2)));
 constexpr float kTol32 = 3e-7f;
 
-// Eigenvalues lam and eigenvectors (columns of *Qp) of G; see eig_member.
+// Eigenvalues lam and eigenvectors of G; see eig_member.  Q, Y, P, Z: matrices; G's
+// space may hold the basis afterwards.
 template <typename T, typename T32>
-__device__ void eig_vectors(const double2* G, T** Qp, T** Yp, T* P, T* Z, T32* f32, int M, double* lam, int* status) {
+__device__ Basis<T> eig_vectors(double2* G, T* Q, T* Y, T* P, T* Z, T32* f32, int M, double* lam, int* status) {
   T32 *A32 = f32, *V32 = f32 + kEigMat;
-  T *Q = *Qp, *Y = *Yp;
   const int tid = threadIdx.x, MM = M * M;
   for (int i = tid; i < MM; i += kEigThreads) {
     const int p = i / M, q = i % M;
@@ -1246,13 +1284,17 @@ __device__ void eig_vectors(const double2* G, T** Qp, T** Yp, T* P, T* Z, T32* f
   }
   __syncthreads();
   jacobi<T32>(A32, V32, M, kTol32, kJacobiSweeps32);    // not converging here only costs FP64 sweeps
-  for (int i = tid; i < MM; i += kEigThreads) Q[(i / M) * kJP + i % M] = to64(V32[(i / M) * kJP + i % M]);
+  for (int i = tid; i < MM; i += kEigThreads) Q[(i / M) * kJP + i % M] = quantum(to64(V32[(i / M) * kJP + i % M]));
   __syncthreads();
   if (refine<T, T32>(G, Q, Y, P, Z, f32, M, lam)) {
-    T* t = Q;
-    Q = Y;
-    Y = t;
-  } else {
+    T* S = reinterpret_cast<T*>(G);
+    for (int i = tid; i < MM; i += kEigThreads) {
+      const int at = (i / M) * kJP + i % M;
+      S[at] = tadd(Q[at], Y[at]);
+    }
+    return Basis<T>{Q, Y, S, false};
+  }
+  {
     for (int i = tid; i < MM; i += kEigThreads) {          // Z = -R / 2 + 3 R^2 / 8 (R^2 in FP32: it is 1e-12)
       const int rr = i / M, c = i % M;
       T32 acc = tscal<T32>(0.0);
@@ -1291,8 +1333,7 @@ __device__ void eig_vectors(const double2* G, T** Qp, T** Yp, T* P, T* Z, T32* f
     __syncthreads();
     for (int i = tid; i < M; i += kEigThreads) lam[i] = tre(Y[i * kJP + i]);
   }
-  *Qp = Q;
-  *Yp = Y;
+  return Basis<T>{Q, nullptr, Q, true};
 }
 
 // Eigendecomposition of G (Hermitian, M x M, in shared memory, scaled to a
@@ -1301,10 +1342,10 @@ __device__ void eig_vectors(const double2* G, T** Qp, T** Yp, T* P, T* Z, T32* f
 // products.  Where it declines (close eigenvalues outside a tie cluster, as the
 // symmetric noise of Grover's search makes them) the basis is made orthonormal,
 // Q (I - R / 2 + 3 R^2 / 8) with R = Q^dagger Q - I (an error of |R|^3, 1e-18), and
-// the FP64 Jacobi takes Q^dagger G Q, nearly diagonal by then.  Returns the kept
-// canonical eigenvectors (columns, pitch kJP, shared memory).
+// the FP64 Jacobi takes Q^dagger G Q, nearly diagonal by then.  The kept canonical
+// eigenvectors are *basis + *low (columns, pitch kJP, shared memory).
 template <typename T, typename T32>
-__device__ T* eig_member(double2* G, bool diagonal, int M, int r, int normalize, double unscale, double* __restrict__ W,
+__device__ void eig_member(T** basis, T** low, double2* G, bool diagonal, int M, int r, int normalize, double unscale, double* __restrict__ W,
                          double* __restrict__ lam_out, int* keep, double* scale, int* status) {
   __shared__ double lam[kMaxGramDim];
   T* Q = reinterpret_cast<T*>(G + kEigMat);
@@ -1313,6 +1354,7 @@ __device__ T* eig_member(double2* G, bool diagonal, int M, int r, int normalize,
   T* Z = reinterpret_cast<T*>(G + 4 * kEigMat);
   T32* f32 = reinterpret_cast<T32*>(G + 5 * kEigMat);
   const int tid = threadIdx.x, MM = M * M;
+  Basis<T> B{Q, nullptr, Q, false};
   if (diagonal) {
     for (int i = tid; i < MM; i += kEigThreads) {
       const int p = i / M, q = i % M;
@@ -1320,11 +1362,12 @@ __device__ T* eig_member(double2* G, bool diagonal, int M, int r, int normalize,
       if (p == q) lam[p] = G[p * kJP + p].x;
     }
   } else {
-    eig_vectors<T, T32>(G, &Q, &Y, P, Z, f32, M, lam, status);
+    B = eig_vectors<T, T32>(G, Q, Y, P, Z, f32, M, lam, status);
   }
   __syncthreads();
-  eig_finish<T>(Q, P, lam, M, r, normalize, unscale, W, lam_out, keep, scale, status);
-  return P;
+  eig_finish<T>(B, P, Z, lam, M, r, normalize, unscale, W, lam_out, keep, scale, status);
+  *basis = P;
+  *low = Z;
 }
 
 // Where k_eig_truncate takes its Gram matrices from: the members' blocks
@@ -1452,14 +1495,17 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_truncate(double* __restrict
     if (i / M != i % M) offdiag |= above(G[(i / M) * kJP + i % M], thr);
   const bool diagonal = !__syncthreads_or(offdiag) && scaled;
   double *W = base + kSmallW, *lam = base + kSmallLam, *scale = base + kSmallScale;
-  double2* basis_c = nullptr;
-  double* basis_r = nullptr;
-  if (cplx) basis_c = eig_member<double2, float2>(G, diagonal, M, r, normalize, unscale, W, lam, rc.keep + b, scale, status);
-  else basis_r = eig_member<double, float>(G, diagonal, M, r, normalize, unscale, W, lam, rc.keep + b, scale, status);
+  double2 *basis_c = nullptr, *low_c = nullptr;
+  double *basis_r = nullptr, *low_r = nullptr;
+  if (cplx) eig_member<double2, float2>(&basis_c, &low_c, G, diagonal, M, r, normalize, unscale, W, lam, rc.keep + b, scale, status);
+  else eig_member<double, float>(&basis_r, &low_r, G, diagonal, M, r, normalize, unscale, W, lam, rc.keep + b, scale, status);
   if (src.form == 0) return;
   __threadfence_block();
   __syncthreads();
-  // V_ij = scale sum_a (E_a)_ij W_a, [ij][p][c]
+  // V_ij = scale sum_a (E_a)_ij W_a, [ij][p][c], the small terms first: V's rounding
+  // is the same for every row of L, and with W rounded before it the trace of a channel
+  // that truncates nothing was off by 2.7e-16 (rms, random factors of 1 to 8 columns;
+  // 1.7e-16 through L', now 1.1e-16, for 1.7 us more a channel)
   const int keep = r < M ? r : M;
   const double sc = normalize ? *(volatile double*)scale : 1.0;
   const int nv = diag ? D : D * D;
@@ -1468,11 +1514,15 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_truncate(double* __restrict
     const int c = i % keep, p = (i / keep) % m, ij = i / (keep * m);
     const int at = diag ? ij * D + ij : ij;
     double2 acc = make_double2(0.0, 0.0);
-    for (int a = 0; a < K; ++a) {
-      const int row = (a * m + p) * kJP + c;
-      const double2 w = cplx ? basis_c[row] : make_double2(basis_r[row], 0.0);
-      if (src.real) acc.x = fma(sE[a * D * D + at].x, w.x, acc.x);
-      else acc = cmacc(sE[a * D * D + at], w, acc);
+    for (int part = 0; part < 2; ++part) {
+      const double2* wc = part ? basis_c : low_c;
+      const double* wr = part ? basis_r : low_r;
+      for (int a = K - 1; a >= 0; --a) {
+        const int row = (a * m + p) * kJP + c;
+        const double2 w = cplx ? wc[row] : make_double2(wr[row], 0.0);
+        if (src.real) acc.x = fma(sE[a * D * D + at].x, w.x, acc.x);
+        else acc = cmacc(sE[a * D * D + at], w, acc);
+      }
     }
     if (src.real) V[i] = acc.x * sc;
     else { V[2 * i] = acc.x * sc; V[2 * i + 1] = acc.y * sc; }
