@@ -2139,11 +2139,11 @@ qs_status run_plan(qs_plan p, double e, uint64_t seed, uint64_t gate_id0, int wa
 // result does not depend on how many share its launch.  The outer product adds
 // two launches (about 10 us) and saves the pass's arithmetic, 3 ps an amplitude in
 // complex64 and 80 in complex128, and the pass's chain of FP64 latencies on tiles
-// beyond one a warp.  From 17 (14) qubits: QFT of 17, 1024 complex64 members 555 ->
-// 359 us, one 72 -> 77, four 71 -> 85; 14, 75 complex128 members 207 -> 170, one 148 ->
-// 159; at 16, 1024 members 354 -> 308 but four 63 -> 85, at 13 complex128, 75 members
-// 148 -> 171.
-int outer_qubits(size_t esize) { return esize == 8 ? 17 : 14; }
+// beyond one a warp.  From 17 (12) qubits, where it loses least either way, against
+// the pass on every tile: QFT of 17, one complex64 member 71 -> 83 us, 1024 555 -> 356;
+// of 16, 1024 members 368 -> 282 but up to 32 of them 62-71 -> 78-84; of 12 in
+// complex128, up to 32 members 138-145 -> 146-158, 256 228 -> 194, 1024 677 -> 472.
+int outer_qubits(size_t esize) { return esize == 8 ? 17 : 12; }
 void find_start(qs_plan p) {
   p->start_full = -1;
   p->start_outer = false;

@@ -47,6 +47,7 @@ def run_qft(n, batch, dtype, m, per_member, ref, take):
     (17, 1, 33, qs.QS_C64, 10, False),
     (17, 3, 514, qs.QS_C64, 12, True),       # window states of 513 members and more: two turns
     (18, 2, 20, qs.QS_C64, 11, False),
+    (12, 2, 300, qs.QS_C128, 10, False),
     (13, 2, 33, qs.QS_C128, 10, False),
     (14, 3, 1025, qs.QS_C128, 10, True),     # two turns
     (15, 2, 9, qs.QS_C128, 10, True),
