@@ -268,7 +268,7 @@ qs_status rank_apply_kraus(qs_handle h, const int* targets, int k, const std::ve
   for (const auto& E : ks) diag &= is_diagonal(E, d);
   int max_M, max_keep;
   advance_counts(h, K, 0, &max_M, &max_keep);
-  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, Edev, K, 0, qs::KrausGate{}, max_cols, max_keep, h->normalize));
+  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, Edev, K, qs::KrausGate{}, max_cols, max_keep, h->normalize));
   return QS_OK;
 }
 
@@ -289,7 +289,7 @@ qs_status rank_channel_gate(qs_handle h, const int* targets, const qs::KrausGate
   const bool diag = g.noise == QS_NOISE_PHASE && qs::gate_diagonal(g.U, g.k);
   int max_M, max_keep;
   advance_counts(h, K, 0, &max_M, &max_keep);
-  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, nullptr, K, 0, g, max_cols, max_keep, h->normalize));
+  QS_CUDA(h, qs::launch_rank_channel(h, tg, h->real_factor, diag, nullptr, K, g, max_cols, max_keep, h->normalize));
   return QS_OK;
 }
 

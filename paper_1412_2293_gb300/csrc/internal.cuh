@@ -251,11 +251,11 @@ inline int kraus_count(int k, int noise) { return noise == QS_NOISE_ROTATION && 
 cudaError_t launch_gram(qs_ctx* h, bool real, int max_M);
 cudaError_t launch_eig_truncate(qs_ctx* h, int trunc_r, int normalize);
 cudaError_t launch_project(qs_ctx* h, bool real, int K, int max_keep);
-// A whole channel (K Kraus operators, member b's at E + b e_stride, e_stride = 0:
-// shared; or g's averaged set when g.k > 0) with truncation to the members' ranks.  diag: every operator is diagonal.
+// A whole channel (the K Kraus operators at E, or g's averaged set when g.k > 0)
+// with truncation to the members' ranks.  diag: every operator is diagonal.
 // One-qubit and diagonal channels never form L' (k_moments, k_project_fused).
 cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool diag, const double* E_dev, int K,
-                                int e_stride, const KrausGate& g, int max_cols, int max_keep, int normalize);
+                                const KrausGate& g, int max_cols, int max_keep, int normalize);
 bool gate_diagonal(const double* U, int k);   // U (2^k x 2^k interleaved) has no off-diagonal entry
 int rank_counters();                          // words of h->rcounters per member
 int gram_rows_per_block(int n);

@@ -1973,7 +1973,7 @@ qs_status run_rank_ops(qs_plan p) {
         kg.e_run = &p->d_run->e;
         const int K = kraus_count(g.k, g.noise);
         const bool diag = g.noise == QS_NOISE_PHASE && gate_diagonal(g.U, g.k);
-        e = launch_rank_channel(h, tg, real, diag, nullptr, K, 0, kg, h->rank, p->rank_kmax, normalize);
+        e = launch_rank_channel(h, tg, real, diag, nullptr, K, kg, h->rank, p->rank_kmax, normalize);
       }
     }
     if (e != cudaSuccess) return pfail(p, QS_ERR_CUDA, std::string("fixed-rank plan: ") + cudaGetErrorString(e));

@@ -75,14 +75,14 @@ __device__ double2 kraus_entry(const KrausGate& g, double e, int op, int row, in
 }
 
 // Lp_b[a m_b + c] = E_a L_b[c] for member b = blockIdx.y; one thread per
-// (group, column) of a two-qubit channel.  The member's Kraus operators are E + b e_stride (e_stride
-// = 0: one set for every member).  Block (0, b) records M_b = K m_b.  REAL: L
-// and the E_a are real (imaginary parts zero), real arithmetic.
+// (group, column) of a two-qubit channel.  The Kraus operators are E, or the gate's
+// at the member's noise level.  Block (0, b) records M_b = K m_b.  REAL: L and the
+// E_a are real (imaginary parts zero), real arithmetic.
 template <typename R, bool REAL>
 __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __restrict__ L,
                                                             cplx<R>* __restrict__ Lp, int n, int rcap, int mcap,
                                                             Targets tg, const double* __restrict__ E, int K,
-                                                            int e_stride, RankCounts rc, const KrausGate g) {
+                                                            RankCounts rc, const KrausGate g) {
   using C = cplx<R>;
   constexpr int D = 4;
   __shared__ C sE[8 * D * D];
@@ -95,8 +95,7 @@ __global__ void __launch_bounds__(kExpBlock) k_kraus_expand(const cplx<R>* __res
       sE[i] = mk<R>((R)v.x, (R)v.y);
     }
   } else {
-    const double* Eb = E + (size_t)b * e_stride;
-    for (int i = threadIdx.x; i < K * D * D; i += blockDim.x) sE[i] = mk<R>((R)Eb[2 * i], (R)Eb[2 * i + 1]);
+    for (int i = threadIdx.x; i < K * D * D; i += blockDim.x) sE[i] = mk<R>((R)E[2 * i], (R)E[2 * i + 1]);
   }
   const int m = rc.cols[b];
   if (blockIdx.x == 0 && threadIdx.x == 0) rc.M[b] = K * m;
@@ -1600,14 +1599,14 @@ unsigned rows_blocks(uint64_t rows, int members) {
 }
 
 template <typename R>
-cudaError_t expand_launch(qs_ctx* h, const Targets& tg, bool real, const double* E, int K, int e_stride,
+cudaError_t expand_launch(qs_ctx* h, const Targets& tg, bool real, const double* E, int K,
                             int max_cols, const KrausGate& g) {
   const uint64_t work = ((1ull << h->n) >> 2) * (uint64_t)max_cols;
   const dim3 grid(rows_blocks(work, h->batch), h->batch);
   auto* l = static_cast<const cplx<R>*>(h->state);
   auto* lp = static_cast<cplx<R>*>(h->work);
-  if (real) k_kraus_expand<R, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, e_stride, h->rc, g);
-  else k_kraus_expand<R, false><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, e_stride, h->rc, g);
+  if (real) k_kraus_expand<R, true><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, h->rc, g);
+  else k_kraus_expand<R, false><<<grid, kExpBlock, 0, h->stream>>>(l, lp, h->n, h->rank, h->mcap, tg, E, K, h->rc, g);
   return cudaGetLastError();
 }
 
@@ -1681,7 +1680,7 @@ cudaError_t launch_eig_truncate(qs_ctx* h, int trunc_r, int normalize) {
 namespace {
 // moments, eigensolver and projection of a one-qubit or diagonal channel
 template <typename R, bool REAL, int KQ, bool DIAG>
-cudaError_t channel_launch(qs_ctx* h, const Targets& tg, const double* E, int K, int e_stride, const KrausGate& g,
+cudaError_t channel_launch(qs_ctx* h, const Targets& tg, const double* E, int K, const KrausGate& g,
                            int max_cols, int max_keep, int normalize) {
   constexpr int D = 1 << KQ, CB = 4;
   const MomSplit sp = mom_split(h->n, KQ);
@@ -1697,7 +1696,7 @@ cudaError_t channel_launch(qs_ctx* h, const Targets& tg, const double* E, int K,
   src.estride = mom_stride(h->rank);
   src.partials = h->partials;
   src.E = g.k > 0 ? h->rsmall + kSmallE : E;             // a gate's set: written by k_moments
-  src.e_stride = g.k > 0 ? kRankStride : e_stride;
+  src.e_stride = g.k > 0 ? kRankStride : 0;
   src.real = REAL ? 1 : 0;
   k_eig_truncate<<<h->batch, kEigThreads, kEigSmem, h->stream>>>(h->rsmall, kRankStride, h->rc, 0, normalize, h->dstatus + 1,
                                                                  src);
@@ -1712,11 +1711,11 @@ cudaError_t channel_launch(qs_ctx* h, const Targets& tg, const double* E, int K,
 }
 
 template <typename R, bool REAL>
-cudaError_t channel_form(qs_ctx* h, const Targets& tg, bool diag, const double* E, int K, int e_stride, const KrausGate& g,
+cudaError_t channel_form(qs_ctx* h, const Targets& tg, bool diag, const double* E, int K, const KrausGate& g,
                          int max_cols, int max_keep, int normalize) {
-  if (tg.k == 2) return channel_launch<R, REAL, 2, true>(h, tg, E, K, e_stride, g, max_cols, max_keep, normalize);
-  if (diag) return channel_launch<R, REAL, 1, true>(h, tg, E, K, e_stride, g, max_cols, max_keep, normalize);
-  return channel_launch<R, REAL, 1, false>(h, tg, E, K, e_stride, g, max_cols, max_keep, normalize);
+  if (tg.k == 2) return channel_launch<R, REAL, 2, true>(h, tg, E, K, g, max_cols, max_keep, normalize);
+  if (diag) return channel_launch<R, REAL, 1, true>(h, tg, E, K, g, max_cols, max_keep, normalize);
+  return channel_launch<R, REAL, 1, false>(h, tg, E, K, g, max_cols, max_keep, normalize);
 }
 }  // namespace
 
@@ -1728,12 +1727,12 @@ bool gate_diagonal(const double* U, int k) {
   return true;
 }
 
-cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool diag, const double* E, int K, int e_stride,
+cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool diag, const double* E, int K,
                                 const KrausGate& g, int max_cols, int max_keep, int normalize) {
   if (tg.k == 2 && !diag) {                              // through L'
     const int max_M = std::min(kMaxGramDim, K * max_cols);
-    cudaError_t e = h->dtype == QS_C64 ? expand_launch<float>(h, tg, real, E, K, e_stride, max_cols, g)
-                                       : expand_launch<double>(h, tg, real, E, K, e_stride, max_cols, g);
+    cudaError_t e = h->dtype == QS_C64 ? expand_launch<float>(h, tg, real, E, K, max_cols, g)
+                                       : expand_launch<double>(h, tg, real, E, K, max_cols, g);
     if (e == cudaSuccess) e = launch_gram(h, real, max_M);
     if (e == cudaSuccess) e = launch_eig_truncate(h, 0, normalize);
     if (e == cudaSuccess) e = launch_project(h, real, K, max_keep);
@@ -1741,10 +1740,10 @@ cudaError_t launch_rank_channel(qs_ctx* h, const Targets& tg, bool real, bool di
   }
   const cudaError_t e = rank_kernel_attributes();
   if (e != cudaSuccess) return e;
-  if (h->dtype == QS_C64 && real) return channel_form<float, true>(h, tg, diag, E, K, e_stride, g, max_cols, max_keep, normalize);
-  if (h->dtype == QS_C64) return channel_form<float, false>(h, tg, diag, E, K, e_stride, g, max_cols, max_keep, normalize);
-  if (real) return channel_form<double, true>(h, tg, diag, E, K, e_stride, g, max_cols, max_keep, normalize);
-  return channel_form<double, false>(h, tg, diag, E, K, e_stride, g, max_cols, max_keep, normalize);
+  if (h->dtype == QS_C64 && real) return channel_form<float, true>(h, tg, diag, E, K, g, max_cols, max_keep, normalize);
+  if (h->dtype == QS_C64) return channel_form<float, false>(h, tg, diag, E, K, g, max_cols, max_keep, normalize);
+  if (real) return channel_form<double, true>(h, tg, diag, E, K, g, max_cols, max_keep, normalize);
+  return channel_form<double, false>(h, tg, diag, E, K, g, max_cols, max_keep, normalize);
 }
 
 cudaError_t launch_project(qs_ctx* h, bool real, int K, int max_keep) {

@@ -113,7 +113,7 @@ __device__ __forceinline__ void noise_matrix(R* o, int k, const DMat& U, int noi
         o[2 * r + 1] = (R)im;
       }
     } else {
-        for (int r = 0; r < d; ++r) {
+      for (int r = 0; r < d; ++r) {
         for (int cc = 0; cc < d; ++cc) {
           double re = U.v[2 * (r * d + cc)], im = U.v[2 * (r * d + cc) + 1];
           if (cc == d - 1) {
