@@ -417,7 +417,8 @@ qs_status qs_plan_get_config(qs_plan p, int* low_cfg, int* high_cfg);
  * state; a basis start set before the call (qs_set_basis_state(s)) is
  * created by the first pass of every profiled run, so the passes are timed
  * as the plan's runs from that start will execute them, and it is still the
- * pending start afterwards.  Synchronises. */
+ * pending start afterwards.  Where a reference is stored the last pass is timed
+ * as qs_plan_run_fidelity runs it.  Synchronises. */
 qs_status qs_plan_autotune(qs_plan p, int reps, double e, uint64_t seed, double* best_ms);
 
 /* ------------------------------------------------------------ utilities */

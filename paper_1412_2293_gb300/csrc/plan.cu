@@ -2538,8 +2538,10 @@ qs_status qs_plan_run_fidelity(qs_plan p, double e, uint64_t seed, uint64_t gate
   return read_results(h, out, h->batch);
 }
 
-qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t gate_id0, double* ms,
-                          int* kinds, int cap, int* count) {
+namespace {
+// fid: the last pass reduces the fidelity with the stored reference
+qs_status profile_runs(qs_plan p, int reps, double e, uint64_t seed, uint64_t gate_id0, int fid, double* ms, int* kinds,
+                       int cap, int* count) {
   if (!p || reps < 1 || !ms || !kinds || !count) return QS_ERR_INVALID_ARG;
   qs_ctx* h = p->h;
   // a pending basis start is created by the first pass of every profiled run,
@@ -2585,7 +2587,8 @@ qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t
         cudaError_t x = f32 ? launch_precompute<float>(p, P, mode, h->stream) : launch_precompute<double>(p, P, mode, h->stream);
         cudaEventRecord(ev[k++], h->stream);
         kind[li++] = 0;
-        if (x == cudaSuccess) x = f32 ? launch_pass_kernel<float>(p, P, h->stream, mode, 0) : launch_pass_kernel<double>(p, P, h->stream, mode, 0);
+        const int fd = si + 1 == p->steps.size() ? fid : 0;
+        if (x == cudaSuccess) x = f32 ? launch_pass_kernel<float>(p, P, h->stream, mode, fd) : launch_pass_kernel<double>(p, P, h->stream, mode, fd);
         cudaEventRecord(ev[k++], h->stream);
         kind[li++] = P.high ? 2 : 1;
         if (x != cudaSuccess) { result = pfail(p, QS_ERR_CUDA, cudaGetErrorString(x)); break; }
@@ -2615,6 +2618,12 @@ qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t
   }
   for (auto& x : ev) cudaEventDestroy(x);
   return result;
+}
+}  // namespace
+
+qs_status qs_plan_profile(qs_plan p, int reps, double e, uint64_t seed, uint64_t gate_id0, double* ms,
+                          int* kinds, int cap, int* count) {
+  return profile_runs(p, reps, e, seed, gate_id0, 0, ms, kinds, cap, count);
 }
 
 namespace {
@@ -2703,8 +2712,8 @@ qs_status qs_plan_get_window(qs_plan p, int* m) {
 namespace {
 // Best low and high configurations of the plan's current window width: the
 // time of the low and high passes of one run under each, averaged over reps
-// profiled runs; total = the whole run under the chosen pair.
-qs_status tune_configs(qs_plan p, int reps, double e, uint64_t seed, int* bl, int* bh, double* low_best,
+// profiled runs; total = the whole run under the chosen pair.  fid: see profile_runs.
+qs_status tune_configs(qs_plan p, int reps, double e, uint64_t seed, int fid, int* bl, int* bh, double* low_best,
                        double* high_best, double* total) {
   const int nl = num_low_cfgs(p->h->esize, p->m), nh = num_high_cfgs(p->h->esize, p->m);
   const int ncfg = std::max(nl, nh);
@@ -2718,11 +2727,11 @@ qs_status tune_configs(qs_plan p, int reps, double e, uint64_t seed, int* bl, in
     const int pend = p->h->pending;
     const uint64_t pend_x = p->h->pending_x;
     // one untimed run first: a kernel's first launch also loads its module
-    st = qs_plan_profile(p, 1, e, seed, 0, ms.data(), kinds.data(), (int)ms.size(), &count);
+    st = profile_runs(p, 1, e, seed, 0, fid, ms.data(), kinds.data(), (int)ms.size(), &count);
     if (st != QS_OK) return st;
     p->h->pending = pend;                              // each profile starts from the pending start
     p->h->pending_x = pend_x;
-    st = qs_plan_profile(p, reps, e, seed, 0, ms.data(), kinds.data(), (int)ms.size(), &count);
+    st = profile_runs(p, reps, e, seed, 0, fid, ms.data(), kinds.data(), (int)ms.size(), &count);
     p->h->pending = pend;
     p->h->pending_x = pend_x;
     if (st != QS_OK) return st;
@@ -2765,15 +2774,15 @@ qs_status tune_configs(qs_plan p, int reps, double e, uint64_t seed, int* bl, in
 }
 
 // Time of a run of width m from the state in memory under a configuration.
-qs_status time_from_memory(qs_plan p, int m, int low, int high, int reps, double e, uint64_t seed, double* total) {
+qs_status time_from_memory(qs_plan p, int m, int low, int high, int reps, double e, uint64_t seed, int fid, double* total) {
   qs_status st = qs_plan_set_window(p, m);
   if (st == QS_OK) st = qs_plan_set_config(p, low, high);
   std::vector<double> ms((size_t)std::max(p->launches, 1));
   std::vector<int> kinds(ms.size());
   int count = 0;
   p->h->pending = 0;
-  if (st == QS_OK) st = qs_plan_profile(p, 1, e, seed, 0, ms.data(), kinds.data(), (int)ms.size(), &count);   // untimed
-  if (st == QS_OK) st = qs_plan_profile(p, reps, e, seed, 0, ms.data(), kinds.data(), (int)ms.size(), &count);
+  if (st == QS_OK) st = profile_runs(p, 1, e, seed, 0, fid, ms.data(), kinds.data(), (int)ms.size(), &count);   // untimed
+  if (st == QS_OK) st = profile_runs(p, reps, e, seed, 0, fid, ms.data(), kinds.data(), (int)ms.size(), &count);
   *total = 0.0;
   for (int i = 0; i < count && i < (int)ms.size(); ++i) *total += ms[i];
   return st;
@@ -2796,6 +2805,10 @@ qs_status qs_plan_autotune(qs_plan p, int reps, double e, uint64_t seed, double*
   if (h->mode == QS_STATEVEC && h->dtype == QS_C64 && h->n <= 32)
     for (int m = kWin; m <= kMaxWin; ++m)
       if (m != p->m && h->n >= m) widths.push_back(m);
+  // a handle that holds a reference is one whose runs reduce the fidelity: the outer
+  // product then reads the reference once for four members, which at 24 qubits takes
+  // 0.6 ms with windows of 10 or 11 and 0.3 with 12
+  const int fid = h->mode == QS_STATEVEC && h->has_ref && fusable_end(p);
   struct Tuned { int m, low, high; double lo, hi, total; };
   std::vector<Tuned> tuned;
   size_t best = 0;
@@ -2803,7 +2816,7 @@ qs_status qs_plan_autotune(qs_plan p, int reps, double e, uint64_t seed, double*
     qs_status st = qs_plan_set_window(p, m);
     if (st != QS_OK) return st;
     Tuned t{m, 0, 0, 0.0, 0.0, 0.0};
-    st = tune_configs(p, reps, e, seed, &t.low, &t.high, &t.lo, &t.hi, &t.total);
+    st = tune_configs(p, reps, e, seed, fid, &t.low, &t.high, &t.lo, &t.hi, &t.total);
     if (st != QS_OK) return st;
     tuned.push_back(t);
     if (t.total < tuned[best].total) best = tuned.size() - 1;
@@ -2822,7 +2835,7 @@ qs_status qs_plan_autotune(qs_plan p, int reps, double e, uint64_t seed, double*
     for (size_t i : close) {
       if (close.size() < 2) break;
       double total = 0.0;
-      qs_status st = time_from_memory(p, tuned[i].m, tuned[i].low, tuned[i].high, reps, e, seed, &total);
+      qs_status st = time_from_memory(p, tuned[i].m, tuned[i].low, tuned[i].high, reps, e, seed, fid, &total);
       if (st != QS_OK) return st;
       if (least < 0.0 || total < least) { least = total; best = i; }
     }

@@ -117,3 +117,21 @@ for start, want in ((True, {pending}), (False, {loaded})):
     qs.qs_plan_destroy(p)
 qs.qs_destroy(h)
 """)
+
+
+def test_autotuner_times_the_fidelity_of_a_stored_reference(fake):
+    run(fake, """
+import numpy as np
+L.fake_cost(b"k_outerIfLi4ELb0E", 1.0)                # k_outer without and with the fidelity
+L.fake_cost(b"k_outerIfLi4ELb1E", 5.0)
+for stored, want in ((False, 1.0), (True, 5.0)):
+    h = qs.qs_create(20, 2, 0, qs.QS_STATEVEC, qs.QS_C64)
+    if stored:
+        qs.qs_set_reference(h, np.eye(1, 1 << 20, dtype=complex)[0])
+    p = qs.qs_plan_create(h, circuit("qft", 20, 0))
+    qs.qs_set_basis_state(h, 5)
+    low, high = qs.qs_plan_autotune(p, 2, 0.01, 1, h)
+    assert (low, high) == (want, 0.0), (low, high)
+    qs.qs_plan_destroy(p)
+    qs.qs_destroy(h)
+""")
