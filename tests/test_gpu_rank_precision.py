@@ -1,5 +1,5 @@
-"""Rounding of fixed-rank channels that truncate nothing: what a channel's trace is
-off by, over random factors.
+"""Rounding of fixed-rank channels: what the trace of one that truncates nothing is
+off by, over random factors, and that of a search whose cut amplifies it.
 
 The rounding of the projection's matrices V and of the Kraus operators E is the same
 for every row of L, so it does not average out.  A rounding of a random number is
@@ -11,8 +11,11 @@ the eigenvectors, or their norms off by one, is 2.4 u.)"""
 import numpy as np
 import pytest
 
+from oracle import circuits as ocirc
+from oracle import fixed_rank as ofr
 from oracle import gates as ogates
-from paper_1412_2293_gb300 import qs
+from paper_1412_2293_gb300 import circuits as pcirc
+from paper_1412_2293_gb300 import inputs, qs
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +61,23 @@ def test_trace_of_channels_without_truncation():
                     want += (S[j, k] * np.sum(a.conj() * b)).real
         off.append(float(np.sum(np.abs(got.astype(np.clongdouble)) ** 2) - want))
     assert np.sqrt(np.mean(np.square(off))) < 2 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("n,e,marked", [(8, 0.0191, 141), (8, 0.0159, 52), (9, 0.0161, 240)])
+def test_trace_of_a_truncated_search(n, e, marked):
+    """Grover's search at rank 4, where the cut falls between eigenvalues hundreds of
+    times closer to each other than to the largest: an error of the eigenvectors is
+    divided by that gap.  The trace is allowed what 2 u a channel, all in one
+    direction, come to on either side."""
+    from paper_1412_2293_gb300 import build
+    build.build()
+    ops, r = inputs.grover_circuit(n, 9, marked), 4
+    h = qs.qs_create(n, 1, r, qs.QS_FIXED_RANK, qs.QS_C128)
+    try:
+        qs.qs_set_basis_state(h, 0)
+        pcirc.apply_ops(h, ops, e, 0)
+        got = qs.qs_trace(h)[0]
+    finally:
+        qs.qs_destroy(h)
+    want = ofr.trace(ocirc.run_fixed_rank(n, ops, 0, e, r))
+    assert abs(got - want) <= 2 * 2 * 2.0 ** -53 * sum(o.noisy for o in ops)
